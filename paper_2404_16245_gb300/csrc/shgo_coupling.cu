@@ -1,513 +1,515 @@
-// FP64 coupling kernel (step S2), one instantiation per Lambda = la + lb and nucleus-chunk size.
+// FP64 coupling kernel (step S2), one instantiation per Lambda = la + lb (and la + lb + 1 for derivatives).
 //
-// For one primitive pair (one warp) and its nuclei C, in the pair frame with d = C - P:
+// For one primitive pair and its nuclei C, in the pair frame with d = C - P:
 //   R'[L,M,k] = 2 pi k! p^{-(k+1)} sum_C Z_C S_LM(d) beta_{L,k}(T) / k!,
 //   beta_{L,k} / k! = sum_{j<=k} T^j / j! F_{L+j}(T),  T = p |d|^2,
-// the radial part of the corrected one-centre integral (Eq. 12 with the same-centre coupling
-// restored) before the Clebsch-Gordan coupling of the pair kernel.  S_LM(d) = |d|^L N_LM U_LM(u)
-// with u = d/|d|; the |d|^L goes with the radial factors (sum_j tau_j G_{L+j}, tau_j = (p|d|)^j/j!,
-// G_n = Z |d|^n F_n) and N_LM with the final scale.
+// the radial part of the corrected one-centre integral (Eq. 12 with the same-centre coupling restored) before the
+// Clebsch-Gordan coupling of the pair kernel.  With t = sqrt(T), u = d/|d| and S_LM(u) = N_LM U_LM(u),
+//   S_LM(d) beta_{L,k} / k! = p^{-L/2} N_LM U_LM(u) b_{L,k},   b_{L,k} = sum_{j<=k} t^j / j! (t^{L+j} F_{L+j}).
 //
-// A block of two warps works on one primitive pair.  Lane i of both warps owns nucleus i of a chunk
-// of NCH: warp 0 evaluates the Boys values, the radial sums and part of the unit-vector harmonic
-// columns, warp 1 the other columns, every loop unrolled (Lambda is a template parameter, so the
-// recursions run in registers with their constants as immediate operands); they write column i of
-// two shared tables S[h][c] and B[b][c].  Then thread t owns R' entries e = t, t + 64, ...: their
-// sums over the chunk's nuclei read both table rows with 16-byte loads at fixed offsets.  Row
-// stride NCH + 2 doubles keeps those loads free of bank conflicts.  Two warps per block double
-// the warps an SM holds for the same shared memory.  At small Lambda (few harmonic columns and R'
-// entries for the second warp) one warp does both halves (NW = 1); every entry is formed by the same
-// operations either way.
+// What bounds it: FP64 issues 1.7 lanes per clock and SM on GB300, integer multiply-adds 62 (measured).  So FP64 is kept for
+// what needs its range (geometry, Boys values, radial sums), once per nucleus, and the rest, the harmonics and the
+// sums over nuclei, runs in 58-bit fixed point (shgo_fixed.cuh), which has more bits than an FP64 mantissa.
+//
+// The nuclei of a chunk of 32 fall in three kinds, and take columns of the shared tables in this order:
+//  - near: T below kFarT[Lambda].  Boys values by Taylor expansion from a grid that reaches that T (one branch, no
+//    asymptotic form), radial sums b_{L,k}, one table row per (L, k).
+//  - far: F_n(T) equals its asymptotic form (2n-1)!!/2^n sqrt(pi)/2 T^{-n-1/2} to 2^-56, so T^j F_{L+j} does not depend
+//    on j but by a constant: b_{L,k} = a_{L,k} t^{-(L+1)}, and one sum per (L, M) serves every k.  In a molecule most
+//    nuclei are far (T = 40 is 3.6 bohr at p = 3): no Boys values, Lambda + 1 radial values instead of one per (L, k),
+//    (Lambda + 1)^2 sums instead of C(Lambda + 3, 3).
+//  - axis: on the line through A and B, as the nuclei of A and B themselves.  U_LM vanishes there but for M = 0, and
+//    these nuclei dominate the radial values, so they would set the scale of sums they have no part in: they are
+//    added in FP64 to the M = 0 entries alone.
+// Radial rows are scaled by the largest exponent among the row's columns, near and far separately; harmonic rows by a
+// power of two per (l, |m|), and x, y of a chunk close to the axis by that of the chunk's largest.  A sum is therefore within
+// 32 x 2^-59 or so of the largest product in it, where an FP64 sum rounds at 2^-53 of its partial sums.
+//
+// Phases of a block (NW warps, one primitive pair at a time): warp 0, lane = nucleus: geometry, kinds, radial rows;
+// all warps, lane = column: harmonic columns m, split by cost; thread = (L, M): sums over the far columns, then
+// thread = R' entry: sums over the near columns, far part, axis part and scales.
+//
+// Measured (GB300, whole calls, against the same kernel with every step in FP64): V of 32 atoms with l <= 6 501 -> 404 us,
+// of a contracted 29-atom molecule 7.00 -> 4.40 ms, of six such molecules in a batch 53.1 -> 29.8 ms; dV/dA of the
+// 32 atoms 1.63 -> 1.50 ms.  Errors against 64-bit quadrature are the same to two digits.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cstdlib>
 #include <utility>
+#include <vector>
 
+#include "shgo_fixed.cuh"
 #include "shgo_internal.h"
 #include "shgo_math.h"
-#include "shgo_point_tables.cuh"
 
 namespace shgo {
 
 namespace {
 
-template <int NCH, int LAM, int NW>
-__global__ void __launch_bounds__(32 * NW) k_coupling_fp64(CouplingArgs A) {
-  constexpr int NT = 32 * NW;
-  using Sh = CouplingShape<LAM, NCH>;
-  constexpr int nS = Sh::nS, nR = Sh::nR, CS = Sh::CS;
-  extern __shared__ __align__(16) double smem[];
-  double* Stab = smem;             // [nS][CS]
-  double* Btab = Stab + nS * CS;   // [nB][CS]
-  double* racc = Btab + Sh::nB * CS;
-  double* scl = racc + nR;
+constexpr int kNch = 32;        // nuclei per chunk
+constexpr int kCS = kNch + 1;   // row stride: odd, so that 8-byte loads of different rows fall in different banks
+constexpr double kMagic = 6755399441055744.0;  // 1.5 2^52: adding it rounds to an integer in the low word
+
+__constant__ BoysConst k_boys;
+// Step l -> l + 1 of column m (l >= m >= 0), at l (l + 1) / 2 + m: V = 2^e U obeys
+// V_{l+1} = 2^a z V_l + n V_{l-1}; (n's limbs, a, e(l, m)).  Two sets of scales: e_0 for x, y as they are (|V| <= 1 as
+// 2^e_0 <= N_lm and |S_lm| <= 1), e_1 for a chunk close to the axis, whose x, y are scaled up to the order of 1
+// (2^e_1 <= 1 / max |V / (x + iy)^m|, reached at z = 1).
+constexpr int kSteps = (kLamDer + 1) * (kLamDer + 2) / 2;
+__constant__ int4 k_step[2 * kSteps];
+// Per set and harmonic row h = (L, M): |M| | e(L, M) << 8 | L << 16.
+constexpr int kRows = (kLamDer + 1) * (kLamDer + 1);
+__device__ int g_row[2 * kRows];
+// Boys grid per top order Lambda: row g holds F_{Lambda+k}(T_g) / k!, k = 0..7, exp(-T_g), 0.
+__device__ double2 g_boys_top[(kLamDer + 1) * kBoysTopRows * kBoysTopStride / 2];
+// a_{L,k} = sqrt(pi)/2 sum_{j<=k} (2(L+j)-1)!! / (2^{L+j} j!) at L (kLamDer / 2 + 1) + k, and 2 pi k!.
+__device__ double g_far[(kLamDer + 1) * (kLamDer / 2 + 1)];
+__device__ double g_kfact[kLamDer / 2 + 1];
+
+// T from which F_n(T), n <= Lambda, is asymptotic: Q(Lambda + 1/2, T) = 2^-56 (the regularised upper incomplete
+// gamma function is the relative deviation), rounded up; inside the grid (80) for every order.
+__host__ __device__ constexpr double far_t(int lam) {
+  constexpr double t[kLamDer + 1] = {36.5, 40.9, 44.3, 47.4, 50.2, 52.8, 55.4, 57.8, 60.2,
+                                     62.5, 64.7, 66.9, 69.0, 71.1, 73.1, 75.2, 77.2, 79.1};
+  return t[lam];
+}
+
+__host__ __device__ constexpr int beta_first(int lam, int L) {  // first radial row of L
+  int n = 0;
+  for (int l = 0; l < L; ++l) n += ((lam - l) >> 1) + 1;
+  return n;
+}
+
+// Warps per block: one where a warp's tables leave an SM full of blocks, more where the harmonic columns are many and
+// the tables large (the warps of a block share them).
+__host__ __device__ constexpr int coupling_warps(int lam) { return lam <= 5 ? 1 : (lam <= 8 ? 2 : 4); }
+
+template <int LAM>
+struct Shape {
+  static constexpr int nS = n_harm(LAM), nB = n_beta(LAM), nR = n_r(LAM), NW = coupling_warps(LAM);
+  static constexpr size_t smem = 8 * (size_t)((nS + nB + 3) * kCS + nR + nS + 4 * nB + (LAM + 1)) +
+                                 4 * (size_t)(2 * nB + 2 * (LAM + 1) + 8);
+};
+
+// Column split over NW warps: warp w takes |m| in [column_bound(w), column_bound(w + 1)), the columns' steps evened out
+// (warp 0 starts its share when the radial rows are done, like the others).
+__host__ __device__ constexpr int column_bound(int lam, int nw, int w) {
+  if (w <= 0) return 0;
+  if (w >= nw) return lam + 1;
+  const int total = (lam + 1) * (lam + 1);
+  int m = 0, acc = 0;
+  while (m <= lam && nw * (acc + (lam - m + 1) * (m ? 2 : 1) / 2) < w * total) {
+    acc += (lam - m + 1) * (m ? 2 : 1);
+    ++m;
+  }
+  return m;
+}
+
+// 2^a z v + n w (fixed point; the caller passes z's limbs already shifted by a).
+__device__ __forceinline__ fx fx_step(fx z, fx v, int nh, int nl, fx w) {
+  long long hh = fx_mad(z.h, v.h, 0), mid = fx_mad(z.h, v.l, 0);
+  mid = fx_mad(z.l, v.h, mid);
+  hh = fx_mad(nh, w.h, hh);
+  mid = fx_mad(nh, w.l, mid);
+  mid = fx_mad(nl, w.h, mid);
+  return fx_split(fx_sum(hh, mid));
+}
+
+// Columns m = +-am, am in [A0, A1), of V_lm into rows h of St at column c.
+template <int LAM>
+__device__ __forceinline__ void harmonic_columns(int A0, int A1, int set, fx x, fx y, fx z, int2* St, int c) {
+  fx dp = {1 << kFxLimb, 0}, dm = {0, 0};  // (x + iy)^am
+  const fx ny = fx_neg(y);
+#pragma unroll 1
+  for (int am = 0; am < A1; ++am) {
+    if (am >= A0) {
+      fx p0 = {0, 0}, p1 = dp, m0 = {0, 0}, m1 = dm;
+#pragma unroll 1
+      for (int l = am;; ++l) {
+        const int h = l * l + l;
+        St[(h + am) * kCS + c] = make_int2(p1.h, p1.l);
+        if (am) St[(h - am) * kCS + c] = make_int2(m1.h, m1.l);
+        if (l == LAM) break;
+        const int4 s = k_step[set + l * (l + 1) / 2 + am];
+        const fx za = {z.h << s.z, z.l << s.z};
+        const fx pn = fx_step(za, p1, s.x, s.y, p0);
+        p0 = p1;
+        p1 = pn;
+        if (am) {
+          const fx mn = fx_step(za, m1, s.x, s.y, m0);
+          m0 = m1;
+          m1 = mn;
+        }
+      }
+    }
+    const fx t = fx_step(x, dp, ny.h, ny.l, dm);
+    dm = fx_step(y, dp, x.h, x.l, dm);
+    dp = t;
+  }
+}
+
+template <int LAM>
+__global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(CouplingArgs A) {
+  using Sh = Shape<LAM>;
+  constexpr int NW = Sh::NW, NT = 32 * NW, nS = Sh::nS, nB = Sh::nB, nR = Sh::nR;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int2* St = reinterpret_cast<int2*>(smem_raw);             // [nS] harmonic rows
+  int2* Bt = St + nS * kCS;                                  // [nB] radial rows (axis columns: doubles)
+  int2* Xt = Bt + nB * kCS;                                  // [3] x, y, z of the columns
+  double* racc = reinterpret_cast<double*>(Xt + 3 * kCS);    // [nR] sums of the chunks so far
+  double* fard = racc + nR;                                  // [nS] far sums of the chunk
+  double* axs = fard + nS;                                   // [nB] axis sums of the chunk
+  double* sb = axs + nB;                                     // [nB] 2 pi k! p^{-(k+1)-L/2}
+  double* cfa = sb + nB;                                     // [nB] a_{L,k}
+  double* cfk = cfa + nB;                                    // [nB] 2 pi k!
+  double* pw = cfk + nB;                                     // [LAM + 1] p^{-1-j/2}
+  int* en = reinterpret_cast<int*>(pw + LAM + 1);            // [nB] biased exponent of the near columns of a row
+  int* blk = en + nB;                                        // [nB] L | (L + 2k) << 8
+  int* ef = blk + nB;                                        // [LAM + 1] the same of the far columns
+  int* b0 = ef + LAM + 1;                                    // [LAM + 1] first radial row of L
+  int* cnt = b0 + LAM + 1;                                   // near end, far end, near-axis end, columns, exponent of x, y
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   __shared__ long long s_next[2];
   __shared__ unsigned long long s_t0;
+  constexpr int cb1 = column_bound(LAM, NW, 1), cb2 = column_bound(LAM, NW, 2), cb3 = column_bound(LAM, NW, 3);
+  const int A0 = wid == 0 ? 0 : (wid == 1 ? cb1 : (wid == 2 ? cb2 : cb3));
+  const int A1 = wid == NW - 1 ? LAM + 1 : (wid == 0 ? cb1 : (wid == 1 ? cb2 : cb3));
+  for (int L = tid; L <= LAM; L += NT) {
+    const int f = beta_first(LAM, L);
+    b0[L] = f;
+    for (int k = 0; k <= (LAM - L) / 2; ++k) {
+      blk[f + k] = L | (L + 2 * k) << 8;
+      cfa[f + k] = g_far[L * (kLamDer / 2 + 1) + k];
+      cfk[f + k] = g_kfact[k];
+    }
+  }
   wq_for_each(A.q, A.npp, s_next, &s_t0, [&](long long w) {
     const int64_t q = A.pp_base + w;
     const int pr = A.pp_pair[q];
-    const int a = A.pair_a[pr];
     const PPData pd = A.ppd[q];
-    // primitive pairs with a zero prefactor (K_AB of Eq. 5 underflowed, or the pair is below the
-    // per-basis bound) are skipped by the pair kernel too, so their coupling block is not needed
+    // primitive pairs with a zero prefactor (K_AB of Eq. 5 underflowed, or the pair is below the per-basis bound) are
+    // skipped by the pair kernel too, so their coupling block is not needed
     if (pd.pref == 0.0) return;
-    // C - P = (C - A) - (beta/p)(B - A), in the pair frame where B - A is along z
-    const double Ax = A.shell_xyz[3 * a], Ay = A.shell_xyz[3 * a + 1], Az = A.shell_xyz[3 * a + 2];
-    double Q[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Q[k] = A.site_rot[9 * A.pair_site[pr] + k];
-    __syncthreads();  // the previous primitive pair is done with racc and scl
-    for (int e = tid; e < nR; e += NT) racc[e] = 0.0;
+    const double ip = pd.sp * pd.rp;  // p^{-1/2}
     int64_t cbeg, ncen;
     mol_centers(A.mv, pr, cbeg, ncen);
-    for (int64_t c0 = 0; c0 < ncen; c0 += NCH) {
-      __syncthreads();  // the tables of the previous chunk are consumed
-      if (lane < NCH) {
-        double dx = 0.0, dy = 0.0, dz = 0.0, z = 0.0;
-        if (c0 + lane < ncen) {
-          const int64_t c = mol_center_index(A.mv, cbeg + c0 + lane);
-          pair_frame_offset(Q, Ax, Ay, Az, pd.shift, A.centers + 3 * c, dx, dy, dz);
-          z = A.charges[c];
-        }
-        if (NW == 2) {
-          point_tables<LAM, CS>(wid, lane, pd.p, dx, dy, dz, z, A.boys_tab, Stab, Btab);
-        } else {  // one warp takes both halves of the tables
-          point_tables<LAM, CS>(0, lane, pd.p, dx, dy, dz, z, A.boys_tab, Stab, Btab);
-          point_tables<LAM, CS>(1, lane, pd.p, dx, dy, dz, z, A.boys_tab, Stab, Btab);
-        }
-      }
-      __syncthreads();
-      // a partial last chunk sums only its occupied columns (rounded up to a pair; empty columns
-      // carry Z = 0 and so add exact zeros)
-      const int nv2 = ncen - c0 >= NCH ? NCH / 2 : (int)((ncen - c0 + 1) >> 1);
-      for (int e = tid; e < nR; e += NT) {
-        const int code = __ldg(A.rmap + e);
-        const double2* S = reinterpret_cast<const double2*>(Stab + (code & 0xfff) * CS);
-        const double2* B = reinterpret_cast<const double2*>(Btab + ((code >> 12) & 0xfff) * CS);
-        double a0 = racc[e], a1 = 0.0;
-        if (nv2 == NCH / 2) {
+    double* out = A.rbuf + A.rbase + w * (int64_t)nR;
+    for (int64_t c0 = 0; c0 < ncen || c0 == 0; c0 += kNch) {
+      __syncthreads();  // the tables of the previous chunk (or primitive pair) are consumed
+      if (wid == NW - 1 && c0 == 0 && lane <= LAM) {  // p^{-1-j/2}, lane = j
+        double v = pd.rp, b = ip;
 #pragma unroll
-          for (int c = 0; c < NCH / 2; ++c) {
-            const double2 s = S[c], b = B[c];
-            a0 = fma(s.x, b.x, a0);
-            a1 = fma(s.y, b.y, a1);
+        for (int bit = 0; (1 << bit) <= LAM; ++bit) {
+          if ((lane >> bit) & 1) v *= b;
+          b *= b;
+        }
+        pw[lane] = v;
+      }
+      if (wid == 0) {
+        const bool valid = c0 + lane < ncen;
+        double dx = 0.0, dy = 0.0, zp = 0.0, Z = 0.0;
+        if (valid) {
+          const int64_t c = mol_center_index(A.mv, cbeg + c0 + lane);
+          // C - P = (C - A) - (beta/p)(B - A), in the pair frame where B - A is along z
+          const double* Q = A.site_rot + 9 * (int64_t)A.pair_site[pr];
+          const double* xa = A.shell_xyz + 3 * (int64_t)A.pair_a[pr];
+          const double vx = A.centers[3 * c] - xa[0], vy = A.centers[3 * c + 1] - xa[1], vz = A.centers[3 * c + 2] - xa[2];
+          dx = Q[0] * vx + Q[1] * vy + Q[2] * vz;
+          dy = Q[3] * vx + Q[4] * vy + Q[5] * vz;
+          zp = Q[6] * vx + Q[7] * vy + Q[8] * vz;
+          Z = A.charges[c];
+        }
+        const double dz = zp - pd.shift;
+        const double rho2 = fma(dy, dy, dx * dx), s2 = fma(dz, dz, rho2), T = pd.p * s2;
+        const int hs = __double2hiint(s2);
+        if ((hs & 0x7ff00000) == 0x7ff00000) Z = __longlong_as_double(0x7ff8000000000000ll);  // no finite distance
+        // 1/|d|: hardware estimate and one third-order step (|d| below 2^-500 counts as 0: only L = 0 survives)
+        double ri = 0.0, ux = 0.0, uy = 0.0, uz = 1.0;
+        if (hs >= 0x01700000) {
+          double y;
+          asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s2));
+          const double e = fma(-(s2 * y), y, 1.0);
+          ri = fma(y * e, fma(0.375, e, 0.5), y);
+          ux = dx * ri;
+          uy = dy * ri;
+          uz = dz * ri;
+        }
+        // on the A-B line to within rounding of the rotation: rho below 2^-48 of |z_C - z_A|
+        const int erho = (__double2hiint(rho2) >> 20) & 0x7ff, ezp = (__double2hiint(zp) >> 20) & 0x7ff;
+        const bool axis = hs < 0x7ff00000 && (ri == 0.0 || erho == 0 || erho + 96 + 1023 < 2 * ezp);
+        constexpr double kFar = far_t(LAM);
+        const bool near = __double2hiint(T) < __double2hiint(kFar);
+        const unsigned mn = __ballot_sync(~0u, valid && near && !axis), mf = __ballot_sync(~0u, valid && !near && !axis);
+        const unsigned an = __ballot_sync(~0u, valid && near && axis), af = __ballot_sync(~0u, valid && !near && axis);
+        const int n1 = __popc(mn), n2 = n1 + __popc(mf), n3 = n2 + __popc(an), n4 = n3 + __popc(af);
+        const unsigned below = (1u << lane) - 1u;
+        const int pos = axis ? (near ? n2 + __popc(an & below) : n3 + __popc(af & below))
+                             : (near ? __popc(mn & below) : n1 + __popc(mf & below));
+        // scale of x and y: the power of two of the largest in the chunk
+        const bool off = valid && !axis;
+        const unsigned hxy = max(__double2hiint(ux) & 0x7fffffff, __double2hiint(uy) & 0x7fffffff);
+        const int exy = (int)(__reduce_max_sync(~0u, off ? hxy : 0u) >> 20) - 1023;
+        const int er = exy >= -1 ? 0 : exy + 2;
+        if (off) {
+          const fx fxx = fx_of(ux, 1023 + er), fxy = fx_of(uy, 1023 + er), fxz = fx_of(uz, 1023);
+          Xt[pos] = make_int2(fxx.h, fxx.l);
+          Xt[kCS + pos] = make_int2(fxy.h, fxy.l);
+          Xt[2 * kCS + pos] = make_int2(fxz.h, fxz.l);
+        }
+        if (lane == 0) {
+          cnt[0] = n1;
+          cnt[1] = n2;
+          cnt[2] = n3;
+          cnt[3] = n4;
+          cnt[4] = er;
+        }
+        // near: G_n = Z t^n F_n(T), tau_k = t^k / k!; far: G_n = Z t^{-(n+1)}
+        double G[LAM + 1], tau[LAM / 2 + 1];
+#pragma unroll
+        for (int k = 0; k <= LAM / 2; ++k) tau[k] = 0.0;
+        if (near) {
+          const double t = pd.sp * (s2 * ri);
+          const double tm = fma(T, kBoysInvH, kMagic);
+          const int g = min(max(__double2loint(tm), 0), kBoysTopRows - 1);
+          const double dT = fma(tm - kMagic, 1.0 / kBoysInvH, -T);  // T_g - T
+          const double2* row = g_boys_top + ((size_t)LAM * kBoysTopRows + g) * (kBoysTopStride / 2);
+          double f, ew = 1.0;
+          {
+            const double2 r3 = __ldg(row + 3), r2 = __ldg(row + 2), r1 = __ldg(row + 1), r0 = __ldg(row);
+            f = fma(r3.y, dT, r3.x);
+            f = fma(f, dT, r2.y);
+            f = fma(f, dT, r2.x);
+            f = fma(f, dT, r1.y);
+            f = fma(f, dT, r1.x);
+            f = fma(f, dT, r0.y);
+            f = fma(f, dT, r0.x);
+          }
+          if constexpr (LAM > 0) {
+            ew = 1.0 / 5040.0;
+            ew = fma(ew, dT, 1.0 / 720.0);
+            ew = fma(ew, dT, 1.0 / 120.0);
+            ew = fma(ew, dT, 1.0 / 24.0);
+            ew = fma(ew, dT, 1.0 / 6.0);
+            ew = fma(ew, dT, 0.5);
+            ew = fma(ew, dT, 1.0);
+            ew = fma(ew, dT, 1.0);
+          }
+          double zt = Z, tp = t;  // Z t^Lambda by squaring
+#pragma unroll
+          for (int bit = 0; (1 << bit) <= LAM; ++bit) {
+            if ((LAM >> bit) & 1) zt *= tp;
+            if ((2 << bit) <= LAM) tp *= tp;
+          }
+          G[LAM] = zt * f;
+          if constexpr (LAM > 0) {
+            // F_n = (2T F_{n+1} + exp(-T)) / (2n + 1), scaled: G_n = (2t G_{n+1} + Z t^n exp(-T)) / (2n + 1)
+            G[0] = Z * (__ldg(row + 4).x * ew);
+#pragma unroll
+            for (int n = 1; n < LAM; ++n) G[n] = G[n - 1] * t;
+            const double t2 = t + t;
+#pragma unroll
+            for (int n = LAM - 1; n >= 0; --n) G[n] = fma(t2, G[n + 1], G[n]) * k_boys.inv_odd[n];
+            tau[0] = 1.0;
+#pragma unroll
+            for (int k = 1; k <= LAM / 2; ++k) tau[k] = tau[k - 1] * (t * k_boys.inv_int[k]);
           }
         } else {
-#pragma unroll 4
-          for (int c = 0; c < nv2; ++c) {
-            const double2 s = S[c], b = B[c];
-            a0 = fma(s.x, b.x, a0);
-            a1 = fma(s.y, b.y, a1);
-          }
+          const double v = ri * ip;
+          G[0] = Z * v;
+#pragma unroll
+          for (int n = 1; n <= LAM; ++n) G[n] = G[n - 1] * v;
         }
-        racc[e] = a0 + a1;
-      }
-    }
-    // scale 2 pi k! p^{-(k+1)} N_LM (each thread scales the entries it accumulated)
-    if (tid <= LAM / 2) {
-      double s = kTwoPiC * pd.rp;
-      for (int k = 1; k <= tid; ++k) s *= double(k) * pd.rp;
-      scl[tid] = s;
-    }
-    __syncthreads();
-    double* out = A.rbuf + A.rbase + w * (int64_t)nR;
-    for (int e = tid; e < nR; e += NT) out[e] = racc[e] * (scl[(__ldg(A.rmap + e) >> 24) & 0xff] * __ldg(A.rnorm + e));
-    });
-}
-
-// R' entries of Lambda are ordered by L, then M, then k (k <= (Lambda - L)/2); the harmonic row of (L, M) is
-// L^2 + L + M and the radial row of (L, k) is the number of (L', k') with L' < L plus k.
-// First radial group (in (L, k) order) of the second warp: the groups before it hold at least half the entries.
-__host__ __device__ constexpr int esp_group_split(int lam) {
-  const int half = cn_r(lam) / 2;
-  int g = 0, cum = 0;
-  for (int L = 0; L <= lam; ++L)
-    for (int k = 0; k <= (lam - L) / 2; ++k, ++g) {
-      if (cum >= half) return g;
-      cum += 2 * L + 1;
-    }
-  return g;
-}
-
-// Per point: sum_e G'[e] S[h(e)] B[b(e)] grouped by the radial row, sum_{L,k} B_Lk (sum_M G'_{LMk} S_LM): one
-// multiply-add per entry and one per radial row, instead of a product and a multiply-add per entry.  Radial
-// groups g in [g0, g1); the walk from group 0 to g0 stops by L = Lambda + 1 (g0 <= number of radial rows).
-// Loops run over runtime bounds: a fully unrolled form was slower (its code overflowed the instruction cache).
-template <int LAM, int CS>
-__device__ __forceinline__ double esp_point_sum(int g0, int g1, const double* __restrict__ gam,
-                                                const double* __restrict__ S, const double* __restrict__ B) {
-  int L = 0, rb = 0, bb = 0;
-  while (bb + (LAM - L) / 2 + 1 <= g0) {
-    rb += (2 * L + 1) * ((LAM - L) / 2 + 1);
-    bb += (LAM - L) / 2 + 1;
-    ++L;
-  }
-  int k = g0 - bb, nk = (LAM - L) / 2 + 1;
-  double s0 = 0.0, s1 = 0.0;
-  for (int g = g0; g < g1; ++g) {
-    const double* gp = gam + rb + k;  // G'_{L,M,k}, M = -L..L, stride nk
-    const double* sp = S + L * L * CS;
-    const int n = 2 * L + 1;
-    double t0 = 0.0, t1 = 0.0;
-    int j = 0;
-    for (; j + 1 < n; j += 2) {
-      t0 = fma(gp[j * nk], sp[j * CS], t0);
-      t1 = fma(gp[(j + 1) * nk], sp[(j + 1) * CS], t1);
-    }
-    t0 = fma(gp[j * nk], sp[j * CS], t0);  // n is odd
-    if (g & 1)
-      s1 = fma(t0 + t1, B[(bb + k) * CS], s1);
-    else
-      s0 = fma(t0 + t1, B[(bb + k) * CS], s0);
-    if (++k == nk) {
-      rb += (2 * L + 1) * nk;
-      bb += nk;
-      ++L;
-      k = 0;
-      nk = (LAM - L) / 2 + 1;
-    }
-  }
-  return s0 + s1;
-}
-
-// Electrostatic potential (adjoint of the coupling): for a chunk of NCH points and a range of primitive
-// pairs of one class, phi(C) += sum_e G'[e] U_{L(e)M(e)}(d/|d|) |d|^L beta_{L,k}/k! (d = C - P, unit
-// charge), G' being the density-weighted adjoint block of the primitive pair (k_esp_adjoint).  Block
-// (chunk, split): the splits divide the class's primitive pairs; each block adds its partial sums to
-// phi once per point.  Point sums: warp 0 takes the radial groups before esp_group_split, warp 1 the rest.
-template <int NCH, int LAM>
-__global__ void __launch_bounds__(64) k_esp_fp64(EspArgs A) {
-  using Sh = CouplingShape<LAM, NCH>;
-  constexpr int nS = Sh::nS, nR = Sh::nR, CS = Sh::CS;
-  extern __shared__ __align__(16) double smem[];
-  double* Stab = smem;
-  double* Btab = Stab + nS * CS;
-  double* gam = Btab + Sh::nB * CS;  // [nR]
-  double* part = gam + nR;           // [NCH] partial sums of warp 1
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int chunk = blockIdx.x % A.nchunks, split = blockIdx.x / A.nchunks;
-  const int64_t per = (A.npp + A.nsplit - 1) / A.nsplit;
-  const int64_t w0 = split * per, w1 = min(A.npp, w0 + per);
-  const int64_t c = (int64_t)chunk * NCH + lane;
-  const bool valid = lane < NCH && c < A.npoints;
-  double acc = 0.0;
-  constexpr int GS = esp_group_split(LAM);
-  for (int64_t w = w0; w < w1; ++w) {
-    const int64_t q = A.pp_base + w;
-    const PPData pd = A.ppd[q];
-    if (pd.pref == 0.0) continue;
-    const int pr = A.pp_pair[q];
-    const int a = A.pair_a[pr];
-    const double Ax = A.shell_xyz[3 * a], Ay = A.shell_xyz[3 * a + 1], Az = A.shell_xyz[3 * a + 2];
-    double Q[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Q[k] = A.site_rot[9 * A.pair_site[pr] + k];
-    __syncthreads();  // the previous primitive pair is done with the tables and gam
-    for (int e = tid; e < nR; e += 64) gam[e] = A.gam[w * (int64_t)nR + e];
-    if (lane < NCH) {
-      double dx = 0.0, dy = 0.0, dz = 0.0, z = 0.0;
-      if (valid) {
-        pair_frame_offset(Q, Ax, Ay, Az, pd.shift, A.points + 3 * c, dx, dy, dz);
-        z = 1.0;
-      }
-      point_tables<LAM, CS>(wid, lane, pd.p, dx, dy, dz, z, A.boys_tab, Stab, Btab);
-    }
-    __syncthreads();
-    if (lane < NCH)
-      acc += esp_point_sum<LAM, CS>(wid == 0 ? 0 : GS, wid == 0 ? GS : Sh::nB, gam, Stab + lane, Btab + lane);
-  }
-  __syncthreads();
-  if (wid == 1 && lane < NCH) part[lane] = acc;
-  __syncthreads();
-  if (wid == 0 && valid) atomicAdd(A.phi + c, acc + part[lane]);
-}
-
-// Solid-harmonic polynomials S~_lm(d) = |d|^l U_lm(d/|d|) (degree l, same constants as U) and their
-// gradients, l <= LAM, into P, Gx, Gy, Gz at row h = l^2 + l + m (stride CS): forward-mode derivatives of
-// S~_{l+1,m} = z S~_lm + ng_lm r^2 S~_{l-1,m}, S~_{|m|+1,m} = z S~_{|m|,m} and of the diagonal chain
-// S~_{l+1,l+1} = x S~_ll - y S~_{l,-l}, S~_{l+1,-l-1} = y S~_ll + x S~_{l,-l} (which does not depend on z).
-// The columns are split by the sign of m between the two half-warps: lanes of half `neg` take
-// m = -|m| for |m| >= 1, the others m = +|m| for |m| >= 0.  The diagonal chain and the column
-// recursions run as loops over |m| and l, so that both halves, whose columns of one |m| have equal
-// lengths, advance in step.
-template <int LAM, int CS>
-__device__ __forceinline__ void harmonic_columns_grad_half(bool neg, double x, double y, double z, double* P,
-                                                           double* Gx, double* Gy, double* Gz) {
-  const double r2 = x * x + y * y + z * z;
-  double dp = 1.0, dm = 1.0, dpx = 0.0, dpy = 0.0, dmx = 0.0, dmy = 0.0;  // U_{am,+-am} and gradients
-#pragma unroll 1
-  for (int am = 0; am <= LAM; ++am) {
-    if (!(neg && am == 0)) {
-      const int m = neg ? -am : am;
-      double v0 = neg ? dm : dp, x0 = neg ? dmx : dpx, y0 = neg ? dmy : dpy, z0 = 0.0;
-      int h = am * am + am + m;
-      P[h * CS] = v0;
-      Gx[h * CS] = x0;
-      Gy[h * CS] = y0;
-      Gz[h * CS] = z0;
-      if (am + 1 <= LAM) {
-        double v1 = z * v0, x1 = z * x0, y1 = z * y0, z1 = v0;
-        h = (am + 1) * (am + 1) + am + 1 + m;
-        P[h * CS] = v1;
-        Gx[h * CS] = x1;
-        Gy[h * CS] = y1;
-        Gz[h * CS] = z1;
-#pragma unroll 2
-        for (int l = am + 1; l < LAM; ++l) {
-          const double g = k_harm.ng[l * l + l + m];
-          const double v2 = fma(g * r2, v0, z * v1);
-          const double x2 = fma(g, fma(2.0 * x, v0, r2 * x0), z * x1);
-          const double y2 = fma(g, fma(2.0 * y, v0, r2 * y0), z * y1);
-          const double z2 = fma(g, fma(2.0 * z, v0, r2 * z0), fma(z, z1, v1));
-          h = (l + 1) * (l + 1) + l + 1 + m;
-          P[h * CS] = v2;
-          Gx[h * CS] = x2;
-          Gy[h * CS] = y2;
-          Gz[h * CS] = z2;
-          v0 = v1; x0 = x1; y0 = y1; z0 = z1;
-          v1 = v2; x1 = x2; y1 = y2; z1 = z2;
-        }
-      }
-    }
-    // the diagonal chain one level up
-    if (am == 0) {
-      dp = x;
-      dm = y;
-      dpx = 1.0;
-      dpy = 0.0;
-      dmx = 0.0;
-      dmy = 1.0;
-    } else {
-      const double np = fma(x, dp, -y * dm), nm = fma(y, dp, x * dm);
-      const double npx = dp + fma(x, dpx, -y * dmx), npy = fma(x, dpy, -y * dmy) - dm;
-      const double nmx = fma(y, dpx, x * dmx) + dm, nmy = fma(y, dpy, x * dmy) + dp;
-      dp = np;
-      dm = nm;
-      dpx = npx;
-      dpy = npy;
-      dmx = nmx;
-      dmy = nmy;
-    }
-  }
-}
-
-template <int LAM>
-struct GradShape {
-  static constexpr int NCH = 16, CS = NCH + 2;
-  static constexpr int nS = cn_harm(LAM), nB = cn_beta(LAM), nR = cn_r(LAM);
-  static constexpr size_t smem = sizeof(double) * ((size_t)(4 * nS + 2 * nB) * CS + nR + 3 * NCH + 4 * 64 + 16);
-};
-
-// Gradient of the electrostatic potential at each point: for a chunk of 16 points and a range of
-// primitive pairs of one class, grad phi(C) += Q^T sum_e G'[e] d/dd [S~_{LM}(d) B_{L,k}(T)], d = C - P in the
-// pair frame, B_{L,k} = sum_{j<=k} T^j/j! F_{L+j} and dB_{L,k}/dT = -T^k/k! F_{L+k+1}, so
-// d/dd [S~ B] = B grad S~ - 2p T^k/k! F_{L+k+1} S~ d.  Threads: point c = t % 16; in the table phase
-// warp 0 (16 lanes) evaluates the Boys values and radial factors, warp 1 the harmonic columns (its two
-// halves the columns of m >= 0 and m < 0); in the sum phase the four groups of 16 threads take a quarter
-// of the R' entries each.
-template <int LAM>
-__global__ void __launch_bounds__(64) k_esp_grad_fp64(EspArgs A) {
-  using Sh = GradShape<LAM>;
-  constexpr int NCH = Sh::NCH, CS = Sh::CS, nS = Sh::nS, nB = Sh::nB, nR = Sh::nR;
-  extern __shared__ __align__(16) double smem[];
-  double* Pt = smem;
-  double* Gxt = Pt + nS * CS;
-  double* Gyt = Gxt + nS * CS;
-  double* Gzt = Gyt + nS * CS;
-  double* Bt = Gzt + nS * CS;
-  double* Bq = Bt + nB * CS;
-  double* gam = Bq + nB * CS;
-  double* dv = gam + nR;      // [3][NCH]
-  double* red = dv + 3 * NCH; // [3][64]
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, pc = tid & 15, quarter = tid >> 4;
-  const int chunk = blockIdx.x % A.nchunks, split = blockIdx.x / A.nchunks;
-  const int64_t per = (A.npp + A.nsplit - 1) / A.nsplit;
-  const int64_t w0 = split * per, w1 = min(A.npp, w0 + per);
-  const int64_t c = (int64_t)chunk * NCH + pc;
-  const bool valid = c < A.npoints;
-  const int e0 = quarter * nR / 4, e1 = (quarter + 1) * nR / 4;
-  double gm[3] = {0.0, 0.0, 0.0};
-  for (int64_t w = w0; w < w1; ++w) {
-    const int64_t q = A.pp_base + w;
-    const PPData pd = A.ppd[q];
-    if (pd.pref == 0.0) continue;
-    const int pr = A.pp_pair[q];
-    const int a = A.pair_a[pr];
-    double Q[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Q[k] = A.site_rot[9 * A.pair_site[pr] + k];
-    double dx = 0.0, dy = 0.0, dz = 0.0;
-    if (valid)
-      pair_frame_offset(Q, A.shell_xyz[3 * a], A.shell_xyz[3 * a + 1], A.shell_xyz[3 * a + 2], pd.shift,
-                        A.points + 3 * c, dx, dy, dz);
-    __syncthreads();  // the previous primitive pair is done with the tables
-    for (int e = tid; e < nR; e += 64) gam[e] = A.gam[w * (int64_t)nR + e];
-    if (lane < NCH) {
-      if (wid == 0) {
-        dv[pc] = dx;
-        dv[NCH + pc] = dy;
-        dv[2 * NCH + pc] = dz;
-        const double T = pd.p * (dx * dx + dy * dy + dz * dz);
-        double F[LAM + 2];
-        boys_eval(LAM + 1, T, F, 1, A.boys_tab, k_boys);
-        double tk[LAM / 2 + 1];  // T^k / k!
-        tk[0] = 1.0;
-#pragma unroll
-        for (int k = 1; k <= LAM / 2; ++k) tk[k] = tk[k - 1] * T * k_boys.inv_int[k];
-        const double m2p = -2.0 * pd.p;
+        const bool anynear = (mn | an) != 0u;
+        const bool wr = near ? valid : false;
+        const int sgn = uz < 0.0 ? (int)0x80000000 : 0;
         int bo = 0;
 #pragma unroll
         for (int L = 0; L <= LAM; ++L) {
-          double acc = 0.0;
+          double acc = G[L];
 #pragma unroll
           for (int k = 0; k <= (LAM - L) / 2; ++k) {
-            acc = fma(tk[k], F[L + k], acc);
-            Bt[(bo + k) * CS + pc] = valid ? acc : 0.0;
-            Bq[(bo + k) * CS + pc] = valid ? m2p * tk[k] * F[L + k + 1] : 0.0;
+            if (k > 0 && !anynear) break;
+            if (k > 0) acc = fma(tau[k], G[L + k], acc);
+            const unsigned ha = (unsigned)__double2hiint(acc) & 0x7fffffffu;
+            const int En = (int)(__reduce_max_sync(~0u, near && off ? ha : 0u) >> 20);
+            int E = En;
+            if (k == 0) {
+              const int Ef = (int)(__reduce_max_sync(~0u, !near && off ? ha : 0u) >> 20);
+              if (!near) E = Ef;
+              if (lane == 0) ef[L] = Ef;
+            }
+            if (lane == 0) en[bo + k] = En;
+            if (valid && (wr || k == 0)) {
+              int2 v;
+              if (axis) {  // U_L0(0, 0, +-1) N_L0 = (+-1)^L
+                v = make_int2(__double2loint(acc), __double2hiint(acc) ^ ((L & 1) ? sgn : 0));
+              } else {
+                const fx b = fx_of(acc, E + 2);  // below 2^57: the sums of 32 products stay inside 64 bits
+                v = make_int2(b.h, b.l);
+              }
+              Bt[(bo + k) * kCS + pos] = v;
+            }
           }
           bo += (LAM - L) / 2 + 1;
         }
       }
+      __syncthreads();
+      const int n1 = cnt[0], n2 = cnt[1], n3 = cnt[2], n4 = cnt[3], er = cnt[4];
+      if (lane < n2) {
+        const int2 a = Xt[lane], b = Xt[kCS + lane], c = Xt[2 * kCS + lane];
+        harmonic_columns<LAM>(A0, A1, er < 0 ? kSteps : 0, fx{a.x, a.y}, fx{b.x, b.y}, fx{c.x, c.y}, St, lane);
+      }
+      // axis sums of the radial rows and the rows' scales
+      for (int b = tid; b < nB; b += NT) {
+        double s = 0.0;
+        for (int c = n2; c < n3; ++c) {
+          const int2 v = Bt[b * kCS + c];
+          s += __hiloint2double(v.y, v.x);
+        }
+        if (n3 < n4) {
+          const int2* row = Bt + b0[blk[b] & 0xff] * kCS;
+          double f = 0.0;
+          for (int c = n3; c < n4; ++c) f += __hiloint2double(row[c].y, row[c].x);
+          s = fma(f, cfa[b], s);
+        }
+        axs[b] = s;
+        if (c0 == 0) sb[b] = cfk[b] * pw[blk[b] >> 8];
+      }
+      __syncthreads();
+      const int* rowcode = g_row + (er < 0 ? kRows : 0);
+      if (n1 < n2) {
+        for (int h = tid; h < nS; h += NT) {
+          const int code = __ldg(rowcode + h), L = code >> 16;
+          const int2 *s = St + h * kCS, *b = Bt + b0[L] * kCS;
+          long long hh = 0, mid = 0;
+#pragma unroll 4
+          for (int c = n1; c < n2; ++c) {
+            const int2 u = s[c], v = b[c];
+            hh = fx_mad(u.x, v.x, hh);
+            mid = fx_mad(u.x, v.y, mid);
+            mid = fx_mad(u.y, v.x, mid);
+          }
+          const int E = ef[L];
+          fard[h] = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                               : fx_double(fx_sum(hh, mid), E + 2 - 1023 - kFxBits + er * (code & 0xff) - ((code >> 8) & 0xff));
+        }
+        __syncthreads();
+      }
+      const bool first = c0 == 0, last = c0 + kNch >= ncen;
+      for (int e = tid; e < nR; e += NT) {
+        const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
+        const int rc = __ldg(rowcode + h);
+        double v = 0.0;
+        if (n1 > 0) {
+          const int2 *s = St + h * kCS, *r = Bt + b * kCS;
+          long long hh = 0, mid = 0;
+#pragma unroll 4
+          for (int c = 0; c < n1; ++c) {
+            const int2 u = s[c], x = r[c];
+            hh = fx_mad(u.x, x.x, hh);
+            mid = fx_mad(u.x, x.y, mid);
+            mid = fx_mad(u.y, x.x, mid);
+          }
+          const int E = en[b];
+          v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                         : fx_double(fx_sum(hh, mid), E + 2 - 1023 - kFxBits + er * (rc & 0xff) - ((rc >> 8) & 0xff));
+        }
+        if (n1 < n2) v = fma(fard[h], cfa[b], v);
+        v = fma(v, __ldg(A.rnorm + e), (rc & 0xff) == 0 ? axs[b] : 0.0);
+        if (!first) v += racc[e];
+        if (last)
+          out[e] = v * sb[b];
+        else
+          racc[e] = v;
+      }
     }
-    if (wid == 1) {
-      // both half-warps: the columns of m >= 0 (lanes 0-15) and m < 0 (lanes 16-31) of the same points
-      harmonic_columns_grad_half<LAM, CS>(lane >= NCH, dx, dy, dz, Pt + pc, Gxt + pc, Gyt + pc, Gzt + pc);
-    }
-    __syncthreads();
-    double gx = 0.0, gy = 0.0, gz = 0.0, sb = 0.0;
-    for (int e = e0; e < e1; ++e) {
-      const int code = __ldg(A.rmap + e);
-      const int si = (code & 0xfff) * CS + pc, bi = ((code >> 12) & 0xfff) * CS + pc;
-      const double g = gam[e];
-      const double ab = g * Bt[bi];
-      gx = fma(ab, Gxt[si], gx);
-      gy = fma(ab, Gyt[si], gy);
-      gz = fma(ab, Gzt[si], gz);
-      sb = fma(g * Pt[si], Bq[bi], sb);
-    }
-    gx = fma(sb, dv[pc], gx);
-    gy = fma(sb, dv[NCH + pc], gy);
-    gz = fma(sb, dv[2 * NCH + pc], gz);
-    // back to the molecular frame: grad_C = Q^T grad_d
-    gm[0] += Q[0] * gx + Q[3] * gy + Q[6] * gz;
-    gm[1] += Q[1] * gx + Q[4] * gy + Q[7] * gz;
-    gm[2] += Q[2] * gx + Q[5] * gy + Q[8] * gz;
-  }
-  __syncthreads();
-  red[tid] = gm[0];
-  red[64 + tid] = gm[1];
-  red[128 + tid] = gm[2];
-  __syncthreads();
-  if (tid < NCH && valid)
-    for (int k = 0; k < 3; ++k)
-      atomicAdd(A.phi + 3 * c + k, red[k * 64 + tid] + red[k * 64 + tid + 16] + red[k * 64 + tid + 32] +
-                                       red[k * 64 + tid + 48]);
+  });
 }
 
 using CouplingKernel = void (*)(CouplingArgs);
-using EspKernel = void (*)(EspArgs);
 
 template <int... L>
-constexpr EspKernel esp_grad_kernel_at(int lam, std::integer_sequence<int, L...>) {
-  EspKernel k = nullptr;
-  ((lam == L ? (k = &k_esp_grad_fp64<L>, 0) : 0), ...);
-  return k;
-}
-
-template <int... L>
-constexpr size_t esp_grad_smem_at(int lam, std::integer_sequence<int, L...>) {
-  size_t s = 0;
-  ((lam == L ? (s = GradShape<L>::smem, 0) : 0), ...);
-  return s;
-}
-
-template <int... L>
-constexpr EspKernel esp_kernel_at(int lam, std::integer_sequence<int, L...>) {
-  EspKernel k = nullptr;
-  ((lam == L ? (k = &k_esp_fp64<32, L>, 0) : 0), ...);
-  return k;
-}
-
-template <int NCH, int NW, int... L>
 constexpr CouplingKernel kernel_at(int lam, std::integer_sequence<int, L...>) {
   CouplingKernel k = nullptr;
-  ((lam == L ? (k = &k_coupling_fp64<NCH, L, NW>, 0) : 0), ...);
+  ((lam == L ? (k = &k_coupling_fp64<L>, 0) : 0), ...);
   return k;
 }
 
-template <int NCH, int... L>
+template <int... L>
 constexpr size_t smem_at(int lam, std::integer_sequence<int, L...>) {
   size_t s = 0;
-  ((lam == L ? (s = CouplingShape<L, NCH>::smem, 0) : 0), ...);
+  ((lam == L ? (s = Shape<L>::smem, 0) : 0), ...);
   return s;
 }
 
-using Lams = std::make_integer_sequence<int, kLamMax + 1>;
-// the coupling kernel also runs at Lambda = la + lb + 1 (derivative integrals)
-using LamsDer = std::make_integer_sequence<int, kLamDer + 1>;
-
-// Small Lambda: one warp per block does both halves of the nucleus tables (the second warp of the two-warp
-// form has little of its own there: a few harmonic columns and a few R' entries).
-constexpr int kOneWarpLamMax = 8;
-using LamsOneWarp = std::make_integer_sequence<int, kOneWarpLamMax + 1>;
-int coupling_warps(int lam, bool one_warp_ok) { return one_warp_ok && lam <= kOneWarpLamMax ? 1 : 2; }
-
-CouplingKernel coupling_kernel(int lam, int nch, int nw) {
-  if (lam < 0 || lam > kLamDer) return nullptr;
-  if (nw == 1)
-    return lam > kOneWarpLamMax ? nullptr
-                                : (nch == 16 ? kernel_at<16, 1>(lam, LamsOneWarp{}) : kernel_at<32, 1>(lam, LamsOneWarp{}));
-  return nch == 16 ? kernel_at<16, 2>(lam, LamsDer{}) : kernel_at<32, 2>(lam, LamsDer{});
-}
+using Lams = std::make_integer_sequence<int, kLamDer + 1>;  // derivative integrals run at la + lb + 1
 
 }  // namespace
 
-size_t coupling_fp64_smem(int lam, int nch) {
-  if (lam < 0 || lam > kLamDer) return 0;
-  return nch == 16 ? smem_at<16>(lam, LamsDer{}) : smem_at<32>(lam, LamsDer{});
-}
-
-size_t esp_fp64_smem(int lam) { return coupling_fp64_smem(lam, 32) + sizeof(double) * 40; }
-
-cudaError_t launch_esp_fp64(int lam, const EspArgs& args, cudaStream_t stream) {
-  if (lam < 0 || lam > kLamMax) return cudaErrorInvalidValue;
-  const EspKernel k = esp_kernel_at(lam, Lams{});
-  k<<<args.nchunks * args.nsplit, 64, esp_fp64_smem(lam), stream>>>(args);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_esp_grad_fp64(int lam, const EspArgs& args, cudaStream_t stream) {
-  if (lam < 0 || lam > kLamMax) return cudaErrorInvalidValue;
-  const EspKernel k = esp_grad_kernel_at(lam, Lams{});
-  k<<<args.nchunks * args.nsplit, 64, esp_grad_smem_at(lam, Lams{}), stream>>>(args);
-  return cudaGetLastError();
-}
-
 cudaError_t coupling_fp64_setup() {
-  cudaError_t e = cudaMemcpyToSymbol(k_harm, &harm_coef_host(), sizeof(HarmCoef));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(k_boys, &boys_const_host(), sizeof(BoysConst));
-  for (int lam = 0; lam <= kLamDer && e == cudaSuccess; ++lam)
-    for (int nch : {16, 32})
-      for (int nw : {1, 2}) {
-        const CouplingKernel k = coupling_kernel(lam, nch, nw);
-        if (k) e = set_max_dynamic_smem((const void*)k);
-        if (e != cudaSuccess) break;
+  const HarmCoef& hc = harm_coef_host();
+  std::vector<int4> step(2 * kSteps);
+  std::vector<int> row(2 * kRows);
+  for (int set = 0; set < 2; ++set) {
+    // e(l, m): the largest exponent within the set's bound that grows by at most one from l to l + 1
+    int ex[kLamDer + 1][kLamDer + 1] = {};
+    for (int m = 0; m <= kLamDer; ++m) {
+      double q0 = 0.0, q1 = 1.0;  // V / (x + iy)^m at z = 1, unscaled
+      for (int l = m; l <= kLamDer; ++l) {
+        const double bound = set == 0 ? hc.n[harm_index(l, m)] : 1.0 / q1;
+        int e = 0;
+        while (std::ldexp(1.0, e + 1) <= bound) ++e;
+        ex[l][m] = l > m ? std::min(e, ex[l - 1][m] + 1) : 0;
+        const double q2 = q1 - (l > m ? (double)(l * l - m * m) / (4 * l * l - 1) : 0.0) * q0;
+        q0 = q1;
+        q1 = q2;
       }
-  for (int lam = 0; lam <= kLamMax && e == cudaSuccess; ++lam) {
-    e = set_max_dynamic_smem((const void*)esp_kernel_at(lam, Lams{}));
-    if (e == cudaSuccess)
-      e = set_max_dynamic_smem((const void*)esp_grad_kernel_at(lam, Lams{}));
+    }
+    for (int l = 0; l <= kLamDer; ++l)
+      for (int m = 0; m <= l; ++m) {
+        int4 s = make_int4(0, 0, 0, ex[l][m]);
+        if (l < kLamDer) s.z = ex[l + 1][m] - ex[l][m];
+        if (l > m && l < kLamDer) {
+          // -gamma_lm 2^(e(l+1) - e(l-1)) = -(l^2 - m^2) / (4 l^2 - 1) 2^(..), rounded to 2^-58
+          const __int128 num = (__int128)(l * l - m * m) << (kFxBits + ex[l + 1][m] - ex[l - 1][m]);
+          const long long den = 4 * l * l - 1, qq = -(long long)((2 * num + den) / (2 * den));
+          const long long lo = (long long)((unsigned long long)qq << (64 - kFxLimb)) >> (64 - kFxLimb);
+          s.x = (int)((qq - lo) >> kFxLimb);
+          s.y = (int)lo;
+        }
+        step[set * kSteps + l * (l + 1) / 2 + m] = s;
+        row[set * kRows + harm_index(l, m)] = row[set * kRows + harm_index(l, -m)] = m | ex[l][m] << 8 | l << 16;
+      }
   }
+  double far[(kLamDer + 1) * (kLamDer / 2 + 1)] = {}, kf[kLamDer / 2 + 1];
+  for (int L = 0; L <= kLamDer; ++L) {
+    long double g = 0.886226925452758013649083741670572591398L, s = 0.0L, jf = 1.0L;  // Gamma(L + j + 1/2) / 2
+    for (int n = 1; n <= L; ++n) g *= (2 * n - 1) / 2.0L;
+    for (int k = 0; k <= kLamDer / 2; ++k) {
+      s += g / jf;
+      far[L * (kLamDer / 2 + 1) + k] = (double)s;
+      g *= (2 * (L + k) + 1) / 2.0L;
+      jf *= k + 1;
+    }
+  }
+  kf[0] = 6.283185307179586476925286766559;
+  for (int k = 1; k <= kLamDer / 2; ++k) kf[k] = kf[k - 1] * k;
+  cudaError_t e = cudaMemcpyToSymbol(k_boys, &boys_const_host(), sizeof(BoysConst));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(k_step, step.data(), sizeof(int4) * step.size());
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_row, row.data(), sizeof(int) * row.size());
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_far, far, sizeof(far));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_kfact, kf, sizeof(kf));
+  const std::vector<double>& bt = tables_host().boys_top;
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_boys_top, bt.data(), sizeof(double) * bt.size());
+  for (int lam = 0; lam <= kLamDer && e == cudaSuccess; ++lam)
+    e = set_max_dynamic_smem((const void*)kernel_at(lam, Lams{}));
   return e;
 }
 
-cudaError_t launch_coupling_fp64(int lam, int nch, const CouplingArgs& args, int grid, cudaStream_t stream) {
-  const int nw = coupling_warps(lam, args.one_warp_ok != 0);
-  const CouplingKernel k = coupling_kernel(lam, nch, nw);
-  if (!k) return cudaErrorInvalidValue;
-  // one-warp blocks: twice the blocks for the same warps per SM
-  if (nw == 1) grid = (int)std::min<int64_t>(2 * (int64_t)grid, std::max<int64_t>(args.npp, 1));
-  k<<<grid, 32 * nw, coupling_fp64_smem(lam, nch), stream>>>(args);
+cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, int grid, cudaStream_t stream) {
+  if (lam < 0 || lam > kLamDer) return cudaErrorInvalidValue;
+  kernel_at(lam, Lams{})<<<grid, 32 * coupling_warps(lam), smem_at(lam, Lams{}), stream>>>(args);
   return cudaGetLastError();
 }
 

@@ -677,7 +677,7 @@ constexpr Kernel kernel_at(int lam, std::integer_sequence<int, L...>) {
 }
 
 // Two warps per block up to Lambda = 8 (measured: the batched workload 6 % faster, the high-l molecule 1.5 %),
-// for the bases that allow the smaller blocks (CouplingArgs::one_warp_ok).
+// for the bases that allow the smaller blocks (CouplingArgs::small_blocks_ok).
 constexpr int kTwoWarpLamMax = 8;
 int f32_warps(int lam, bool small_ok) { return small_ok && lam <= kTwoWarpLamMax ? 2 : 4; }
 
@@ -757,7 +757,7 @@ cudaError_t coupling_f32_setup() {
 cudaError_t launch_coupling_f32(int lam, bool compensated, const CouplingArgs& args, int grid, cudaStream_t stream) {
   if (lam < 0 || lam > kLamMax || !args.boys_ff || !args.exp_ff || !args.items || !args.rnorm_ff)
     return cudaErrorInvalidValue;
-  const int nw = f32_warps(lam, args.one_warp_ok != 0);
+  const int nw = f32_warps(lam, args.small_blocks_ok != 0);
   const Kernel k = nw == 2 ? (compensated ? kernel_at<true, 2>(lam, Lams{}) : kernel_at<false, 2>(lam, Lams{}))
                            : (compensated ? kernel_at<true, 4>(lam, Lams{}) : kernel_at<false, 4>(lam, Lams{}));
   // two-warp blocks: twice the blocks

@@ -668,15 +668,13 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
       ca.mv.nbf = nbf;
       ca.centers = centers;
       ca.charges = charges;
-      ca.boys_tab = dt.boys;
       ca.rmap = dt.rmap + th.rmap_off[lam1];
       ca.rnorm = dt.rnorm + th.rmap_off[lam1];
       ca.site_rot = db.site_rot;
       ca.pair_site = db.pair_site;
       ca.ppd = db.ppd;
       ca.rbuf = r1buf;
-      ca.one_warp_ok = db.coupling_one_warp;
-      e = launch_coupling_fp64(lam1, lam1 <= 12 ? 32 : 16, ca, grid_cap_sm(w.npp, 8), s);
+      e = launch_coupling_fp64(lam1, ca, grid_cap_sm(w.npp, 16), s);
       if (e != cudaSuccess) break;
     }
     DerivArgs& d = P.d;

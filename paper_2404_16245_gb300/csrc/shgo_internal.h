@@ -26,6 +26,10 @@ constexpr double kBoysTsw = 40.0;
 constexpr int kBoysNg = 641;
 constexpr int kBoysNmax = kLamMax + 1 + kBoysK;  // 24: F_{Lambda+1} may be needed by the expansion
 constexpr int kBoysStride = kBoysNmax + 2;       // exp slot + orders 0..kBoysNmax
+// Boys values of one top order (the coupling kernel): per order Lambda <= kLamDer a grid of the same spacing up to
+// T = 80, row g holding F_{Lambda+k}(T_g) / k!, k = 0..kBoysK, exp(-T_g) and padding to 16 bytes.
+constexpr int kBoysTopRows = 1281;
+constexpr int kBoysTopStride = kBoysK + 3;
 
 // Sizes of the per-primitive-pair layouts for Lambda = la + lb.
 __host__ __device__ constexpr inline int n_harm(int lam) { return (lam + 1) * (lam + 1); }
@@ -66,6 +70,7 @@ struct __align__(16) GTerm {
 // Host tables, built once per process (long double arithmetic, stored as double).
 struct Tables {
   std::vector<double> boys;  // [kBoysNg][kBoysStride]
+  std::vector<double> boys_top;  // [kLamDer + 1][kBoysTopRows][kBoysTopStride]
   // Real translation tensors: for la, entry (ma, l1, m1, nu) at etab[eoff[la] + ...] with the
   // index ((ma + la) * (la+1)^2 + l1^2 + l1 + m1) * (2 la + 1) + (nu + la - l1) ... packed densely
   // per (ma, l1 m1) over nu = -(la-l1)..(la-l1): see translation_index().
@@ -381,7 +386,7 @@ struct DeviceBasis {
   int64_t rbuf_len = 0;
   int precision = SHGO_PREC_FP64;  // a shgo_precision value
   int prim_bound = 1;              // 1: primitive pairs below the elementwise bound are skipped
-  int coupling_one_warp = 0;       // 1: the FP64 coupling kernel runs one warp per block at small Lambda
+  int f32_small_blocks = 0;        // 1: the FP32-bulk coupling kernel runs two warps per block at small Lambda
   // Bounded coupling buffer: region > 0 means rbuf holds one region of `region` doubles per pool
   // stream and each class runs in chunks of whole shell pairs that fit its stream's region;
   // h_ppoff (host, npairs + 1) gives the primitive-pair offsets used to cut the chunks.
@@ -506,7 +511,6 @@ struct CouplingArgs {
   MolView mv;
   const double* centers = nullptr;
   const double* charges = nullptr;
-  const double* boys_tab = nullptr;
   const int* rmap = nullptr;     // R layout of this Lambda
   const double* rnorm = nullptr; // N_LM per R entry of this Lambda
   const double* site_rot = nullptr;
@@ -518,8 +522,7 @@ struct CouplingArgs {
   const float2* exp_ff = nullptr;
   const int* items = nullptr;         // work items of this Lambda (coupling_f32_items)
   const float2* rnorm_ff = nullptr;   // rnorm of this Lambda as (hi, lo) pairs
-  int one_warp_ok = 0;                // small Lambda may run smaller blocks (DeviceBasis::coupling_one_warp): one
-                                      // warp (FP64) or two (FP32-bulk)
+  int small_blocks_ok = 0;            // small Lambda may run blocks of two warps (DeviceBasis::f32_small_blocks)
 };
 // Arguments of the electrostatic-potential kernel for one class (shgo_coupling.cu).
 struct EspArgs {
@@ -542,11 +545,11 @@ cudaError_t launch_esp_fp64(int lam, const EspArgs& args, cudaStream_t stream);
 // Gradient of the potential: args.phi receives 3 values per point; chunks of 16 points.
 cudaError_t launch_esp_grad_fp64(int lam, const EspArgs& args, cudaStream_t stream);
 
-// Launches the Lambda = lam instantiation with nucleus chunks of nch (16 or 32) on `grid` warps.
-cudaError_t launch_coupling_fp64(int lam, int nch, const CouplingArgs& args, int grid, cudaStream_t stream);
-size_t coupling_fp64_smem(int lam, int nch);
-// Constants and launch attributes of the FP64 coupling kernels on the current device.
+// Launches the Lambda = lam instantiation on `grid` blocks.
+cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, int grid, cudaStream_t stream);
+// Constants and launch attributes of the FP64 coupling kernels on the current device, and of the potential's.
 cudaError_t coupling_fp64_setup();
+cudaError_t esp_fp64_setup();
 
 // Two-centre Coulomb integrals (a|b) of every class of `work` into out (layout of V, both triangles).
 shgo_status launch_coulomb2c(const DeviceBasis& db, const DeviceTables& dt, const Tables& th,
@@ -593,10 +596,8 @@ shgo_status launch_pair_build(const DeviceBasis& db, int64_t npp, cudaStream_t s
 // Fills db.rotd for every ordered centre pair (asynchronous on `stream`).
 shgo_status launch_pair_rotations(const DeviceBasis& db, const DeviceTables& dt, cudaStream_t stream, std::string* err);
 
-// Launch shape of one class: nucleus chunk of the coupling kernel (16 or 32) and threads per
-// block of the pair kernel (32, 64 or 128); 0 = the default rule.
+// Launch shape of one class: threads per block of the pair kernel (32, 64 or 128); 0 = the default rule.
 struct ClassTune {
-  int nch = 0;
   int threads = 0;
 };
 

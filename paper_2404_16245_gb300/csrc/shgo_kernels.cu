@@ -786,6 +786,7 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_harm, &harm_coef_host(), sizeof(HarmCoef));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_boys, &boys_const_host(), sizeof(BoysConst));
   if (e == cudaSuccess) e = coupling_fp64_setup();
+  if (e == cudaSuccess) e = esp_fp64_setup();
   if (e == cudaSuccess) e = coupling_f32_setup();
   if (e == cudaSuccess) {
     int lof[(kLmax + 1) * (kLmax + 1)];
@@ -809,6 +810,7 @@ shgo_status upload_constants(std::string* err) {
   cudaError_t e = cudaMemcpyToSymbol(c_harm, &harm_coef_host(), sizeof(HarmCoef));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_boys, &boys_const_host(), sizeof(BoysConst));
   if (e == cudaSuccess) e = coupling_fp64_setup();
+  if (e == cudaSuccess) e = esp_fp64_setup();
   if (e == cudaSuccess) {
     int lof[(kLmax + 1) * (kLmax + 1)];
     for (int l = 0; l <= kLmax; ++l)
@@ -891,10 +893,6 @@ struct Launcher {
   double* out;
   const std::vector<ClassTune>* tune;  // per entry of `work`, or nullptr for the default shapes
 
-  int nch_of(size_t c, int lam) const {
-    if (tune && (*tune)[c].nch) return (*tune)[c].nch;
-    return lam <= 12 ? 32 : 16;
-  }
   int threads_of(size_t c, int la, int lb) const {
     if (tune && (*tune)[c].threads) return (*tune)[c].threads;
     return pair_threads(la, lb);
@@ -931,7 +929,6 @@ struct Launcher {
   void coupling(const ClassWork& w, size_t c, int64_t rbase, cudaStream_t s) const {
     if (w.npp == 0) return;
     const int lam = w.la + w.lb;
-    const int nch = nch_of(c, lam);
     const int* rmap = dt.rmap + th.rmap_off[lam];
     CouplingArgs a;
     a.q = queue(w, c, 0);
@@ -944,14 +941,13 @@ struct Launcher {
     a.mv = mv;
     a.centers = centers;
     a.charges = charges;
-    a.boys_tab = dt.boys;
     a.rmap = rmap;
     a.rnorm = dt.rnorm + th.rmap_off[lam];
     a.site_rot = db.site_rot;
     a.pair_site = db.pair_site;
     a.ppd = db.ppd;
     a.rbuf = db.rbuf;
-    a.one_warp_ok = db.coupling_one_warp;
+    a.small_blocks_ok = db.f32_small_blocks;
     if (db.precision != SHGO_PREC_FP64) {
       a.boys_ff = dt.boys_ff;
       a.exp_ff = dt.exp_ff;
@@ -960,7 +956,7 @@ struct Launcher {
       launch_coupling_f32(lam, db.precision == SHGO_PREC_FP32_BULK, a, grid_cap(w.npp, 8), s);
       return;
     }
-    launch_coupling_fp64(lam, nch, a, grid_cap(w.npp, 8), s);
+    launch_coupling_fp64(lam, a, grid_cap(w.npp, 16), s);
   }
   void pair(const ClassWork& w, size_t c, int64_t rbase, cudaStream_t s) const {
     if (w.npairs == 0) return;
@@ -1221,24 +1217,9 @@ shgo_status autotune_batched(const DeviceBasis& db, const DeviceTables& dt, cons
     const ClassWork& first = chunks[0];
     std::vector<ClassTune> trial(work.size());
     const Launcher L{db, dt, th, mv, centers, charges, out, &trial};
-    float best = 1e30f;
-    int best_nch = 32;
-    for (int nch : {16, 32}) {
-      trial[c].nch = nch;
-      L.reset(c, stream);
-      L.coupling(first, c, rb, stream);  // warm
-      L.reset(c, stream);
-      const float ms = time_it([&] { L.coupling(first, c, rb, stream); });
-      if (ms < best) {
-        best = ms;
-        best_nch = nch;
-      }
-    }
-    trial[c].nch = best_nch;
     L.reset(c, stream);
-    L.coupling(first, c, rb, stream);  // the kept shape leaves its coupling block in place
-    (*tune)[c].nch = best_nch;
-    best = 1e30f;
+    L.coupling(first, c, rb, stream);
+    float best = 1e30f;
     int best_thr = pair_threads(w.la, w.lb);
     for (int thr : {32, 64, 128}) {
       trial[c].threads = thr;

@@ -274,6 +274,21 @@ void build_tables(Tables& t) {
     t.boys[(size_t)g * kBoysStride] = (double)ex;
     for (int n = 0; n <= kBoysNmax; ++n) t.boys[(size_t)g * kBoysStride + 1 + n] = (double)F[n];
   }
+  // per top order, F_{Lambda+k} / k!, on to T = 80
+  t.boys_top.assign((size_t)(kLamDer + 1) * kBoysTopRows * kBoysTopStride, 0.0);
+  for (int g = 0; g < kBoysTopRows; ++g) {
+    ld F[kBoysNmax + 1], ex;
+    boys_grid_row((ld)g / (ld)kBoysInvH, kBoysNmax, F, &ex);
+    for (int lam = 0; lam <= kLamDer; ++lam) {
+      double* row = &t.boys_top[((size_t)lam * kBoysTopRows + g) * kBoysTopStride];
+      ld kf = 1;
+      for (int k = 0; k <= kBoysK; ++k) {
+        row[k] = (double)(F[lam + k] / kf);
+        kf *= k + 1;
+      }
+      row[kBoysK + 1] = (double)ex;
+    }
+  }
   // Translation tensors
   t.eoff.assign(kLmax + 2, 0);
   for (int la = 0; la <= kLmax; ++la) {
