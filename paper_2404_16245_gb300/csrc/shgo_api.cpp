@@ -970,7 +970,7 @@ shgo_status esp_call(const shgo_basis* basis, const double* density, const shgo_
   if (prev != basis->device) cudaSetDevice(basis->device);
   std::string err;
   const shgo_status st = launch_esp(basis->d, *basis->tabs, basis->work, basis->nbf, density, points->n, points->xyz,
-                                    phi, basis->d.rbuf, gradient, (cudaStream_t)stream, &err);
+                                    phi, gradient, (cudaStream_t)stream, &err);
   if (prev != basis->device) cudaSetDevice(prev);
   if (st != SHGO_OK) return fail(st, err);
   return SHGO_OK;

@@ -132,6 +132,11 @@ struct Tables {
   std::vector<GTerm> d_raise, d_field;
   std::vector<double> d_low;
   std::vector<int> d_low_off;
+  // The transposed field step (gradient of the potential): for Lambda, entry e' of the Lambda + 1 layout and component c,
+  // the entries e of the Lambda layout whose field step (d_field, and -2p times d_raise) reads e':
+  // dt_terms[dt_ptr[dt_base[Lambda] + 3 e' + c] .. + 1] = (coefficient, e, 1 for a d_raise term).
+  std::vector<int> dt_ptr, dt_base;
+  std::vector<GTerm> dt_terms;
   // Four-centre electron repulsion: r^{2k} S_LM(r) e^{-p r^2} = sum_{n<=k} eps_{k,n}(L) p^{-(k+n)}
   // Laplacian^n [S_LM(r) e^{-p r^2}], with eps_{k,n}(L) at eri_eps[(L (kC2K + 1) + k)(kC2K + 1) + n].
   std::vector<double> eri_eps;
@@ -198,6 +203,8 @@ struct DeviceTables {
   GTerm* d_raise = nullptr;
   GTerm* d_field = nullptr;
   double* d_low = nullptr;
+  int* dt_ptr = nullptr;
+  GTerm* dt_terms = nullptr;
 };
 shgo_status device_tables(int device, const DeviceTables** out, std::string* err);
 
@@ -468,10 +475,10 @@ shgo_status launch_class_timed(const DeviceBasis& db, const DeviceTables& dt, co
                                cudaStream_t stream, double* ms, std::string* err);
 
 // Electrostatic potential phi[k] = sum_ab D_ab <a|1/|r - points_k||b> of a single basis (D device,
-// nbf x nbf row-major, symmetric); gbuf holds n_r(Lambda) doubles per primitive pair of every class.
-// gradient = true: phi receives grad_x phi at each point, [npoints][3].
+// nbf x nbf row-major, symmetric); db.h_ppoff must be set.  gradient = true: phi receives grad_x phi at each point,
+// [npoints][3].
 shgo_status launch_esp(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
-                       int64_t nbf, const double* D, int64_t npoints, const double* points, double* phi, double* gbuf,
+                       int64_t nbf, const double* D, int64_t npoints, const double* points, double* phi,
                        bool gradient, cudaStream_t stream, std::string* err);
 
 // Contraction of the centre derivatives with a density (shgo_nuclear_attraction_gradient): P (device,
@@ -524,32 +531,13 @@ struct CouplingArgs {
   const float2* rnorm_ff = nullptr;   // rnorm of this Lambda as (hi, lo) pairs
   int small_blocks_ok = 0;            // small Lambda may run blocks of two warps (DeviceBasis::f32_small_blocks)
 };
-// Arguments of the electrostatic-potential kernel for one class (shgo_coupling.cu).
-struct EspArgs {
-  int64_t npp = 0, pp_base = 0;  // the class's primitive pairs
-  const int* pp_pair = nullptr;
-  const int* pair_a = nullptr;
-  const double* shell_xyz = nullptr;
-  const double* site_rot = nullptr;
-  const int* pair_site = nullptr;
-  const PPData* ppd = nullptr;
-  const double* boys_tab = nullptr;
-  const int* rmap = nullptr;     // R layout of this Lambda
-  const double* gam = nullptr;   // adjoint blocks of the class, n_r(Lambda) per primitive pair
-  int64_t npoints = 0;
-  const double* points = nullptr;
-  double* phi = nullptr;
-  int nchunks = 0, nsplit = 0;   // blocks = nchunks x nsplit
-};
-cudaError_t launch_esp_fp64(int lam, const EspArgs& args, cudaStream_t stream);
-// Gradient of the potential: args.phi receives 3 values per point; chunks of 16 points.
-cudaError_t launch_esp_grad_fp64(int lam, const EspArgs& args, cudaStream_t stream);
-
 // Launches the Lambda = lam instantiation on `grid` blocks.
 cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, int grid, cudaStream_t stream);
 // Constants and launch attributes of the FP64 coupling kernels on the current device, and of the potential's.
 cudaError_t coupling_fp64_setup();
 cudaError_t esp_fp64_setup();
+// Device address of the Boys grid of top order lam (set up by coupling_fp64_setup).
+cudaError_t boys_top_table(int lam, const double2** out);
 
 // Two-centre Coulomb integrals (a|b) of every class of `work` into out (layout of V, both triangles).
 shgo_status launch_coulomb2c(const DeviceBasis& db, const DeviceTables& dt, const Tables& th,

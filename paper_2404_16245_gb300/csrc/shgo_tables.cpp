@@ -252,6 +252,26 @@ void build_deriv_tables(Tables& t) {
             }
           }
   }
+  t.dt_base.assign(kLamMax + 2, 0);
+  t.dt_ptr.clear();
+  t.dt_terms.clear();
+  for (int lam = 0; lam <= kLamMax; ++lam) {
+    t.dt_base[lam] = (int)t.dt_ptr.size();
+    std::vector<std::vector<GTerm>> lists((size_t)3 * n_r(lam + 1));
+    for (int e = 0; e < n_r(lam); ++e)
+      for (int c = 0; c < 3; ++c)
+        for (int which = 0; which < 2; ++which)
+          for (int s = 0; s < kDerivSlots; ++s) {
+            const GTerm& g = (which ? t.d_raise : t.d_field)[((size_t)(t.d_xoff[lam] + e) * 3 + c) * kDerivSlots + s];
+            if (g.coef != 0.0) lists[(size_t)3 * g.ridx + c].push_back(GTerm{g.coef, e, which});
+          }
+    for (const auto& l : lists) {
+      t.dt_ptr.push_back((int)t.dt_terms.size());
+      t.dt_terms.insert(t.dt_terms.end(), l.begin(), l.end());
+    }
+    t.dt_ptr.push_back((int)t.dt_terms.size());
+  }
+  t.dt_base[kLamMax + 1] = (int)t.dt_ptr.size();
   t.d_low_off.assign(kLmax + 2, 0);
   t.d_low.clear();
   for (int l = 0; l <= kLmax; ++l) {
