@@ -1124,7 +1124,7 @@ shgo_status shgo_coulomb_2c(const shgo_basis* basis, double* out, void* stream) 
   }
   mv.nbf = basis->nbf;
   std::string err;
-  const shgo_status st = launch_coulomb2c(basis->d, *basis->tabs, tables_host(), basis->work, mv, out,
+  const shgo_status st = launch_coulomb2c(basis->d, *basis->tabs, basis->work, mv, out,
                                           (cudaStream_t)stream, &err);
   if (prev != basis->device) cudaSetDevice(prev);
   if (st != SHGO_OK) return fail(st, err);

@@ -539,10 +539,12 @@ cudaError_t esp_fp64_setup();
 // Device address of the Boys grid of top order lam (set up by coupling_fp64_setup).
 cudaError_t boys_top_table(int lam, const double2** out);
 
-// Two-centre Coulomb integrals (a|b) of every class of `work` into out (layout of V, both triangles).
-shgo_status launch_coulomb2c(const DeviceBasis& db, const DeviceTables& dt, const Tables& th,
-                             const std::vector<ClassWork>& work, const MolView& mv, double* out, cudaStream_t stream,
-                             std::string* err);
+// Two-centre Coulomb integrals (a|b) of every class of `work` into out (layout of V, both triangles); db.h_ppoff must be
+// set, for launch_overlap too.
+shgo_status launch_coulomb2c(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
+                             const MolView& mv, double* out, cudaStream_t stream, std::string* err);
+// Constants of the overlap and two-centre kernels on the current device.
+cudaError_t twocentre_setup();
 
 // Largest shell l of the four-centre electron-repulsion integrals (la + lb + lc + ld <= 16).
 constexpr int kEriLmax = 4;

@@ -436,151 +436,6 @@ __global__ void __launch_bounds__(128) k_pair_block(int la, int lb, int npairs, 
     });
 }
 
-// Overlap block of one shell pair (Eqs. 9-10): both orbitals translated to P (Eq. 7) in the pair
-// frame, where the one-centre integrals are diagonal by orthogonality,
-//   int S_{l1 m1}(r_P) S_{l2 m2}(r_P) e^{-p r_P^2} = delta delta 4 pi (pi/2)^{1/2} (2 l1 - 1)!! / (2p)^{l1+3/2},
-// so S'[ma][mb] = delta_{ma mb} sum_{l1 >= |ma|} t_A(l1, ma) t_B(l1, ma) w(l1) with
-// w(l1) = sum_ij c~_i c~_j K_ij (beta/p)^{la-l1} (alpha/p)^{lb-l1} 4 pi (pi/2)^{1/2} (2 l1 - 1)!!/(2p)^{l1+3/2};
-// the block is rotated back with D^{la} S' (D^{lb})^T.
-//
-// One launch covers every class: the shell pairs of all classes form one list of work items, class c holding
-// items [first[c], first[c + 1]) (its shell pairs pair_base[c] onwards).  One warp per shell pair, four per
-// block, each with its own slice of shared memory and no block-wide barrier: the work per pair is a few
-// hundred operations behind a short chain of loads, so what counts is how many pairs are in flight.
-constexpr int kOverlapMaxClasses = 64;
-struct OverlapClasses {
-  int n;
-  int first[kOverlapMaxClasses + 1];
-  int pair_base[kOverlapMaxClasses];
-  unsigned char la[kOverlapMaxClasses], lb[kOverlapMaxClasses];
-};
-constexpr int kOverlapWarps = 4;
-
-// Shared doubles of one warp for angular momenta up to lm: D^{la} and D^{lb}, t_A and t_B, w(l1), |b - a|^k,
-// d(m) and X = D^{la} diag(d).
-__host__ __device__ inline int overlap_warp_doubles(int lm) {
-  const int n = 2 * lm + 1;
-  return 3 * n * n + 2 * (lm + 1) * n + 2 * (lm + 1) + n + 1;
-}
-
-__global__ void __launch_bounds__(32 * kOverlapWarps) k_overlap(OverlapClasses cls, int lm_max,
-                                                                const int* __restrict__ pair_a,
-                                                                const int* __restrict__ pair_b,
-                                                                const int64_t* __restrict__ pair_ppoff,
-                                                                const int* __restrict__ pair_site, int64_t rot_per,
-                                                                const double* __restrict__ rotd,
-                                                                const int* __restrict__ shell_nprim,
-                                                                const int64_t* __restrict__ shell_foff,
-                                                                const double* __restrict__ etab,
-                                                                const int* __restrict__ eoff,
-                                                                const PPData* __restrict__ ppd, MolView mv,
-                                                                double* __restrict__ out) {
-  extern __shared__ double smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  double* wsm = smem + wib * overlap_warp_doubles(lm_max);
-  const int total = cls.first[cls.n];
-  for (int item = blockIdx.x * kOverlapWarps + wib; item < total; item += gridDim.x * kOverlapWarps) {
-    int c = 0, hi = cls.n - 1;  // class of the item (uniform over the warp)
-    while (c < hi) {
-      const int mid = (c + hi + 1) >> 1;
-      if (cls.first[mid] <= item)
-        c = mid;
-      else
-        hi = mid - 1;
-    }
-    const int la = cls.la[c], lb = cls.lb[c];
-    const int pr = cls.pair_base[c] + (item - cls.first[c]);
-    const int na = 2 * la + 1, nb = 2 * lb + 1;
-    const int lm = la > lb ? la : lb, ln = la < lb ? la : lb;
-    const int nDb = la != lb ? nb * nb : 0;
-    double* Dm = wsm;  // D^{la}(Q^T), then D^{lb}(Q^T) when lb != la
-    double* tA = Dm + na * na + nb * nb;
-    double* tB = tA + (la + 1) * na;
-    double* wl = tB + (lb + 1) * nb;  // w(l1)
-    double* dpow = wl + lm + 1;       // |b - a|^k
-    double* dm = dpow + lm + 1;       // d(m), m = -ln..ln
-    double* X = dm + 2 * lm + 1;      // [ma][m] = D^{la}[ma][m] d(m)
-    const int nm = 2 * ln + 1;
-    const int a = pair_a[pr], b = pair_b[pr];
-    const double* rd = rotd + (int64_t)pair_site[pr] * rot_per;
-    __syncwarp();  // the warp's previous pair is done with its tables
-    if (lane == 0) {
-      const double dist = rd[0];
-      double v = 1.0;
-      for (int k = 0; k <= lm; ++k) {
-        dpow[k] = v;
-        v *= dist;
-      }
-    }
-    for (int e = lane; e < na * na; e += 32) Dm[e] = rd[1 + rot_doff(la) + e];
-    for (int e = lane; e < nDb; e += 32) Dm[na * na + e] = rd[1 + rot_doff(lb) + e];
-    // radial sums over primitive pairs, one l1 per lane
-    if (lane <= ln) {
-      const int l1 = lane;
-      double dfact = 1.0;
-      for (int k = 2 * l1 - 1; k > 1; k -= 2) dfact *= k;
-      // 4 pi (pi/2)^{1/2} / 2^{l1 + 3/2} (2 l1 - 1)!!
-      double cf = 4.0 * 3.14159265358979323846 * 1.2533141373155002512 * dfact * 0.35355339059327376220;
-      for (int k = 0; k < l1; ++k) cf *= 0.5;
-      const int64_t q0 = pair_ppoff[pr];
-      const int npp = shell_nprim[a] * shell_nprim[b];
-      double acc = 0.0;
-      for (int ij = 0; ij < npp; ++ij) {
-        const PPData pd = ppd[q0 + ij];
-        if (pd.pref == 0.0) continue;
-        double v = pd.pref * pd.rp / pd.sp;  // p^{-3/2}
-        for (int k = 0; k < l1; ++k) v *= pd.rp;
-        for (int k = 0; k < la - l1; ++k) v *= pd.ra;
-        for (int k = 0; k < lb - l1; ++k) v *= pd.rb;
-        acc += v;
-      }
-      wl[l1] = cf * acc;
-    }
-    __syncwarp();
-    for (int e = lane; e < (la + 1) * na; e += 32) {
-      const int l1 = e / na, ma = e % na - la, lr = la - l1;
-      tA[e] = l1 >= (ma < 0 ? -ma : ma) ? etab[eoff[la] + translation_offset_dev(la, ma, l1, ma) + lr] * dpow[lr] : 0.0;
-    }
-    for (int e = lane; e < (lb + 1) * nb; e += 32) {
-      const int l2 = e / nb, mb = e % nb - lb, lr = lb - l2;
-      tB[e] = l2 >= (mb < 0 ? -mb : mb)
-                  ? etab[eoff[lb] + translation_offset_dev(lb, mb, l2, mb) + lr] * ((lr & 1) ? -dpow[lr] : dpow[lr])
-                  : 0.0;
-    }
-    __syncwarp();
-    // S' = diag(d), d(m) = sum_{l1 >= |m|} t_A(l1, m) t_B(l1, m) w(l1) for |m| <= min(la, lb), once per pair
-    if (lane < nm) {
-      const int m = lane - ln, am = m < 0 ? -m : m;
-      double d = 0.0;
-      for (int l1 = am; l1 <= ln; ++l1) d = fma(tA[l1 * na + m + la] * tB[l1 * nb + m + lb], wl[l1], d);
-      dm[lane] = d;
-    }
-    __syncwarp();
-    const double* Da = Dm;
-    const double* Db = la != lb ? Dm + na * na : Dm;
-    for (int e = lane; e < na * nm; e += 32) {
-      const int r = e / nm, j = e - r * nm;
-      X[e] = Da[r * na + j - ln + la] * dm[j];
-    }
-    __syncwarp();
-    // S = X (D^{lb})^T; a diagonal block (a == b) takes the entry below its diagonal from the products of the
-    // entry above it, so it is exactly symmetric
-    const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
-    int64_t obase, ld;
-    mol_output(mv, pr, obase, ld);
-    double* o = out + obase;
-    for (int e = lane; e < na * nb; e += 32) {
-      const int ma = e / nb, mb = e % nb;
-      const bool lower = a == b && ma > mb;
-      const int r = lower ? mb : ma, q = lower ? ma : mb;
-      double s = 0.0;
-      for (int j = 0; j < nm; ++j) s = fma(X[r * nm + j], Db[q * nb + j - ln + lb], s);
-      o[(fa0 + ma) * ld + fb0 + mb] = s;
-      if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = s;
-    }
-  }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -645,6 +500,7 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_boys, &boys_const_host(), sizeof(BoysConst));
   if (e == cudaSuccess) e = coupling_fp64_setup();
   if (e == cudaSuccess) e = esp_fp64_setup();
+  if (e == cudaSuccess) e = twocentre_setup();
   if (e == cudaSuccess) e = coupling_f32_setup();
   if (e == cudaSuccess) {
     int lof[(kLmax + 1) * (kLmax + 1)];
@@ -1170,17 +1026,6 @@ shgo_status live_counts(const DeviceBasis& db, const std::vector<ClassWork>& wor
   return SHGO_OK;
 }
 
-// Two-centre Coulomb integrals (a|b) of one class, one block per shell pair.  With Eq. 3 each primitive is
-// N (2 alpha)^{-l} S_l(grad_A) exp(-alpha |r - A|^2), so for R = A - B (grad_B = -grad_R on functions of R)
-//   (a|b) = c_a c_b (2 alpha)^{-la} (2 beta)^{-lb} (-1)^lb S_la(grad_R) S_lb(grad_R) g(|R|^2),
-//   g(u) = 2 pi^{5/2} / (alpha beta sqrt(alpha + beta)) F_0(rho u),  rho = alpha beta / (alpha + beta),
-// the Coulomb integral of two s Gaussians.  The product rule of solid harmonics (the Gaunt coupling of the
-// pair kernel) gives S_la S_lb = sum_{L,M} G |v|^{2k} S_LM with k = (la + lb - L)/2, Hobson's theorem
-// S_LM(grad) f(u) = 2^L S_LM(R) f^{(L)}(u), and the Laplacian of S_LM(R) f(u) is S_LM(R) (4u f'' + (4L + 6) f'),
-// so every term is 2^L S_LM(R) sum_j a_{k,j}(L) u^j g^{(L+k+j)}(u), with
-// g^{(n)}(u) = 2 pi^{5/2} / (alpha beta sqrt(alpha + beta)) (-rho)^n F_n(rho u).
-// Threads: one primitive pair each for the Boys values, one L each for the radial sums over primitive pairs,
-// one block entry each for the coupling; the block and its transpose are written as in the overlap.
 // Real solid harmonics S_lm(x, y, z), l <= lmax, by columns: thread t of nth takes the columns
 // m = t - lmax, t + nth - lmax, ...; each walks the diagonal chain S_{l+1,+-(l+1)} = c_l (x S_ll -+ y S_{l,-l})
 // (S_11 = x, S_1-1 = y) up to |m| and then S_{l+1,m} = a_lm z S_lm - b_lm r^2 S_{l-1,m} (the recursion of
@@ -1211,154 +1056,6 @@ __device__ void solid_harmonics_columns(int lmax, double x, double y, double z, 
       cur = v;
     }
   }
-}
-
-__global__ void __launch_bounds__(64) k_coulomb2c(int la, int lb, int npairs, int pair_base,
-                                                  const int* __restrict__ pair_a, const int* __restrict__ pair_b,
-                                                  const double* __restrict__ shell_xyz,
-                                                  const int* __restrict__ shell_poff, const int* __restrict__ shell_nprim,
-                                                  const int64_t* __restrict__ shell_foff,
-                                                  const double* __restrict__ prim_exp,
-                                                  const double* __restrict__ prim_coef,
-                                                  const double* __restrict__ boys_tab, const int* __restrict__ c2_ptr,
-                                                  const GTerm* __restrict__ c2_terms, const double* __restrict__ c2_a,
-                                                  MolView mv, double* __restrict__ out) {
-  extern __shared__ double smem[];
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int lam = la + lb, na = 2 * la + 1, nb = 2 * lb + 1, nf = lam + 1;
-  double* S = smem;                      // [(lam + 1)^2] S_LM(R)
-  double* X = S + nf * nf;               // [lam + 1] radial sums over primitive pairs, by L
-  double* F = X + nf;                    // [64][lam + 1] Boys values of a batch of primitive pairs
-  double* pf = F + 64 * nf;              // [64] prefactors
-  double* mr = pf + 64;                  // [64] -rho
-  double* ru = mr + 64;                  // [1] |R|^2
-  for (int w = blockIdx.x; w < npairs; w += gridDim.x) {
-    const int pr = pair_base + w;
-    const int a = pair_a[pr], b = pair_b[pr];
-    const double Rx = shell_xyz[3 * a] - shell_xyz[3 * b], Ry = shell_xyz[3 * a + 1] - shell_xyz[3 * b + 1],
-                 Rz = shell_xyz[3 * a + 2] - shell_xyz[3 * b + 2];
-    const double u = Rx * Rx + Ry * Ry + Rz * Rz;
-    __syncthreads();  // the previous pair is done with S and X
-    solid_harmonics_columns(lam, Rx, Ry, Rz, S, tid, nth);
-    if (tid == 0) *ru = u;
-    if (tid < nf) X[tid] = 0.0;
-    const int npa = shell_nprim[a], npb = shell_nprim[b], npp = npa * npb;
-    for (int q0 = 0; q0 < npp; q0 += 64) {
-      __syncthreads();  // the previous batch is consumed
-      const int q = q0 + tid;
-      if (tid < 64 && q < npp) {
-        const int i = q / npb, j = q - i * npb;
-        const double al = prim_exp[shell_poff[a] + i], be = prim_exp[shell_poff[b] + j];
-        const double rho = al * be / (al + be);
-        double v = prim_coef[shell_poff[a] + i] * prim_coef[shell_poff[b] + j] * 6.2831853071795864769 *
-                   5.5683279968317078453 / (al * be * sqrt(al + be));  // 2 pi^{5/2} = 2 pi x pi^{3/2}
-        const double ia = 0.5 / al, ib = 0.5 / be;
-        for (int k = 0; k < la; ++k) v *= ia;
-        for (int k = 0; k < lb; ++k) v *= ib;
-        pf[tid] = (lb & 1) ? -v : v;
-        mr[tid] = -rho;
-        boys_eval(lam, rho * u, F + tid * nf, 1, boys_tab, c_boys);
-      }
-      __syncthreads();
-      const int nq = min(64, npp - q0);
-      // radial sums: one L per thread (L = la - lb, la - lb + 2, ..., la + lb)
-      const int L = la - lb + 2 * tid;
-      if (L <= lam) {
-        const int k = (lam - L) / 2;
-        const double* ak = c2_a + ((size_t)L * (kC2K + 1) + k) * (kC2K + 1);
-        double acc = X[L];
-        for (int t = 0; t < nq; ++t) {
-          const double* Ft = F + t * nf;
-          double mrp = 1.0;  // (-rho)^{L+k}
-          for (int n = 0; n < L + k; ++n) mrp *= mr[t];
-          double s = 0.0, uj = 1.0;
-          for (int j = 0; j <= k; ++j) {
-            s = fma(ak[j] * uj, mrp * Ft[L + k + j], s);
-            uj *= u;
-            mrp *= mr[t];
-          }
-          acc = fma(pf[t], s, acc);
-        }
-        X[L] = acc;
-      }
-    }
-    __syncthreads();
-    if (tid <= lam) X[tid] = ldexp(X[tid], tid);  // 2^L X_L
-    __syncthreads();
-    // coupling: sum over (L, M) of G 2^L S_LM(R) X_L, one block entry per thread
-    const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
-    int64_t obase, ld;
-    mol_output(mv, pr, obase, ld);
-    double* o = out + obase;
-    const int* ptr = c2_ptr;
-    for (int e = tid; e < na * nb; e += nth) {
-      double v = 0.0;
-      for (int t = ptr[e]; t < ptr[e + 1]; ++t) {
-        const GTerm g = c2_terms[t];
-        v = fma(g.coef * S[g.ridx], X[g.pad], v);
-      }
-      const int ma = e / nb, mb = e - ma * nb;
-      o[(fa0 + ma) * ld + fb0 + mb] = v;
-      if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = v;
-    }
-  }
-}
-
-size_t coulomb2c_smem(int la, int lb) {
-  const int nf = la + lb + 1;
-  return sizeof(double) * ((size_t)nf * nf + nf + 64 * (size_t)nf + 64 + 64 + 1 + 8);
-}
-
-// Launches `launch(w, s)` for every non-empty class of `work`, the classes (which write disjoint blocks) spread
-// over the pool streams, the costliest first (cost: an estimate of the class's work), after the work already
-// queued on `stream`, which then waits for all of them.
-template <typename Cost, typename Launch>
-cudaError_t classes_concurrent(const std::vector<ClassWork>& work, cudaStream_t stream, Cost&& cost, Launch&& launch) {
-  cudaStream_t* pool = nullptr;
-  cudaError_t e = stream_pool(&pool);
-  std::vector<int> order;
-  for (size_t c = 0; c < work.size(); ++c)
-    if (work[c].npairs > 0) order.push_back((int)c);
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(work[x]) > cost(work[y]); });
-  const int ns = (int)std::min<size_t>(order.size(), (size_t)kPoolStreams);
-  cudaEvent_t fork = nullptr;
-  if (e == cudaSuccess && ns > 0) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-  if (e == cudaSuccess && fork) e = cudaEventRecord(fork, stream);
-  for (int i = 0; i < ns && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(pool[i], fork, 0);
-  for (size_t k = 0; k < order.size() && e == cudaSuccess; ++k) {
-    launch(work[order[k]], pool[k % ns]);
-    e = cudaGetLastError();
-  }
-  for (int i = 0; i < ns && fork; ++i) {
-    cudaEvent_t join;
-    if (cudaEventCreateWithFlags(&join, cudaEventDisableTiming) != cudaSuccess) break;
-    cudaEventRecord(join, pool[i]);
-    cudaStreamWaitEvent(stream, join, 0);
-    cudaEventDestroy(join);
-  }
-  if (fork) cudaEventDestroy(fork);
-  return e;
-}
-
-shgo_status launch_coulomb2c(const DeviceBasis& db, const DeviceTables& dt, const Tables& th,
-                             const std::vector<ClassWork>& work, const MolView& mv, double* out, cudaStream_t stream,
-                             std::string* err) {
-  const cudaError_t e = classes_concurrent(
-      work, stream,
-      [](const ClassWork& w) {
-        return (double)w.npp * (w.la + w.lb + 1) + (double)w.npairs * (2 * w.la + 1) * (2 * w.lb + 1);
-      },
-      [&](const ClassWork& w, cudaStream_t s) {
-        k_coulomb2c<<<grid_cap(w.npairs, 16), 64, coulomb2c_smem(w.la, w.lb), s>>>(
-            w.la, w.lb, w.npairs, w.pair_base, db.pair_a, db.pair_b, db.shell_xyz, db.shell_poff, db.shell_nprim,
-            db.shell_foff, db.prim_exp, db.prim_coef, dt.boys, dt.c2_ptr + th.c2_base[class_id(w.la, w.lb)],
-            dt.c2_terms, dt.c2_a, mv, out);
-      });
-  if (e != cudaSuccess) {
-    *err = std::string("two-centre launch: ") + cudaGetErrorString(e);
-    return SHGO_ERR_CUDA;
-  }
-  return launch_error(err);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1902,38 +1599,6 @@ shgo_status launch_eri(const DeviceBasis& db, const DeviceTables& dt, const Tabl
   }
   cudaFreeAsync(dist, stream);
   return st;
-}
-
-shgo_status launch_overlap(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
-                           const MolView& mv, double* out, cudaStream_t stream, std::string* err) {
-  OverlapClasses cls{};
-  int total = 0, lm_max = 0;
-  for (const ClassWork& w : work) {
-    if (w.npairs == 0) continue;
-    if (cls.n == kOverlapMaxClasses) {
-      *err = "overlap: more classes than one launch holds";
-      return SHGO_ERR_INVALID_ARG;
-    }
-    cls.first[cls.n] = total;
-    cls.pair_base[cls.n] = w.pair_base;
-    cls.la[cls.n] = (unsigned char)w.la;
-    cls.lb[cls.n] = (unsigned char)w.lb;
-    ++cls.n;
-    total += w.npairs;
-    lm_max = std::max(lm_max, std::max(w.la, w.lb));
-  }
-  cls.first[cls.n] = total;
-  if (total == 0) return SHGO_OK;
-  const size_t sm = sizeof(double) * (size_t)kOverlapWarps * overlap_warp_doubles(lm_max);
-  k_overlap<<<grid_cap((total + kOverlapWarps - 1) / kOverlapWarps, 12), 32 * kOverlapWarps, sm, stream>>>(
-      cls, lm_max, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, rot_block(db.rot_lmax), db.rotd,
-      db.shell_nprim, db.shell_foff, dt.etab, dt.eoff, db.ppd, mv, out);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    *err = std::string("overlap launch: ") + cudaGetErrorString(e);
-    return SHGO_ERR_CUDA;
-  }
-  return launch_error(err);
 }
 
 cudaError_t ensure_max_dynamic_smem(const void* func, int bytes) {

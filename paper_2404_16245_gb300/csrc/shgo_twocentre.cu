@@ -1,0 +1,393 @@
+// Matrices over shell pairs that depend on the vector between the two centres alone: overlap (Eqs. 9-10) and two-centre
+// Coulomb integrals (a|b).  Both have blocks
+//   B[ma][mb] = sum_{L, M} G(la ma, lb mb; L M) X_L S_LM(n),  L = la - lb, la - lb + 2, ..., la + lb,
+// n the unit vector between the centres and G the product-rule coefficients of solid harmonics; only the X_L differ.
+//
+// Coulomb: with Eq. 3 each primitive is N (2 alpha)^{-l} S_l(grad_A) exp(-alpha |r - A|^2), so for R = A - B
+// (grad_B = -grad_R on functions of R)
+//   (a|b) = c_a c_b (2 alpha)^{-la} (2 beta)^{-lb} (-1)^lb S_la(grad_R) S_lb(grad_R) g(|R|^2),
+//   g(u) = 2 pi^{5/2} / (alpha beta sqrt(alpha + beta)) F_0(rho u),  rho = alpha beta / (alpha + beta),
+// the Coulomb integral of two s Gaussians.  The product rule gives S_la S_lb = sum_{L,M} G |v|^{2k} S_LM with
+// k = (la + lb - L)/2, Hobson's theorem S_LM(grad) f(u) = 2^L S_LM(R) f^{(L)}(u), and the Laplacian of S_LM(R) f(u) is
+// S_LM(R) (4u f'' + (4L + 6) f'), so X_L = 2^L (-|R|)^L sum_j a_{k,j}(L) u^j g^{(L+k+j)}(u), with
+// g^{(n)}(u) = 2 pi^{5/2} / (alpha beta sqrt(alpha + beta)) (-rho)^n F_n(rho u), summed over primitive pairs.
+//
+// Overlap: both orbitals translated to P (Eq. 7) in the pair frame, where the one-centre integrals are diagonal,
+//   int S_{l1 m1}(r_P) S_{l2 m2}(r_P) e^{-p r_P^2} = delta delta 4 pi (pi/2)^{1/2} (2 l1 - 1)!! / (2p)^{l1+3/2},
+// so the block is diagonal there with d(m) = sum_{l1 >= m} K(m, l1) w(l1), and as S_LM(z) = delta_M0 the X_L solve
+// sum_L G(la m, lb m; L 0) X_L = d(m), m = 0..lb: a (lb + 1)^2 system per class, inverted on the host (its condition is
+// below 2.6 for every class to (8, 8)).
+//
+// What bounds it: FP64 at 1.7 lanes per clock and SM.  The scalar steps (Boys values, powers, divisions) therefore run
+// with full lanes, one thread per primitive pair (Coulomb) or shell pair (overlap), in a launch of their own; the
+// harmonics once per pair of centres; a warp per shell pair is left with one product per (L, M) and one multiply-add per
+// coupling coefficient, about five per element.
+//
+// Measured (GB300, 32 atoms with l <= 6, 25,200 shell pairs): (a|b) 421 -> 86 us against one block per shell pair for all
+// steps, overlap 94 -> 78 us against a warp per pair with D^la diag(d) (D^lb)^T.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <string>
+#include <vector>
+
+#include "shgo_internal.h"
+#include "shgo_math.h"
+
+namespace shgo {
+
+namespace {
+
+__constant__ HarmCoef k_harm;
+__constant__ BoysConst k_boys;
+// Per class: K(m, l1) cf(l1) at (m, l1) of a (lb + 1)^2 square (zero below m), then the inverse of G(la m, lb m; L 0) at
+// (j, m), L = la + lb - 2 j; cf(l1) = 4 pi (pi/2)^{1/2} (2 l1 - 1)!! / 2^{l1 + 3/2}.
+constexpr int kOvStride = 2 * (kLmax + 1) * (kLmax + 1);
+__device__ double g_overlap[kNumClasses * kOvStride];
+
+constexpr int kMaxClasses = kNumClasses;
+struct PairClasses {  // classes with pairs: class c holds the items [first[c], first[c + 1])
+  int n;
+  int first[kMaxClasses + 1];
+  int pair_base[kMaxClasses];
+  unsigned char la[kMaxClasses], lb[kMaxClasses];
+};
+
+__device__ __forceinline__ int class_of_item(const PairClasses& cls, int item) {
+  int c = 0, hi = cls.n - 1;
+  while (c < hi) {
+    const int mid = (c + hi + 1) >> 1;
+    if (cls.first[mid] <= item)
+      c = mid;
+    else
+      hi = mid - 1;
+  }
+  return c;
+}
+
+// S_LM(n), L <= lam, of the unit vector n = (B - A)/|B - A| (z for A = B) of every ordered pair of centres: one thread
+// per column M.
+__global__ void __launch_bounds__(128) k_site_harmonics(int n_sites, int lam, const double* __restrict__ site_rot,
+                                                        double* __restrict__ S) {
+  const int ncol = 2 * lam + 1, ns = (lam + 1) * (lam + 1);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)n_sites * ncol;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t site = t / ncol;
+    const int m = (int)(t - site * ncol) - lam, am = m < 0 ? -m : m;
+    const double x = site_rot[9 * site + 6], y = site_rot[9 * site + 7], z = site_rot[9 * site + 8];
+    double* o = S + site * ns;
+    double sp = 1.0, sm = 0.0;  // S_{l,l}, S_{l,-l}
+    if (am >= 1) {
+      sp = x;
+      sm = y;
+      for (int l = 1; l < am; ++l) {
+        const double c = k_harm.c[l];
+        const double np = c * (x * sp - y * sm), nm = c * (y * sp + x * sm);
+        sp = np;
+        sm = nm;
+      }
+    }
+    double prv = 0.0, cur = m < 0 ? sm : sp;
+    o[am * am + am + m] = cur;
+    for (int l = am; l < lam; ++l) {
+      const int k = l * l + l + m;
+      double v = k_harm.a[k] * (z * cur);
+      if (m > -l && m < l) v -= k_harm.b[k] * prv;
+      o[(l + 1) * (l + 1) + l + 1 + m] = v;
+      prv = cur;
+      cur = v;
+    }
+  }
+}
+
+// Coulomb: X of one primitive pair per thread, X[(q - q0) stride + k], L = la + lb - 2k.
+__global__ void __launch_bounds__(128) k_coulomb_radial(int64_t q0, int64_t n, int stride, const int* __restrict__ pp_pair,
+                                                        const int* __restrict__ pp_ij, const int* __restrict__ pair_a,
+                                                        const int* __restrict__ pair_b,
+                                                        const double* __restrict__ shell_xyz,
+                                                        const int* __restrict__ shell_l,
+                                                        const int* __restrict__ shell_poff,
+                                                        const double* __restrict__ prim_exp,
+                                                        const double* __restrict__ prim_coef,
+                                                        const double* __restrict__ boys_tab,
+                                                        const double* __restrict__ c2_a, double* __restrict__ X) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int pr = pp_pair[q0 + i], ij = pp_ij[q0 + i], a = pair_a[pr], b = pair_b[pr];
+    const int la = shell_l[a], lb = shell_l[b], lam = la + lb;
+    const int ia = shell_poff[a] + (ij >> 8), ib = shell_poff[b] + (ij & 255);
+    const double al = prim_exp[ia], be = prim_exp[ib];
+    const double Rx = shell_xyz[3 * a] - shell_xyz[3 * b], Ry = shell_xyz[3 * a + 1] - shell_xyz[3 * b + 1],
+                 Rz = shell_xyz[3 * a + 2] - shell_xyz[3 * b + 2];
+    const double u = Rx * Rx + Ry * Ry + Rz * Rz, r = sqrt(u);
+    const double rp = 1.0 / (al + be), ra = 1.0 / al, rb = 1.0 / be, rho = al * be * rp;
+    double v = prim_coef[ia] * prim_coef[ib] * 34.986836655249725693 * (ra * rb * sqrt(rp));  // 2 pi^{5/2}
+    for (int k = 0; k < la; ++k) v *= 0.5 * ra;
+    for (int k = 0; k < lb; ++k) v *= 0.5 * rb;
+    double H[kLamMax + 1];
+    boys_eval(lam, rho * u, H, 1, boys_tab, k_boys);
+    double f = (lb & 1) ? -v : v;  // v (-rho)^n (-1)^lb
+    for (int k = 0; k <= lam; ++k) {
+      H[k] *= f;
+      f *= -rho;
+    }
+    double rl = 1.0;  // (-2 |R|)^L from the lowest L up
+    for (int k = 0; k < la - lb; ++k) rl *= -2.0 * r;
+    double* o = X + i * stride;
+    for (int k = lb; k >= 0; --k) {
+      const int L = lam - 2 * k;
+      const double* ak = c2_a + ((size_t)L * (kC2K + 1) + k) * (kC2K + 1);
+      double s = 0.0, uj = 1.0;
+      for (int j = 0; j <= k; ++j) {
+        s = fma(ak[j] * uj, H[L + k + j], s);
+        uj *= u;
+      }
+      o[k] = s * rl;
+      rl *= 4.0 * u;
+    }
+  }
+}
+
+// Overlap: X of one shell pair per thread, X[item stride + j], L = la + lb - 2j.
+__global__ void __launch_bounds__(128) k_overlap_radial(PairClasses cls, int stride, const int* __restrict__ pair_a,
+                                                        const int* __restrict__ pair_b,
+                                                        const int64_t* __restrict__ pair_ppoff,
+                                                        const int* __restrict__ pair_site, int64_t rot_per,
+                                                        const double* __restrict__ rotd,
+                                                        const int* __restrict__ shell_nprim,
+                                                        const PPData* __restrict__ ppd, double* __restrict__ X) {
+  const int total = cls.first[cls.n];
+  for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < total; item += gridDim.x * blockDim.x) {
+    const int c = class_of_item(cls, item), la = cls.la[c], lb = cls.lb[c];
+    const int pr = cls.pair_base[c] + (item - cls.first[c]);
+    const int npp = shell_nprim[pair_a[pr]] * shell_nprim[pair_b[pr]];
+    const double r = rotd[(int64_t)pair_site[pr] * rot_per];
+    double w[kLmax + 1];
+    for (int k = 0; k <= lb; ++k) w[k] = 0.0;
+    const PPData* pp = ppd + pair_ppoff[pr];
+    for (int i = 0; i < npp; ++i) {
+      const PPData pd = pp[i];
+      if (pd.pref == 0.0) continue;
+      // w(lb) = pref p^{-3/2} (beta/p)^{la-lb} p^{-lb}, w(l1 - 1) = w(l1) p (beta/p)(alpha/p)
+      double v = pd.pref * pd.rp * (pd.sp * pd.rp);
+      for (int k = 0; k < la - lb; ++k) v *= pd.ra;
+      for (int k = 0; k < lb; ++k) v *= pd.rp;
+      const double f = pd.ra * pd.rb * pd.p;
+      for (int l1 = lb; l1 >= 0; --l1) {
+        w[l1] += v;
+        v *= f;
+      }
+    }
+    // |b - a|^{la - l1} (-|b - a|)^{lb - l1}
+    double rl = 1.0;
+    for (int k = 0; k < la - lb; ++k) rl *= r;
+    for (int l1 = lb; l1 >= 0; --l1) {
+      w[l1] *= rl;
+      rl *= -(r * r);
+    }
+    const double* K = g_overlap + (size_t)(la * (la + 1) / 2 + lb) * kOvStride;
+    const double* Ti = K + (kLmax + 1) * (kLmax + 1);
+    double x[kLmax + 1];
+    for (int j = 0; j <= lb; ++j) x[j] = 0.0;
+    for (int m = 0; m <= lb; ++m) {
+      double d = 0.0;
+      for (int l1 = m; l1 <= lb; ++l1) d = fma(K[m * (lb + 1) + l1], w[l1], d);
+      for (int j = 0; j <= lb; ++j) x[j] = fma(Ti[j * (lb + 1) + m], d, x[j]);
+    }
+    for (int j = 0; j <= lb; ++j) X[(int64_t)item * stride + j] = x[j];
+  }
+}
+
+// Blocks from the X_L: a warp per shell pair, four per block.  nx[] = rows of X per pair: its primitive pairs from
+// pair_ppoff - q0 on (Coulomb), or the item itself (per_pair).
+constexpr int kBlockWarps = 4;
+__global__ void __launch_bounds__(32 * kBlockWarps) k_twocentre_blocks(
+    PairClasses cls, int lam_max, int stride, bool per_pair, int64_t q0, const int* __restrict__ pair_a,
+    const int* __restrict__ pair_b, const int64_t* __restrict__ pair_ppoff, const int* __restrict__ pair_site,
+    const int* __restrict__ shell_nprim, const int64_t* __restrict__ shell_foff, const double* __restrict__ S,
+    const double* __restrict__ X, const int* __restrict__ c2_ptr, const int* __restrict__ c2_cbase,
+    const GTerm* __restrict__ c2_terms, MolView mv, double* __restrict__ out) {
+  extern __shared__ double smem[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, ns = (lam_max + 1) * (lam_max + 1);
+  double* SX = smem + wib * (ns + kLmax + 1);  // [ns] X_L S_LM(n)
+  double* xs = SX + ns;
+  const int total = cls.first[cls.n];
+  for (int item = blockIdx.x * kBlockWarps + wib; item < total; item += gridDim.x * kBlockWarps) {
+    const int c = class_of_item(cls, item), la = cls.la[c], lb = cls.lb[c], lam = la + lb;
+    const int pr = cls.pair_base[c] + (item - cls.first[c]);
+    const int a = pair_a[pr], b = pair_b[pr];
+    const int nx = per_pair ? 1 : shell_nprim[a] * shell_nprim[b];
+    const double* x0 = X + (per_pair ? (int64_t)item : pair_ppoff[pr] - q0) * stride;
+    __syncwarp();  // the warp's previous pair is done with its tables
+    if (lane <= lb) {
+      double s = 0.0;
+      for (int i = 0; i < nx; ++i) s += x0[(int64_t)i * stride + lane];
+      xs[lane] = s;
+    }
+    __syncwarp();
+    const double* Sp = S + (int64_t)pair_site[pr] * ns;
+    for (int k = 0; k <= lb; ++k) {
+      const int L = lam - 2 * k;
+      const double x = xs[k];
+      for (int m = lane; m <= 2 * L; m += 32) SX[L * L + m] = Sp[L * L + m] * x;
+    }
+    __syncwarp();
+    const int* ptr = c2_ptr + c2_cbase[la * (la + 1) / 2 + lb];
+    const int na = 2 * la + 1, nb = 2 * lb + 1;
+    const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
+    int64_t obase, ld;
+    mol_output(mv, pr, obase, ld);
+    double* o = out + obase;
+    for (int e = lane; e < na * nb; e += 32) {
+      const int ma = e / nb, mb = e - ma * nb;
+      // a diagonal block takes the entry below its diagonal from the terms of the one above it: exactly symmetric
+      const int es = a == b && ma > mb ? mb * nb + ma : e;
+      double v = 0.0;
+      for (int t = ptr[es]; t < ptr[es + 1]; ++t) {
+        const GTerm g = c2_terms[t];
+        v = fma(g.coef, SX[g.ridx], v);
+      }
+      o[(fa0 + ma) * ld + fb0 + mb] = v;
+      if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = v;
+    }
+  }
+}
+
+// Doubles of X formed at a time (128 MiB); larger bases run in pieces of whole shell pairs.
+constexpr int64_t kXDoubles = (int64_t)1 << 24;
+
+shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTables& dt,
+                             const std::vector<ClassWork>& work, const MolView& mv, double* out, cudaStream_t stream,
+                             std::string* err) {
+  const int lam_max = 2 * db.rot_lmax, stride = db.rot_lmax + 1, ns = (lam_max + 1) * (lam_max + 1);
+  int64_t npairs = 0, npp = 0;
+  for (const ClassWork& w : work) {
+    npairs += w.npairs;
+    npp += w.npp;
+  }
+  if (npairs == 0) return SHGO_OK;
+  // pieces: consecutive (class, pairs) runs whose rows of X fit
+  std::vector<std::vector<ClassWork>> pieces(1);
+  int64_t rows = 0, most = 0;
+  for (const ClassWork& w : work) {
+    for (int q = w.pair_base; q < w.pair_base + w.npairs;) {
+      ClassWork c{w.la, w.lb, 0, q, 0, db.h_ppoff[q]};
+      int64_t r = 0;
+      while (q < w.pair_base + w.npairs) {
+        const int64_t add = coulomb ? db.h_ppoff[q + 1] - db.h_ppoff[q] : 1;
+        if (rows + r + add > std::max<int64_t>(kXDoubles / stride, 1) && rows + r > 0) break;
+        r += add;
+        ++c.npairs;
+        ++q;
+      }
+      c.npp = db.h_ppoff[q] - c.pp_base;
+      if (c.npairs) pieces.back().push_back(c);
+      rows += r;
+      most = std::max(most, rows);
+      if (q < w.pair_base + w.npairs) {
+        pieces.emplace_back();
+        rows = 0;
+      }
+    }
+  }
+  double* buf = nullptr;  // S of every pair of centres, then X
+  cudaError_t e = cudaMallocAsync((void**)&buf, sizeof(double) * ((size_t)db.n_sites * ns + (size_t)most * stride), stream);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *err = std::string("two-centre buffers: ") + cudaGetErrorString(e);
+    return SHGO_ERR_OOM;
+  }
+  double *S = buf, *X = buf + (size_t)db.n_sites * ns;
+  k_site_harmonics<<<grid_cap_sm(((int64_t)db.n_sites * (2 * lam_max + 1) + 127) / 128, 16), 128, 0, stream>>>(
+      db.n_sites, lam_max, db.site_rot, S);
+  for (const std::vector<ClassWork>& piece : pieces) {
+    if (piece.empty()) continue;
+    PairClasses cls{};
+    int total = 0;
+    int64_t pp = 0;
+    for (const ClassWork& w : piece) {
+      cls.first[cls.n] = total;
+      cls.pair_base[cls.n] = w.pair_base;
+      cls.la[cls.n] = (unsigned char)w.la;
+      cls.lb[cls.n] = (unsigned char)w.lb;
+      ++cls.n;
+      total += w.npairs;
+      pp += w.npp;
+    }
+    cls.first[cls.n] = total;
+    const int64_t q0 = piece[0].pp_base;
+    if (coulomb)
+      k_coulomb_radial<<<grid_cap_sm((pp + 127) / 128, 16), 128, 0, stream>>>(
+          q0, pp, stride, db.pp_pair, db.pp_ij, db.pair_a, db.pair_b, db.shell_xyz, db.shell_l, db.shell_poff, db.prim_exp,
+          db.prim_coef, dt.boys, dt.c2_a, X);
+    else
+      k_overlap_radial<<<grid_cap_sm(((int64_t)total + 127) / 128, 16), 128, 0, stream>>>(
+          cls, stride, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, rot_block(db.rot_lmax), db.rotd, db.shell_nprim,
+          db.ppd, X);
+    k_twocentre_blocks<<<grid_cap_sm(((int64_t)total + kBlockWarps - 1) / kBlockWarps, 12), 32 * kBlockWarps,
+                         sizeof(double) * kBlockWarps * (size_t)(ns + kLmax + 1), stream>>>(
+        cls, lam_max, stride, !coulomb, q0, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, db.shell_nprim,
+        db.shell_foff, S, X, dt.c2_ptr, dt.c2_cbase, dt.c2_terms, mv, out);
+  }
+  e = cudaGetLastError();
+  cudaFreeAsync(buf, stream);
+  if (e != cudaSuccess) {
+    *err = std::string(coulomb ? "two-centre launch: " : "overlap launch: ") + cudaGetErrorString(e);
+    return SHGO_ERR_CUDA;
+  }
+  return SHGO_OK;
+}
+
+}  // namespace
+
+shgo_status launch_overlap(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
+                           const MolView& mv, double* out, cudaStream_t stream, std::string* err) {
+  return launch_twocentre(false, db, dt, work, mv, out, stream, err);
+}
+
+shgo_status launch_coulomb2c(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
+                             const MolView& mv, double* out, cudaStream_t stream, std::string* err) {
+  return launch_twocentre(true, db, dt, work, mv, out, stream, err);
+}
+
+cudaError_t twocentre_setup() {
+  std::vector<double> ov((size_t)kNumClasses * kOvStride, 0.0);
+  for (int la = 0; la <= kLmax; ++la)
+    for (int lb = 0; lb <= la; ++lb) {
+      const int n = lb + 1;
+      double* K = ov.data() + (size_t)class_id(la, lb) * kOvStride;
+      double* Ti = K + (kLmax + 1) * (kLmax + 1);
+      std::vector<long double> A((size_t)n * 2 * n, 0.0L);  // [G | 1], reduced to [1 | G^-1]
+      for (int m = 0; m < n; ++m) {
+        long double cf = 4.0L * 3.14159265358979323846264338328L * 1.25331413731550025120788264241L *
+                         0.353553390593273762200422181052L;  // 4 pi (pi/2)^{1/2} 2^{-3/2}
+        for (int l1 = 0; l1 < n; ++l1) {
+          if (l1 > 0) cf *= (2 * l1 - 1) / 2.0L;
+          if (l1 >= m)
+            K[m * n + l1] = (double)((long double)translation_real(la, m, l1, m, 0) * translation_real(lb, m, l1, m, 0) * cf);
+        }
+        for (int j = 0; j < n; ++j) A[m * 2 * n + j] = gaunt_real(la, m, lb, m, la + lb - 2 * j, 0);
+        A[m * 2 * n + n + m] = 1.0L;
+      }
+      for (int c = 0; c < n; ++c) {
+        int p = c;
+        for (int r = c + 1; r < n; ++r)
+          if (std::fabs(A[r * 2 * n + c]) > std::fabs(A[p * 2 * n + c])) p = r;
+        for (int k = 0; k < 2 * n; ++k) std::swap(A[c * 2 * n + k], A[p * 2 * n + k]);
+        const long double d = A[c * 2 * n + c];
+        for (int k = 0; k < 2 * n; ++k) A[c * 2 * n + k] /= d;
+        for (int r = 0; r < n; ++r) {
+          if (r == c) continue;
+          const long double f = A[r * 2 * n + c];
+          for (int k = 0; k < 2 * n; ++k) A[r * 2 * n + k] -= f * A[c * 2 * n + k];
+        }
+      }
+      for (int j = 0; j < n; ++j)
+        for (int m = 0; m < n; ++m) Ti[j * n + m] = (double)A[j * 2 * n + n + m];
+    }
+  cudaError_t e = cudaMemcpyToSymbol(g_overlap, ov.data(), sizeof(double) * ov.size());
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(k_harm, &harm_coef_host(), sizeof(HarmCoef));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(k_boys, &boys_const_host(), sizeof(BoysConst));
+  return e;
+}
+
+}  // namespace shgo
