@@ -200,6 +200,7 @@ void release(shgo_basis* b) {
   if (b->h_err) release_status_word(b->h_err);
   for (void* p : b->allocations) cudaFreeAsync(p, 0);
   cudaStreamSynchronize(0);
+  workspace_user(b->device, -1);
   cudaSetDevice(prev);
   delete b;
 }
@@ -290,6 +291,7 @@ shgo_status build_basis(int32_t n_shells, const int32_t* l, const int32_t* n_pri
 
   auto* b = new shgo_basis();
   b->device = device;
+  workspace_user(device, 1);
   b->n_shells = n_shells;
   b->d.precision = opt ? opt->precision : SHGO_PREC_FP64;
   b->d.prim_bound = (flags & SHGO_FLAG_NO_PRIM_BOUND) ? 0 : 1;

@@ -619,10 +619,10 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
   double* r1buf = nullptr;
   double* scr = nullptr;
   double* partial = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&r1buf, sizeof(double) * (size_t)std::max<int64_t>(r1_total, 1), stream);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&scr, sizeof(double) * (size_t)std::max<int64_t>(scr_total, 1), stream);
+  cudaError_t e = workspace_alloc((void**)&r1buf, sizeof(double) * (size_t)std::max<int64_t>(r1_total, 1), stream);
+  if (e == cudaSuccess) e = workspace_alloc((void**)&scr, sizeof(double) * (size_t)std::max<int64_t>(scr_total, 1), stream);
   if (e == cudaSuccess && contract)
-    e = cudaMallocAsync((void**)&partial, sizeof(double) * 6 * (size_t)std::max<int64_t>(npairs_all, 1), stream);
+    e = workspace_alloc((void**)&partial, sizeof(double) * 6 * (size_t)std::max<int64_t>(npairs_all, 1), stream);
   if (e != cudaSuccess) {
     if (r1buf) cudaFreeAsync(r1buf, stream);
     if (scr) cudaFreeAsync(scr, stream);

@@ -561,7 +561,7 @@ cudaError_t launch_pieces(const DeviceBasis& db, const DeviceTables& dt, const s
     total += region[i];
   }
   int2* buf = nullptr;
-  e = cudaMallocAsync((void**)&buf, sizeof(int2) * (size_t)std::max<int64_t>(total, 1), stream);
+  e = workspace_alloc((void**)&buf, sizeof(int2) * (size_t)std::max<int64_t>(total, 1), stream);
   if (e != cudaSuccess) return e;
   cudaEvent_t fork = nullptr;
   e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);

@@ -499,6 +499,10 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
                                  int64_t nbf, int64_t ncenters, const double* centers, const double* charges,
                                  double* out, bool field, cudaStream_t stream, std::string* err,
                                  const DerivContraction* contract = nullptr);
+// Work array of a call, stream-ordered (released with cudaFreeAsync), from the library's per-device pool; a basis counts
+// as a user of its device's pool while it lives, and the pool gives its memory back with the last one.
+cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t stream);
+void workspace_user(int device, int change);
 // The per-device pool of non-blocking streams on which the classes of one call run concurrently.
 cudaError_t pool_streams(cudaStream_t** out, int* n);
 // Blocks for n units of work, at most per_sm per SM.

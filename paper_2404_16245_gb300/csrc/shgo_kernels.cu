@@ -1523,7 +1523,7 @@ shgo_status launch_eri(const DeviceBasis& db, const DeviceTables& dt, const Tabl
   }
   const int64_t region = std::max<int64_t>(std::min<int64_t>(need_max, cap), one_max);
   double* dist = nullptr;
-  e = cudaMallocAsync((void**)&dist, sizeof(double) * (size_t)(doff[nw] + (int64_t)ns * region), stream);
+  e = workspace_alloc((void**)&dist, sizeof(double) * (size_t)(doff[nw] + (int64_t)ns * region), stream);
   if (e != cudaSuccess) {
     *err = std::string("distribution and scratch buffers: ") + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? SHGO_ERR_OOM : SHGO_ERR_CUDA;

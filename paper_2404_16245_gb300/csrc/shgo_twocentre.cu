@@ -290,7 +290,7 @@ shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTa
     }
   }
   double* buf = nullptr;  // S of every pair of centres, then X
-  cudaError_t e = cudaMallocAsync((void**)&buf, sizeof(double) * ((size_t)db.n_sites * ns + (size_t)most * stride), stream);
+  cudaError_t e = workspace_alloc((void**)&buf, sizeof(double) * ((size_t)db.n_sites * ns + (size_t)most * stride), stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     *err = std::string("two-centre buffers: ") + cudaGetErrorString(e);
