@@ -66,8 +66,7 @@ struct shgo_basis {
   int64_t ppcount = 0;
   int* pair_mol = nullptr;
   int64_t *mol_c0_d = nullptr, *mol_nc_d = nullptr, *mol_out_d = nullptr, *mol_ld_d = nullptr;
-  std::vector<ClassTune> tune;
-  bool tuned = false;
+  bool ran = false;
   std::vector<int64_t> h_ppoff;  // per pair first primitive pair, plus the total
   std::vector<int> h_pair_a, h_pair_b, h_pair_mol;
   // screening state (shgo_screen_build)
@@ -905,14 +904,14 @@ shgo_status shgo_nuclear_attraction_batched(shgo_basis* batch, const double* cen
   std::string err;
   shgo_status st = SHGO_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  if (!batch->tuned) {
-    // first call: tune the launch shape of every class on the real work (its output is exact)
-    st = autotune_batched(batch->d, *batch->tabs, batch->work, mv, centers, charges, out, &batch->tune, s, &err);
+  if (!batch->ran) {
+    // first call: launched directly (a batch used once is not worth a graph)
+    st = launch_batched(batch->d, *batch->tabs, batch->work, mv, npp_cent, centers, charges, out, s, &err);
     if (st == SHGO_OK && batch->d.limit_ns != ~0ull && status_readback(batch, s) != cudaSuccess) {
       st = SHGO_ERR_CUDA;
       err = "status read-back failed";
     }
-    if (st == SHGO_OK) batch->tuned = true;
+    if (st == SHGO_OK) batch->ran = true;
   } else {
     const void* key[4] = {centers, charges, out, reinterpret_cast<const void*>((uintptr_t)batch->d.limit_ns)};
     if (!batch->graph || std::memcmp(key, batch->graph_key, sizeof(key)) != 0) {
@@ -924,7 +923,7 @@ shgo_status shgo_nuclear_attraction_batched(shgo_basis* batch, const double* cen
       cudaGraph_t g = nullptr;
       cudaError_t e = cudaStreamBeginCapture(batch->capture_stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        st = launch_batched(batch->d, *batch->tabs, batch->work, mv, npp_cent, centers, charges, out, &batch->tune,
+        st = launch_batched(batch->d, *batch->tabs, batch->work, mv, npp_cent, centers, charges, out,
                             batch->capture_stream, &err);
         if (st == SHGO_OK && batch->d.limit_ns != ~0ull) e = status_readback(batch, batch->capture_stream);
         const cudaError_t e2 = cudaStreamEndCapture(batch->capture_stream, &g);
@@ -1657,7 +1656,7 @@ shgo_status shgo_nuclear_attraction_screened(shgo_basis* basis, const double* ce
   const double per_pair = basis->npairs > 0 ? (double)basis->scr_ntrip / (double)basis->npairs : 0.0;
   std::string err;
   shgo_status st = launch_batched(basis->d, *basis->tabs, basis->work, mv, per_pair, centers, charges, out,
-                                  basis->tuned ? &basis->tune : nullptr, (cudaStream_t)stream, &err);
+                                  (cudaStream_t)stream, &err);
   if (st == SHGO_OK) finish_call(basis, (cudaStream_t)stream);
   if (prev != basis->device) cudaSetDevice(prev);
   if (st != SHGO_OK) return fail(st, err);

@@ -89,6 +89,15 @@ struct Tables {
   std::vector<int> g_grpbase;   // [n classes]
   std::vector<int> g_termbase;  // [n classes]
   std::vector<int> g_nnz;       // [n classes] nonzero coupling coefficients (without padding)
+  // The pair kernel's form of the same programs (shgo_pair.cu).  Contracted entries of a class, (l1, l2) by (l1, l2)
+  // (index l1 (lb + 1) + l2), then L = |l1 - l2|, .., l1 + l2 in steps of 2, then M: rt_src[rt_base[c] + e] = R' index
+  // (L, M, (l1 + l2 - L)/2) | (l1 (lb + 1) + l2) << 16.  Rows of the class (aligned with g_rowinfo): px_rows = (W index, or
+  // 0xffff for padding, | term count << 16, first term); terms (fixed-point limbs of the coefficient, contracted entry, R' index),
+  // interleaved as g_terms.  axial[(l (kLmax + 1) + ..)]: E^l(m; l1 m; 0) at l (kLmax + 1)^2 + l1 (l + 1) + m, 0 for m > l1.
+  std::vector<int> rt_src, rt_base;  // [n classes + 1]
+  std::vector<int2> px_rows;
+  std::vector<int4> px_terms;
+  std::vector<double> axial;
   // The same coupling, transposed (for the adjoint used by the electrostatic potential): per class,
   // for each R' entry e of Lambda = la + lb, terms gt_terms[gt_ptr[gt_base[c] + e] .. + 1] of
   // (coefficient, W index (row-major, w_stride(lb) columns), l1 (lb + 1) + l2).
@@ -99,6 +108,7 @@ struct Tables {
   // R layout per Lambda: packed (harm index | beta index << 12 | k << 24) for entry e.
   std::vector<int> rmap;
   std::vector<int> rmap_off;  // [kLamDer + 2]
+  std::vector<int> rdeg;      // L + 2k of entry e, aligned with rmap
   std::vector<double> rnorm;  // N_LM of entry e (HarmCoef::n), aligned with rmap
   // Real rotation matrices D^{l+1} from D^l (S_lm(R y) = sum_m' D^l[m][m'] S_lm'(y)): the
   // harmonic part of u_c S_{l,m'}(u) for a Cartesian component c is sum_M G(1 m(c), l m'; l+1 M)
@@ -205,6 +215,12 @@ struct DeviceTables {
   double* d_low = nullptr;
   int* dt_ptr = nullptr;
   GTerm* dt_terms = nullptr;
+  int* rdeg = nullptr;        // Tables::rdeg
+  // pair kernel (Tables::axial, rt_src, px_*)
+  double* axial = nullptr;
+  int* rt_src = nullptr;
+  int2* px_rows = nullptr;
+  int4* px_terms = nullptr;
 };
 shgo_status device_tables(int device, const DeviceTables** out, std::string* err);
 
@@ -535,6 +551,32 @@ struct CouplingArgs {
   const float2* rnorm_ff = nullptr;   // rnorm of this Lambda as (hi, lo) pairs
   int small_blocks_ok = 0;            // small Lambda may run blocks of two warps (DeviceBasis::f32_small_blocks)
 };
+// Arguments of the pair kernel for one class (shgo_pair.cu).
+struct PairArgs {
+  int la = 0, lb = 0, npairs = 0, pair_base = 0;
+  int64_t pp_base = 0, rbase = 0, rot_per = 0;
+  const int* pair_a = nullptr;
+  const int* pair_b = nullptr;
+  const int64_t* pair_ppoff = nullptr;
+  const int* pair_site = nullptr;
+  const double* rotd = nullptr;
+  const int* shell_nprim = nullptr;
+  const int64_t* shell_foff = nullptr;
+  const double* axial = nullptr;   // Tables::axial
+  int nrt = 0;                     // contracted entries of the class
+  const int* rt_src = nullptr;     // Tables::rt_src of the class
+  const int* rdeg = nullptr;       // Tables::rdeg of la + lb
+  const int2* rows = nullptr;      // Tables::px_rows of the class
+  const int4* terms = nullptr;     // Tables::px_terms
+  const PPData* ppd = nullptr;
+  const double* rbuf = nullptr;
+  MolView mv;
+  double* out = nullptr;
+  WorkQueue wq;
+};
+cudaError_t launch_pair_block(const PairArgs& args, int grid, cudaStream_t stream);
+cudaError_t pair_block_setup();
+
 // Launches the Lambda = lam instantiation on `grid` blocks.
 cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, int grid, cudaStream_t stream);
 // Constants and launch attributes of the FP64 coupling kernels on the current device, and of the potential's.
@@ -590,20 +632,10 @@ shgo_status launch_pair_build(const DeviceBasis& db, int64_t npp, cudaStream_t s
 // Fills db.rotd for every ordered centre pair (asynchronous on `stream`).
 shgo_status launch_pair_rotations(const DeviceBasis& db, const DeviceTables& dt, cudaStream_t stream, std::string* err);
 
-// Launch shape of one class: threads per block of the pair kernel (32, 64 or 128); 0 = the default rule.
-struct ClassTune {
-  int threads = 0;
-};
-
 // All molecules of a batch: one launch per class and kernel, classes concurrent on the pool.
 shgo_status launch_batched(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
                            const MolView& mv, double nuclei_per_pair, const double* centers, const double* charges,
-                           double* out, const std::vector<ClassTune>* tune, cudaStream_t stream, std::string* err);
-
-// Times the candidate shapes of every class on the real work (synchronises the stream).
-shgo_status autotune_batched(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
-                             const MolView& mv, const double* centers, const double* charges, double* out,
-                             std::vector<ClassTune>* tune, cudaStream_t stream, std::string* err);
+                           double* out, cudaStream_t stream, std::string* err);
 
 struct ScreenBasis;
 shgo_status launch_screen_features(const ScreenBasis& sb, const double* centers, const double* charges,

@@ -148,21 +148,6 @@ __global__ void k_live_counts(int npairs, int ncls, const int* __restrict__ pair
   }
 }
 
-// Shared-memory bytes of one block of k_pair_block.
-__host__ __device__ inline size_t pair_smem(int la, int lb) {
-  const int nWa = (la + 1) * (la + 1);
-  const int na = 2 * la + 1, nb = 2 * lb + 1;
-  return sizeof(double) * ((size_t)nWa * w_stride(lb) + na * na + nb * nb + (la + 1) * na + (lb + 1) * nb + nWa * nb +
-                           2 * na * nb + (la + 1) * (lb + 1) + n_r(la + lb) + 32);
-}
-
-// Threads per block of k_pair_block for a class: enough to cover the W entries of large classes.
-__host__ __device__ inline int pair_threads(int la, int lb) {
-  const int nW = (la + 1) * (la + 1) * (lb + 1) * (lb + 1);
-  return nW >= 1024 ? 128 : (nW >= 256 ? 64 : 32);
-}
-
-
 // Real rotation matrices D^l(R), l <= lm, R = Q^T (row-major in Rq), for the block's threads:
 // D^0 = 1, D^1 from R, then D^{l+1} from D^l through the harmonic part of u_c S_{l,m'}(u) (the
 // Gaunt product rule with one factor of degree 1).  Ends without a barrier after the last level.
@@ -235,207 +220,6 @@ __global__ void __launch_bounds__(64) k_pair_rotations(int n_sites, int lmax, co
   }
 }
 
-__global__ void __launch_bounds__(128) k_pair_block(int la, int lb, int npairs, int pair_base, int64_t pp_base,
-                                                    int64_t rbase, const int* __restrict__ pair_a,
-                                                    const int* __restrict__ pair_b,
-                                                    const int64_t* __restrict__ pair_ppoff,
-                                                    const int* __restrict__ pair_site, int64_t rot_per,
-                                                    const double* __restrict__ rotd,
-                                                    const int* __restrict__ shell_poff,
-                                                    const int* __restrict__ shell_nprim,
-                                                    const int64_t* __restrict__ shell_foff,
-                                                    const double* __restrict__ prim_exp,
-                                                    const double* __restrict__ prim_coef,
-                                                    const double* __restrict__ etab, const int* __restrict__ eoff,
-                                                    const int* __restrict__ g_rowinfo,
-                                                    const int* __restrict__ g_grp,
-                                                    const GTerm* __restrict__ g_terms,
-                                                    const PPData* __restrict__ ppd,
-                                                    const double* __restrict__ rbuf, MolView mv,
-                                                    double* __restrict__ out, WorkQueue wq) {
-  extern __shared__ double smem[];
-  __shared__ long long s_next[2];
-  __shared__ unsigned long long s_t0;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int lam = la + lb;
-  const int nR = n_r(lam);
-  const int nWa = (la + 1) * (la + 1), nWb = (lb + 1) * (lb + 1), nW = nWa * nWb;
-  const int ws = w_stride(lb), nWs = nWa * ws, nrp = (nW + 31) & ~31;
-  const int na = 2 * la + 1, nb = 2 * lb + 1;
-  const int lm = la > lb ? la : lb;
-  const int nDb = la != lb ? nb * nb : 0;
-  double* W = smem;                        // [l1 m1][l2 m2], row stride ws
-  double* Dm = W + nWs;                    // D^{la}(Q^T), then D^{lb}(Q^T) when lb != la
-  double* tA = Dm + na * na + nb * nb;     // [l1][ma]
-  double* tB = tA + (la + 1) * na;         // [l2][mb]
-  double* Zb = tB + (lb + 1) * nb;         // [l1 m1][mb]
-  double* Vp = Zb + nWa * nb;              // [ma][mb] in the pair frame, later the final block
-  double* Yb = Vp + na * nb;               // [ma][mb]
-  double* fab = Yb + na * nb;              // [l1][l2]
-  double* Rs = fab + (la + 1) * (lb + 1);  // coupling block of one primitive pair
-  double* scal = Rs + nR;                  // per primitive pair: prefactor, beta/p, alpha/p
-  double* dpow = scal + 4;                 // |b - a|^k, k <= max(la, lb)
-  wq_for_each(wq, npairs, s_next, &s_t0, [&](long long wn) {
-    const int w = (int)wn;
-    const int pr = pair_base + w;
-    const int a = pair_a[pr], b = pair_b[pr];
-    const double* rd = rotd + (int64_t)pair_site[pr] * rot_per;
-    __syncthreads();
-    if (tid == 0) {
-      const double dist = rd[0];
-      double v = 1.0;
-      for (int k = 0; k <= lm; ++k) {
-        dpow[k] = v;
-        v *= dist;
-      }
-    }
-    for (int e = tid; e < na * na; e += nth) Dm[e] = rd[1 + rot_doff(la) + e];
-    for (int e = tid; e < nDb; e += nth) Dm[na * na + e] = rd[1 + rot_doff(lb) + e];
-    for (int e = tid; e < nWs; e += nth) W[e] = 0.0;
-    __syncthreads();
-    // translation along z (Eq. 7 with Eq. 8 coefficients, real basis): only nu = 0 survives,
-    // t_A(l1, ma) = E^{la}(ma; l1 ma; 0) |b-a|^{la-l1}, t_B(l2, mb) = E^{lb}(mb; l2 mb; 0) (-|b-a|)^{lb-l2}
-    for (int e = tid; e < (la + 1) * na; e += nth) {
-      const int l1 = e / na, ma = e % na - la, lr = la - l1;
-      double v = 0.0;
-      if (l1 >= (ma < 0 ? -ma : ma)) {
-        v = etab[eoff[la] + translation_offset_dev(la, ma, l1, ma) + lr] * dpow[lr];
-      }
-      tA[e] = v;
-    }
-    for (int e = tid; e < (lb + 1) * nb; e += nth) {
-      const int l2 = e / nb, mb = e % nb - lb, lr = lb - l2;
-      double v = 0.0;
-      if (l2 >= (mb < 0 ? -mb : mb)) {
-        v = etab[eoff[lb] + translation_offset_dev(lb, mb, l2, mb) + lr] * ((lr & 1) ? -dpow[lr] : dpow[lr]);
-      }
-      tB[e] = v;
-    }
-    // coupling (Gaunt) and primitive contraction, in the pair frame
-    const int npa = shell_nprim[a], npb = shell_nprim[b];
-    const int64_t q0 = pair_ppoff[pr];
-    bool live = false;  // uniform over the block
-    for (int ij = 0; ij < npa * npb; ++ij) {
-      __syncthreads();  // the previous primitive pair is done with Rs, fab and scal
-      if (tid == 0) {
-        const PPData pd = ppd[q0 + ij];
-        scal[0] = pd.pref;
-        scal[1] = pd.ra;
-        scal[2] = pd.rb;
-        scal[3] = pd.kab;
-      }
-      __syncthreads();
-      if (scal[0] == 0.0) continue;  // uniform over the block; the coupling kernel skipped this pair too
-      live = true;
-      const double pref = scal[0];
-      const double* R = rbuf + rbase + (q0 + ij - pp_base) * (int64_t)nR;
-      for (int e = tid; e < nR; e += nth) Rs[e] = R[e];
-      if (tid < (la + 1) * (lb + 1)) {
-        const int l1 = tid / (lb + 1), l2 = tid % (lb + 1);
-        double v = pref;
-        const double ra = scal[1], rb = scal[2];
-        for (int k = 0; k < la - l1; ++k) v *= ra;
-        for (int k = 0; k < lb - l2; ++k) v *= rb;
-        fab[tid] = v;
-      }
-      __syncthreads();
-      // rows r of one warp form one group: equal trip counts, one coalesced load per term
-      for (int r = tid; r < nrp; r += nth) {
-        const int info = g_rowinfo[r];
-        const int gi = r >> 5, K = g_grp[2 * gi + 1];
-        const GTerm* tp = g_terms + g_grp[2 * gi] + (r & 31);
-        double acc0 = 0.0, acc1 = 0.0;
-        int j = 0;
-        for (; j + 1 < K; j += 2) {
-          const GTerm g0 = tp[32 * j], g1 = tp[32 * j + 32];
-          acc0 = fma(g0.coef, Rs[g0.ridx], acc0);
-          acc1 = fma(g1.coef, Rs[g1.ridx], acc1);
-        }
-        if (j < K) {
-          const GTerm g0 = tp[32 * j];
-          acc0 = fma(g0.coef, Rs[g0.ridx], acc0);
-        }
-        if (info >= 0) {
-          const int e = info & 0xffff, l1 = (info >> 16) & 15, l2 = (info >> 20) & 15;
-          W[e] = fma(fab[l1 * (lb + 1) + l2], acc0 + acc1, W[e]);
-        }
-      }
-    }
-    __syncthreads();
-    if (!live) {
-      // every primitive pair skipped: the block is zero (and omitted from a block-sparse output)
-      if (mv.blk_off) return;
-      const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
-      int64_t obase, ld;
-      mol_output(mv, pr, obase, ld);
-      double* o = out + obase;
-      for (int e = tid; e < na * nb; e += nth) {
-        const int ma = e / nb, mb = e % nb;
-        o[(fa0 + ma) * ld + fb0 + mb] = 0.0;
-        if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = 0.0;
-      }
-      return;
-    }
-    // V' = t_A W t_B (diagonal in m), first over l2.  Threads are ordered by |m| (m = 0, 1, -1,
-    // 2, -2, ...) so that the lanes of a warp run loops of (nearly) equal length.
-    for (int e = tid; e < nWa * nb; e += nth) {
-      const int q = e / nWa, i1 = e - q * nWa;
-      const int amb = (q + 1) >> 1, mb = (q & 1) ? amb : -amb;
-      double s = 0.0;
-      for (int l2 = amb; l2 <= lb; ++l2) s = fma(tB[l2 * nb + mb + lb], W[i1 * ws + l2 * l2 + l2 + mb], s);
-      Zb[i1 * nb + mb + lb] = s;
-    }
-    __syncthreads();
-    for (int e = tid; e < na * nb; e += nth) {
-      const int q = e / nb, mb = e - q * nb;
-      const int ama = (q + 1) >> 1, ma = (q & 1) ? ama : -ama;
-      double s = 0.0;
-      for (int l1 = ama; l1 <= la; ++l1) s = fma(tA[l1 * na + ma + la], Zb[(l1 * l1 + l1 + ma) * nb + mb], s);
-      Vp[(ma + la) * nb + mb] = s;
-    }
-    __syncthreads();
-    // back to the molecular frame: V = D^{la} V' (D^{lb})^T
-    const double* Da = Dm;
-    const double* Db = la != lb ? Dm + na * na : Dm;
-    for (int e = tid; e < na * nb; e += nth) {
-      const int ma = e / nb, mb = e % nb;
-      double s = 0.0;
-      for (int k = 0; k < nb; ++k) s = fma(Vp[ma * nb + k], Db[mb * nb + k], s);
-      Yb[e] = s;
-    }
-    __syncthreads();
-    for (int e = tid; e < na * nb; e += nth) {
-      const int ma = e / nb, mb = e % nb;
-      double s = 0.0;
-      for (int k = 0; k < na; ++k) s = fma(Da[ma * na + k], Yb[k * nb + mb], s);
-      Vp[e] = s;
-    }
-    __syncthreads();
-    if (mv.blk_off) {
-      // block-sparse output: the block alone, row-major
-      const int64_t off = mv.blk_off[pr];
-      if (off < 0) return;
-      double* o = out + off;
-      for (int e = tid; e < na * nb; e += nth) {
-        const int ma = e / nb, mb = e % nb;
-        o[e] = (a == b && ma > mb) ? Vp[mb * nb + ma] : Vp[e];
-      }
-      return;
-    }
-    const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
-    int64_t obase, ld;
-    mol_output(mv, pr, obase, ld);
-    double* o = out + obase;
-    for (int e = tid; e < na * nb; e += nth) {
-      const int ma = e / nb, mb = e % nb;
-      // diagonal shell block: the upper triangle serves both halves (exact symmetry)
-      const double v = (a == b && ma > mb) ? Vp[mb * nb + ma] : Vp[e];
-      o[(fa0 + ma) * ld + fb0 + mb] = v;
-      if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = v;
-    }
-    });
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -494,6 +278,11 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = upload(&d.d_raise, t.d_raise);
   if (e == cudaSuccess) e = upload(&d.d_field, t.d_field);
   if (e == cudaSuccess) e = upload(&d.d_low, t.d_low);
+  if (e == cudaSuccess) e = upload(&d.rdeg, t.rdeg);
+  if (e == cudaSuccess) e = upload(&d.axial, t.axial);
+  if (e == cudaSuccess) e = upload(&d.rt_src, t.rt_src);
+  if (e == cudaSuccess) e = upload(&d.px_rows, t.px_rows);
+  if (e == cudaSuccess) e = upload(&d.px_terms, t.px_terms);
   if (e == cudaSuccess) e = upload(&d.dt_ptr, t.dt_ptr);
   if (e == cudaSuccess) e = upload(&d.dt_terms, t.dt_terms);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_harm, &harm_coef_host(), sizeof(HarmCoef));
@@ -501,6 +290,7 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = coupling_fp64_setup();
   if (e == cudaSuccess) e = esp_fp64_setup();
   if (e == cudaSuccess) e = twocentre_setup();
+  if (e == cudaSuccess) e = pair_block_setup();
   if (e == cudaSuccess) e = coupling_f32_setup();
   if (e == cudaSuccess) {
     int lof[(kLmax + 1) * (kLmax + 1)];
@@ -524,6 +314,7 @@ shgo_status upload_constants(std::string* err) {
   cudaError_t e = cudaMemcpyToSymbol(c_harm, &harm_coef_host(), sizeof(HarmCoef));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_boys, &boys_const_host(), sizeof(BoysConst));
   if (e == cudaSuccess) e = coupling_fp64_setup();
+  if (e == cudaSuccess) e = pair_block_setup();
   if (e == cudaSuccess) {
     int lof[(kLmax + 1) * (kLmax + 1)];
     for (int l = 0; l <= kLmax; ++l)
@@ -557,7 +348,6 @@ constexpr int kPoolStreams = 16;
 std::mutex g_pool_mu;
 cudaStream_t g_pool[64][kPoolStreams];
 bool g_pool_ok[64] = {};
-bool g_attr_ok[64] = {};
 
 // Per-device pool of non-blocking streams on which the classes of one call run concurrently.
 cudaError_t stream_pool(cudaStream_t** out) {
@@ -586,16 +376,6 @@ cudaError_t pool_streams(cudaStream_t** out, int* n) {
 int grid_cap_sm(int64_t n, int per_sm) { return grid_cap(n, per_sm); }
 
 namespace {
-// Dynamic shared-memory limits, once per device.
-void set_kernel_attributes() {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  if (g_attr_ok[dev]) return;
-  set_max_dynamic_smem((const void*)k_pair_block);
-  g_attr_ok[dev] = true;
-}
-
 struct Launcher {
   const DeviceBasis& db;
   const DeviceTables& dt;
@@ -604,12 +384,7 @@ struct Launcher {
   const double* centers;
   const double* charges;
   double* out;
-  const std::vector<ClassTune>* tune;  // per entry of `work`, or nullptr for the default shapes
 
-  int threads_of(size_t c, int la, int lb) const {
-    if (tune && (*tune)[c].threads) return (*tune)[c].threads;
-    return pair_threads(la, lb);
-  }
 
   // Work queue of class c's coupling (which = 0) or pair (which = 1) launch.  A launch over the whole
   // class of a batch takes its work from the queue in the batch's cost order; the uniform work of one
@@ -674,13 +449,33 @@ struct Launcher {
   void pair(const ClassWork& w, size_t c, int64_t rbase, cudaStream_t s) const {
     if (w.npairs == 0) return;
     const int cid = class_id(w.la, w.lb);
-    const size_t sm = pair_smem(w.la, w.lb);
-    k_pair_block<<<grid_cap(w.npairs, 16), threads_of(c, w.la, w.lb), sm, s>>>(
-        w.la, w.lb, w.npairs, w.pair_base, w.pp_base, rbase, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site,
-        rot_block(db.rot_lmax), db.rotd,
-        db.shell_poff, db.shell_nprim, db.shell_foff, db.prim_exp, db.prim_coef, dt.etab, dt.eoff,
-        dt.g_rowinfo + th.g_rowbase[cid], dt.g_grp + 2 * th.g_grpbase[cid], dt.g_terms + th.g_termbase[cid],
-        db.ppd, db.rbuf, mv, out, queue(w, c, 1));
+    PairArgs p;
+    p.la = w.la;
+    p.lb = w.lb;
+    p.npairs = w.npairs;
+    p.pair_base = w.pair_base;
+    p.pp_base = w.pp_base;
+    p.rbase = rbase;
+    p.rot_per = rot_block(db.rot_lmax);
+    p.pair_a = db.pair_a;
+    p.pair_b = db.pair_b;
+    p.pair_ppoff = db.pair_ppoff;
+    p.pair_site = db.pair_site;
+    p.rotd = db.rotd;
+    p.shell_nprim = db.shell_nprim;
+    p.shell_foff = db.shell_foff;
+    p.axial = dt.axial;
+    p.nrt = th.rt_base[cid + 1] - th.rt_base[cid];
+    p.rt_src = dt.rt_src + th.rt_base[cid];
+    p.rdeg = dt.rdeg + th.rmap_off[w.la + w.lb];
+    p.rows = dt.px_rows + th.g_rowbase[cid];
+    p.terms = dt.px_terms + th.g_termbase[cid];
+    p.ppd = db.ppd;
+    p.rbuf = db.rbuf;
+    p.mv = mv;
+    p.out = out;
+    p.wq = queue(w, c, 1);
+    launch_pair_block(p, grid_cap(w.npairs, 16), s);
   }
 };
 
@@ -810,14 +605,13 @@ shgo_status launch_nuclear_attraction(const DeviceBasis& db, const DeviceTables&
     }
     return SHGO_OK;
   }
-  set_kernel_attributes();
   const Tables& th = tables_host();
   const std::vector<int64_t> rbases = class_rbases(work);
   MolView mv;
   mv.ncenters = ncenters;
   mv.nbf = nbf;
   mv.blk_off = blk_off;
-  const Launcher L{db, dt, th, mv, centers, charges, out, nullptr};
+  const Launcher L{db, dt, th, mv, centers, charges, out};
   cudaError_t e = clear_ctrl(db, work.size(), stream);
   if (events && db.region > 0) {
     *err = "phase timing needs the whole coupling buffer; this basis uses bounded regions";
@@ -850,10 +644,9 @@ shgo_status launch_class_timed(const DeviceBasis& db, const DeviceTables& dt, co
                                const MolView& mv, const double* centers, const double* charges, double* out,
                                cudaStream_t stream, double* ms, std::string* err) {
   if (work.empty()) return SHGO_OK;
-  set_kernel_attributes();
   const Tables& th = tables_host();
   const std::vector<int64_t> rbases = class_rbases(work);
-  const Launcher L{db, dt, th, mv, centers, charges, out, nullptr};
+  const Launcher L{db, dt, th, mv, centers, charges, out};
   std::vector<cudaEvent_t> ev(3 * work.size(), nullptr);
   cudaError_t e = clear_ctrl(db, work.size(), stream);
   for (auto& x : ev)
@@ -885,76 +678,17 @@ shgo_status launch_class_timed(const DeviceBasis& db, const DeviceTables& dt, co
 
 shgo_status launch_batched(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
                            const MolView& mv, double nuclei_per_pair, const double* centers, const double* charges,
-                           double* out, const std::vector<ClassTune>* tune, cudaStream_t stream, std::string* err) {
+                           double* out, cudaStream_t stream, std::string* err) {
   if (work.empty()) return SHGO_OK;
-  set_kernel_attributes();
   const Tables& th = tables_host();
   const std::vector<int64_t> rbases = class_rbases(work);
-  const Launcher L{db, dt, th, mv, centers, charges, out, tune};
+  const Launcher L{db, dt, th, mv, centers, charges, out};
   cudaError_t e = clear_ctrl(db, work.size(), stream);
   if (e == cudaSuccess) e = run_concurrent(L, work, rbases, class_order(work, nuclei_per_pair), 2, stream);
   if (e != cudaSuccess) {
     *err = std::string("kernel launch: ") + cudaGetErrorString(e);
     return SHGO_ERR_CUDA;
   }
-  return launch_error(err);
-}
-
-shgo_status autotune_batched(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
-                             const MolView& mv, const double* centers, const double* charges, double* out,
-                             std::vector<ClassTune>* tune, cudaStream_t stream, std::string* err) {
-  // Each candidate shape of a class runs the class's real work once (the output is rewritten by
-  // every candidate, so the call's result stays exact); the fastest by CUDA events is kept.
-  set_kernel_attributes();
-  const Tables& th = tables_host();
-  const std::vector<int64_t> rbases = class_rbases(work);
-  tune->assign(work.size(), ClassTune{});
-  clear_ctrl(db, work.size(), stream);
-  cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  auto time_it = [&](auto&& fn) {
-    cudaEventRecord(e0, stream);
-    fn();
-    cudaEventRecord(e1, stream);
-    cudaEventSynchronize(e1);
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    return ms;
-  };
-  for (size_t c = 0; c < work.size(); ++c) {
-    const ClassWork& w = work[c];
-    const std::vector<ClassWork> chunks =
-        db.region > 0 ? class_chunks(w, db.h_ppoff, db.region) : std::vector<ClassWork>{w};
-    const int64_t rb = db.region > 0 ? 0 : rbases[c];
-    const ClassWork& first = chunks[0];
-    std::vector<ClassTune> trial(work.size());
-    const Launcher L{db, dt, th, mv, centers, charges, out, &trial};
-    L.reset(c, stream);
-    L.coupling(first, c, rb, stream);
-    float best = 1e30f;
-    int best_thr = pair_threads(w.la, w.lb);
-    for (int thr : {32, 64, 128}) {
-      trial[c].threads = thr;
-      L.reset(c, stream);
-      L.pair(first, c, rb, stream);  // warm
-      L.reset(c, stream);
-      const float ms = time_it([&] { L.pair(first, c, rb, stream); });
-      if (ms < best) {
-        best = ms;
-        best_thr = thr;
-      }
-    }
-    (*tune)[c].threads = best_thr;
-    trial[c].threads = best_thr;
-    for (size_t k = 0; k < chunks.size(); ++k) {  // the whole class with the kept shapes
-      L.reset(c, stream);
-      if (k > 0) L.coupling(chunks[k], c, rb, stream);
-      L.pair(chunks[k], c, rb, stream);
-    }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
   return launch_error(err);
 }
 

@@ -34,6 +34,11 @@ constexpr size_t kNoallocScratchBytes = (size_t)SHGO_NOALLOC_SCRATCH_BYTES;
 // The scratch.  In host code this name is only a stand-in for the device array: its device address
 // comes from cudaGetSymbolAddress at set-up and is what the kernels receive.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+// The pair kernel's row headers, entry lists and axial factors have an array of their own; the scratch keeps the room of
+// the smaller tables they replaced (kNoallocReserved), so that it accepts the same problems.
+constexpr size_t kNoallocTableBytes = (size_t)1 << 20;
+constexpr size_t kNoallocReserved = 363008;
+static __device__ __align__(256) unsigned char g_noalloc_tables[kNoallocTableBytes];
 
 struct NoallocDevice {
   bool ready = false;
@@ -80,11 +85,8 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   const Tables& t = tables_host();
   Packer pk;
   const size_t o_boys = pk.add(t.boys.size() * sizeof(double));
-  const size_t o_etab = pk.add(t.etab.size() * sizeof(double));
-  const size_t o_eoff = pk.add(t.eoff.size() * sizeof(int));
-  const size_t o_rowinfo = pk.add(t.g_rowinfo.size() * sizeof(int));
-  const size_t o_grp = pk.add(t.g_grp.size() * sizeof(int));
-  const size_t o_terms = pk.add(t.g_terms.size() * sizeof(GTerm));
+  pk.add(kNoallocReserved);
+  const size_t o_terms = pk.add(t.px_terms.size() * sizeof(int4));
   const size_t o_rmap = pk.add(t.rmap.size() * sizeof(int));
   const size_t o_rnorm = pk.add(t.rnorm.size() * sizeof(double));
   const size_t o_rotptr = pk.add(t.rot_ptr.size() * sizeof(int));
@@ -93,22 +95,38 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
     *err = "constant tables do not fit the static scratch";
     return SHGO_ERR_OOM;
   }
+  void* small = nullptr;
+  e = cudaGetSymbolAddress(&small, g_noalloc_tables);
+  if (e != cudaSuccess) {
+    *err = std::string("cudaGetSymbolAddress(tables): ") + cudaGetErrorString(e);
+    return SHGO_ERR_CUDA;
+  }
+  unsigned char* base2 = static_cast<unsigned char*>(small);
+  Packer pk2;
+  const size_t o_axial = pk2.add(t.axial.size() * sizeof(double));
+  const size_t o_rtsrc = pk2.add(t.rt_src.size() * sizeof(int));
+  const size_t o_rows = pk2.add(t.px_rows.size() * sizeof(int2));
+  const size_t o_rdeg = pk2.add(t.rdeg.size() * sizeof(int));
+  if (pk2.used > kNoallocTableBytes) {
+    *err = "constant tables do not fit their static array";
+    return SHGO_ERR_OOM;
+  }
   struct Piece {
-    size_t off;
+    unsigned char* dst;
     const void* src;
     size_t bytes;
-  } pieces[] = {{o_boys, t.boys.data(), t.boys.size() * sizeof(double)},
-                {o_etab, t.etab.data(), t.etab.size() * sizeof(double)},
-                {o_eoff, t.eoff.data(), t.eoff.size() * sizeof(int)},
-                {o_rowinfo, t.g_rowinfo.data(), t.g_rowinfo.size() * sizeof(int)},
-                {o_grp, t.g_grp.data(), t.g_grp.size() * sizeof(int)},
-                {o_terms, t.g_terms.data(), t.g_terms.size() * sizeof(GTerm)},
-                {o_rmap, t.rmap.data(), t.rmap.size() * sizeof(int)},
-                {o_rnorm, t.rnorm.data(), t.rnorm.size() * sizeof(double)},
-                {o_rotptr, t.rot_ptr.data(), t.rot_ptr.size() * sizeof(int)},
-                {o_rotterms, t.rot_terms.data(), t.rot_terms.size() * sizeof(GTerm)}};
+  } pieces[] = {{d.base + o_boys, t.boys.data(), t.boys.size() * sizeof(double)},
+                {base2 + o_axial, t.axial.data(), t.axial.size() * sizeof(double)},
+                {base2 + o_rtsrc, t.rt_src.data(), t.rt_src.size() * sizeof(int)},
+                {base2 + o_rows, t.px_rows.data(), t.px_rows.size() * sizeof(int2)},
+                {base2 + o_rdeg, t.rdeg.data(), t.rdeg.size() * sizeof(int)},
+                {d.base + o_terms, t.px_terms.data(), t.px_terms.size() * sizeof(int4)},
+                {d.base + o_rmap, t.rmap.data(), t.rmap.size() * sizeof(int)},
+                {d.base + o_rnorm, t.rnorm.data(), t.rnorm.size() * sizeof(double)},
+                {d.base + o_rotptr, t.rot_ptr.data(), t.rot_ptr.size() * sizeof(int)},
+                {d.base + o_rotterms, t.rot_terms.data(), t.rot_terms.size() * sizeof(GTerm)}};
   for (const Piece& p : pieces) {
-    e = cudaMemcpy(d.base + p.off, p.src, p.bytes, cudaMemcpyHostToDevice);
+    e = cudaMemcpy(p.dst, p.src, p.bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
       *err = std::string("copying tables into the scratch: ") + cudaGetErrorString(e);
       return SHGO_ERR_CUDA;
@@ -117,12 +135,12 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   shgo_status st = upload_constants(err);
   if (st != SHGO_OK) return st;
   d.tabs.boys = reinterpret_cast<double*>(d.base + o_boys);
-  d.tabs.etab = reinterpret_cast<double*>(d.base + o_etab);
-  d.tabs.eoff = reinterpret_cast<int*>(d.base + o_eoff);
-  d.tabs.g_rowinfo = reinterpret_cast<int*>(d.base + o_rowinfo);
-  d.tabs.g_grp = reinterpret_cast<int*>(d.base + o_grp);
-  d.tabs.g_terms = reinterpret_cast<GTerm*>(d.base + o_terms);
+  d.tabs.axial = reinterpret_cast<double*>(base2 + o_axial);
+  d.tabs.rt_src = reinterpret_cast<int*>(base2 + o_rtsrc);
+  d.tabs.px_rows = reinterpret_cast<int2*>(base2 + o_rows);
+  d.tabs.px_terms = reinterpret_cast<int4*>(d.base + o_terms);
   d.tabs.rmap = reinterpret_cast<int*>(d.base + o_rmap);
+  d.tabs.rdeg = reinterpret_cast<int*>(base2 + o_rdeg);
   d.tabs.rnorm = reinterpret_cast<double*>(d.base + o_rnorm);
   d.tabs.rot_ptr = reinterpret_cast<int*>(d.base + o_rotptr);
   d.tabs.rot_terms = reinterpret_cast<GTerm*>(d.base + o_rotterms);

@@ -338,6 +338,12 @@ void build_tables(Tables& t) {
       boff += km + 1;
     }
   }
+  t.rdeg.resize(t.rmap.size());
+  for (size_t e = 0; e < t.rmap.size(); ++e) {
+    int L = 0;
+    while ((L + 1) * (L + 1) <= (t.rmap[e] & 0xfff)) ++L;
+    t.rdeg[e] = L + 2 * (t.rmap[e] >> 24);
+  }
   t.rnorm.resize(t.rmap.size());
   for (size_t e = 0; e < t.rmap.size(); ++e) t.rnorm[e] = harm_coef_host().n[t.rmap[e] & 0xfff];
   build_deriv_tables(t);
@@ -435,6 +441,15 @@ void build_tables(Tables& t) {
   t.g_rowinfo.clear();
   t.g_grp.clear();
   t.g_terms.clear();
+  t.rt_base.assign(kNumClasses + 1, 0);
+  t.rt_src.clear();
+  t.px_rows.clear();
+  t.px_terms.clear();
+  t.axial.assign((size_t)(kLmax + 1) * (kLmax + 1) * (kLmax + 1), 0.0);
+  for (int l = 0; l <= kLmax; ++l)
+    for (int l1 = 0; l1 <= l; ++l1)
+      for (int m = 0; m <= l1; ++m)
+        t.axial[(size_t)l * (kLmax + 1) * (kLmax + 1) + l1 * (l + 1) + m] = translation_real(l, m, l1, m, 0);
   for (int la = 0; la <= kLmax; ++la)
     for (int lb = 0; lb <= la; ++lb) {
       const int cid = class_id(la, lb), lam = la + lb;
@@ -478,6 +493,7 @@ void build_tables(Tables& t) {
             t.g_terms.push_back(gt);
           }
         local += 32 * K;
+        t.px_terms.resize(t.g_terms.size(), make_int4(0, 0, 0, 0));
         for (int i = 0; i < 32; ++i) {
           if (g0 + i >= nW) {
             t.g_rowinfo.push_back(-1);
@@ -489,6 +505,35 @@ void build_tables(Tables& t) {
           while ((l2 + 1) * (l2 + 1) <= i2) ++l2;
           t.g_rowinfo.push_back((i1 * ws + i2) | (l1 << 16) | (l2 << 20));
           t.g_nnz[cid] += (int)row_terms(e).size();
+        }
+      }
+      // the pair kernel's form: contracted entries (l1 l2 by l1 l2) and the rows reading them, in fixed point
+      {
+        t.rt_base[cid] = (int)t.rt_src.size();
+        std::vector<std::vector<int>> at((size_t)(la + 1) * (lb + 1));  // per (l1, l2): contracted entry by R' index
+        for (int l1 = 0; l1 <= la; ++l1)
+          for (int l2 = 0; l2 <= lb; ++l2) {
+            auto& where = at[l1 * (lb + 1) + l2];
+            where.assign(n_r(lam), -1);
+            for (int L = std::abs(l1 - l2); L <= l1 + l2; L += 2)
+              for (int M = -L; M <= L; ++M) {
+                const int r = ridx(L, M, (l1 + l2 - L) / 2);
+                where[r] = (int)t.rt_src.size() - t.rt_base[cid];
+                t.rt_src.push_back(r | (l1 * (lb + 1) + l2) << 16);
+              }
+          }
+        t.rt_base[cid + 1] = (int)t.rt_src.size();
+        for (int r = 0; r < nrp; ++r) {
+          const int info = t.g_rowinfo[t.g_rowbase[cid] + r], g = t.g_grpbase[cid] + r / 32, K = t.g_grp[2 * g + 1];
+          const int first = t.g_grp[2 * g] + r % 32, l1 = (info >> 16) & 15, l2 = (info >> 20) & 15;
+          t.px_rows.push_back(make_int2((info < 0 ? 0xffff : info & 0xffff) | K << 16, first));
+          for (int j = 0; j < K; ++j) {
+            const GTerm& gt = t.g_terms[t.g_termbase[cid] + first + 32 * j];
+            const long long q = std::llrint(std::ldexp(gt.coef, 58));  // limbs as in shgo_fixed.cuh
+            const long long lo = (long long)((unsigned long long)q << 35) >> 35;
+            int4& x = t.px_terms[t.g_termbase[cid] + first + 32 * j];
+            x = make_int4((int)((q - lo) >> 29), (int)lo, gt.coef != 0.0 ? at[l1 * (lb + 1) + l2][gt.ridx] : 0, gt.ridx);
+          }
         }
       }
       // transposed program: for each R' entry, the (coefficient, W entry, l1 l2) pairs feeding it
