@@ -124,6 +124,11 @@ struct Tables {
   std::vector<int> c2_ptr;
   std::vector<GTerm> c2_terms;
   std::vector<int> c2_base;  // [n classes]
+  // The lists of a class as rows for a warp (overlap, two-centre Coulomb): cx_rows from cx_base[2 c] on = (block entry, or
+  // 0xffff for padding, | term count << 16, first term), terms from cx_base[2 c + 1] on, 32 apart within a row.
+  std::vector<int2> cx_rows;
+  std::vector<GTerm> cx_terms;
+  std::vector<int> cx_base;
   std::vector<double> c2_a;
   // Derivative integrals (shgo_deriv.cu).  For each Lambda <= kLamMax the coupling block of Lambda + 1
   // serves the class: d_map0 maps each entry (L, M, k) of the Lambda layout, d_mapm each entry of the
@@ -201,6 +206,8 @@ struct DeviceTables {
   int* c2_ptr = nullptr;
   GTerm* c2_terms = nullptr;
   double* c2_a = nullptr;
+  int2* cx_rows = nullptr;
+  GTerm* cx_terms = nullptr;
   double* eri_eps = nullptr;  // Tables::eri_eps
   int* c2_cbase = nullptr;    // Tables::c2_base (first c2_ptr entry of each class)
   float2* boys_ff = nullptr;  // boys as (hi, lo) FP32 pairs

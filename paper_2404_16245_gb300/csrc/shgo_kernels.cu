@@ -267,6 +267,8 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = upload(&d.c2_ptr, t.c2_ptr);
   if (e == cudaSuccess) e = upload(&d.c2_terms, t.c2_terms);
   if (e == cudaSuccess) e = upload(&d.c2_a, t.c2_a);
+  if (e == cudaSuccess) e = upload(&d.cx_rows, t.cx_rows);
+  if (e == cudaSuccess) e = upload(&d.cx_terms, t.cx_terms);
   if (e == cudaSuccess) e = upload(&d.eri_eps, t.eri_eps);
   if (e == cudaSuccess) e = upload(&d.c2_cbase, t.c2_base);
   if (e == cudaSuccess) e = upload(&d.boys_ff, boys_table_pairs(t.boys));

@@ -382,6 +382,32 @@ void build_tables(Tables& t) {
         }
       t.c2_ptr.push_back((int)t.c2_terms.size());
     }
+  // the same lists as rows for a warp: sorted by term count, in groups of 32, terms interleaved
+  t.cx_base.assign(2 * kNumClasses, 0);
+  for (int la = 0; la <= kLmax; ++la)
+    for (int lb = 0; lb <= la; ++lb) {
+      const int cid = class_id(la, lb), n = (2 * la + 1) * (2 * lb + 1);
+      const int* ptr = t.c2_ptr.data() + t.c2_base[cid];
+      t.cx_base[2 * cid] = (int)t.cx_rows.size();
+      t.cx_base[2 * cid + 1] = (int)t.cx_terms.size();
+      std::vector<int> order(n);
+      for (int e = 0; e < n; ++e) order[e] = e;
+      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return ptr[x + 1] - ptr[x] > ptr[y + 1] - ptr[y]; });
+      for (int g0 = 0; g0 < n; g0 += 32) {
+        const int K = ptr[order[g0] + 1] - ptr[order[g0]], first = (int)t.cx_terms.size() - t.cx_base[2 * cid + 1];
+        t.cx_terms.resize(t.cx_terms.size() + 32 * (size_t)K, GTerm{0.0, 0, 0});
+        for (int i = 0; i < 32; ++i) {
+          t.cx_rows.push_back(make_int2((g0 + i < n ? order[g0 + i] : 0xffff) | K << 16, first + i));
+          if (g0 + i >= n) continue;
+          const int e = order[g0 + i], m = ptr[e + 1] - ptr[e];
+          for (int j = 0; j < K; ++j) {  // padding: zero times the row's own first value
+            GTerm g = t.c2_terms[ptr[e] + (j < m ? j : 0)];
+            if (j >= m) g.coef = 0.0;
+            t.cx_terms[t.cx_base[2 * cid + 1] + first + i + 32 * (size_t)j] = g;
+          }
+        }
+      }
+    }
   t.c2_a.assign((size_t)(kLamMax + 1) * (kC2K + 1) * (kC2K + 1), 0.0);
   for (int L = 0; L <= kLamMax; ++L) {
     // a_{0,0} = 1; Delta_L (u^j f^{(n)}) = (4j^2 + (4L + 2) j) u^{j-1} f^{(n)} + (8j + 4L + 6) u^j f^{(n+1)}

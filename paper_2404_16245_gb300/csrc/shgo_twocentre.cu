@@ -23,8 +23,9 @@
 // harmonics once per pair of centres; a warp per shell pair is left with one product per (L, M) and one multiply-add per
 // coupling coefficient, about five per element.
 //
-// Measured (GB300, 32 atoms with l <= 6, 25,200 shell pairs): (a|b) 421 -> 86 us against one block per shell pair for all
-// steps, overlap 94 -> 78 us against a warp per pair with D^la diag(d) (D^lb)^T.
+// Measured (GB300, 32 atoms with l <= 6, 25,200 shell pairs): (a|b) 421 -> 63 us against one block per shell pair for all
+// steps, overlap 95 -> 55 us against a warp per pair with D^la diag(d) (D^lb)^T.  Of that, rows of terms read coalesced
+// instead of one list per lane and the harmonics in the radial launch instead of their own: 86 -> 63, 78 -> 55 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -50,6 +51,7 @@ struct PairClasses {  // classes with pairs: class c holds the items [first[c], 
   int n;
   int first[kMaxClasses + 1];
   int pair_base[kMaxClasses];
+  int rows[kMaxClasses], terms[kMaxClasses];  // the class's coupling rows and terms (Tables::cx_base)
   unsigned char la[kMaxClasses], lb[kMaxClasses];
 };
 
@@ -65,17 +67,21 @@ __device__ __forceinline__ int class_of_item(const PairClasses& cls, int item) {
   return c;
 }
 
-// S_LM(n), L <= lam, of the unit vector n = (B - A)/|B - A| (z for A = B) of every ordered pair of centres: one thread
-// per column M.
-__global__ void __launch_bounds__(128) k_site_harmonics(int n_sites, int lam, const double* __restrict__ site_rot,
-                                                        double* __restrict__ S) {
-  const int ncol = 2 * lam + 1, ns = (lam + 1) * (lam + 1);
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)n_sites * ncol;
-       t += (int64_t)gridDim.x * blockDim.x) {
+// S_LM(n), L <= lam, of the unit vector n = (B - A)/|B - A| (z for A = B) of every ordered pair of centres, one thread per
+// column M: the share of block `block` of `blocks`.  The radial launches carry these blocks after their own.
+struct SiteArgs {
+  int n_sites, lam;
+  const double* site_rot;
+  double* S;
+};
+__device__ __forceinline__ void site_harmonics(const SiteArgs& A, int block, int blocks) {
+  const int lam = A.lam, ncol = 2 * lam + 1, ns = (lam + 1) * (lam + 1);
+  for (int64_t t = block * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)A.n_sites * ncol;
+       t += (int64_t)blocks * blockDim.x) {
     const int64_t site = t / ncol;
     const int m = (int)(t - site * ncol) - lam, am = m < 0 ? -m : m;
-    const double x = site_rot[9 * site + 6], y = site_rot[9 * site + 7], z = site_rot[9 * site + 8];
-    double* o = S + site * ns;
+    const double x = A.site_rot[9 * site + 6], y = A.site_rot[9 * site + 7], z = A.site_rot[9 * site + 8];
+    double* o = A.S + site * ns;
     double sp = 1.0, sm = 0.0;  // S_{l,l}, S_{l,-l}
     if (am >= 1) {
       sp = x;
@@ -101,7 +107,7 @@ __global__ void __launch_bounds__(128) k_site_harmonics(int n_sites, int lam, co
 }
 
 // Coulomb: X of one primitive pair per thread, X[(q - q0) stride + k], L = la + lb - 2k.
-__global__ void __launch_bounds__(128) k_coulomb_radial(int64_t q0, int64_t n, int stride, const int* __restrict__ pp_pair,
+__global__ void __launch_bounds__(128) k_coulomb_radial(int own, SiteArgs sites, int64_t q0, int64_t n, int stride, const int* __restrict__ pp_pair,
                                                         const int* __restrict__ pp_ij, const int* __restrict__ pair_a,
                                                         const int* __restrict__ pair_b,
                                                         const double* __restrict__ shell_xyz,
@@ -111,7 +117,11 @@ __global__ void __launch_bounds__(128) k_coulomb_radial(int64_t q0, int64_t n, i
                                                         const double* __restrict__ prim_coef,
                                                         const double* __restrict__ boys_tab,
                                                         const double* __restrict__ c2_a, double* __restrict__ X) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  if (blockIdx.x >= own) {
+    site_harmonics(sites, blockIdx.x - own, gridDim.x - own);
+    return;
+  }
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)own * blockDim.x) {
     const int pr = pp_pair[q0 + i], ij = pp_ij[q0 + i], a = pair_a[pr], b = pair_b[pr];
     const int la = shell_l[a], lb = shell_l[b], lam = la + lb;
     const int ia = shell_poff[a] + (ij >> 8), ib = shell_poff[b] + (ij & 255);
@@ -148,15 +158,19 @@ __global__ void __launch_bounds__(128) k_coulomb_radial(int64_t q0, int64_t n, i
 }
 
 // Overlap: X of one shell pair per thread, X[item stride + j], L = la + lb - 2j.
-__global__ void __launch_bounds__(128) k_overlap_radial(PairClasses cls, int stride, const int* __restrict__ pair_a,
+__global__ void __launch_bounds__(128) k_overlap_radial(int own, SiteArgs sites, PairClasses cls, int stride, const int* __restrict__ pair_a,
                                                         const int* __restrict__ pair_b,
                                                         const int64_t* __restrict__ pair_ppoff,
                                                         const int* __restrict__ pair_site, int64_t rot_per,
                                                         const double* __restrict__ rotd,
                                                         const int* __restrict__ shell_nprim,
                                                         const PPData* __restrict__ ppd, double* __restrict__ X) {
+  if (blockIdx.x >= own) {
+    site_harmonics(sites, blockIdx.x - own, gridDim.x - own);
+    return;
+  }
   const int total = cls.first[cls.n];
-  for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < total; item += gridDim.x * blockDim.x) {
+  for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < total; item += own * blockDim.x) {
     const int c = class_of_item(cls, item), la = cls.la[c], lb = cls.lb[c];
     const int pr = cls.pair_base[c] + (item - cls.first[c]);
     const int npp = shell_nprim[pair_a[pr]] * shell_nprim[pair_b[pr]];
@@ -204,8 +218,8 @@ __global__ void __launch_bounds__(32 * kBlockWarps) k_twocentre_blocks(
     PairClasses cls, int lam_max, int stride, bool per_pair, int64_t q0, const int* __restrict__ pair_a,
     const int* __restrict__ pair_b, const int64_t* __restrict__ pair_ppoff, const int* __restrict__ pair_site,
     const int* __restrict__ shell_nprim, const int64_t* __restrict__ shell_foff, const double* __restrict__ S,
-    const double* __restrict__ X, const int* __restrict__ c2_ptr, const int* __restrict__ c2_cbase,
-    const GTerm* __restrict__ c2_terms, MolView mv, double* __restrict__ out) {
+    const double* __restrict__ X, const int2* __restrict__ cx_rows, const GTerm* __restrict__ cx_terms, MolView mv,
+    double* __restrict__ out) {
   extern __shared__ double smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, ns = (lam_max + 1) * (lam_max + 1);
   double* SX = smem + wib * (ns + kLmax + 1);  // [ns] X_L S_LM(n)
@@ -231,23 +245,29 @@ __global__ void __launch_bounds__(32 * kBlockWarps) k_twocentre_blocks(
       for (int m = lane; m <= 2 * L; m += 32) SX[L * L + m] = Sp[L * L + m] * x;
     }
     __syncwarp();
-    const int* ptr = c2_ptr + c2_cbase[la * (la + 1) / 2 + lb];
+    const int2* rows = cx_rows + cls.rows[c];
+    const GTerm* terms = cx_terms + cls.terms[c];
     const int na = 2 * la + 1, nb = 2 * lb + 1;
     const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
     int64_t obase, ld;
     mol_output(mv, pr, obase, ld);
     double* o = out + obase;
-    for (int e = lane; e < na * nb; e += 32) {
-      const int ma = e / nb, mb = e - ma * nb;
-      // a diagonal block takes the entry below its diagonal from the terms of the one above it: exactly symmetric
-      const int es = a == b && ma > mb ? mb * nb + ma : e;
+    // a diagonal block's entries (ma, mb) and (mb, ma) have equal lists: exactly symmetric
+    for (int r = lane; r < ((na * nb + 31) & ~31); r += 32) {
+      const int2 row = __ldg(rows + r);
+      const int K = row.x >> 16, e = row.x & 0xffff;
+      const GTerm* tp = terms + row.y;
       double v = 0.0;
-      for (int t = ptr[es]; t < ptr[es + 1]; ++t) {
-        const GTerm g = c2_terms[t];
+#pragma unroll 4
+      for (int j = 0; j < K; ++j) {
+        const GTerm g = tp[32 * j];
         v = fma(g.coef, SX[g.ridx], v);
       }
-      o[(fa0 + ma) * ld + fb0 + mb] = v;
-      if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = v;
+      if (e != 0xffff) {
+        const int ma = e / nb, mb = e - ma * nb;
+        o[(fa0 + ma) * ld + fb0 + mb] = v;
+        if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = v;
+      }
     }
   }
 }
@@ -297,8 +317,10 @@ shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTa
     return SHGO_ERR_OOM;
   }
   double *S = buf, *X = buf + (size_t)db.n_sites * ns;
-  k_site_harmonics<<<grid_cap_sm(((int64_t)db.n_sites * (2 * lam_max + 1) + 127) / 128, 16), 128, 0, stream>>>(
-      db.n_sites, lam_max, db.site_rot, S);
+  const Tables& th = tables_host();
+  const int site_blocks = grid_cap_sm(((int64_t)db.n_sites * (2 * lam_max + 1) + 127) / 128, 16);
+  const SiteArgs sites{db.n_sites, lam_max, db.site_rot, S};
+  bool first = true;
   for (const std::vector<ClassWork>& piece : pieces) {
     if (piece.empty()) continue;
     PairClasses cls{};
@@ -309,24 +331,28 @@ shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTa
       cls.pair_base[cls.n] = w.pair_base;
       cls.la[cls.n] = (unsigned char)w.la;
       cls.lb[cls.n] = (unsigned char)w.lb;
+      cls.rows[cls.n] = th.cx_base[2 * class_id(w.la, w.lb)];
+      cls.terms[cls.n] = th.cx_base[2 * class_id(w.la, w.lb) + 1];
       ++cls.n;
       total += w.npairs;
       pp += w.npp;
     }
     cls.first[cls.n] = total;
     const int64_t q0 = piece[0].pp_base;
+    const int own = grid_cap_sm(((coulomb ? pp : (int64_t)total) + 127) / 128, 16), more = first ? site_blocks : 0;
+    first = false;
     if (coulomb)
-      k_coulomb_radial<<<grid_cap_sm((pp + 127) / 128, 16), 128, 0, stream>>>(
-          q0, pp, stride, db.pp_pair, db.pp_ij, db.pair_a, db.pair_b, db.shell_xyz, db.shell_l, db.shell_poff, db.prim_exp,
-          db.prim_coef, dt.boys, dt.c2_a, X);
+      k_coulomb_radial<<<own + more, 128, 0, stream>>>(own, sites, q0, pp, stride, db.pp_pair, db.pp_ij, db.pair_a, db.pair_b,
+                                                       db.shell_xyz, db.shell_l, db.shell_poff, db.prim_exp, db.prim_coef,
+                                                       dt.boys, dt.c2_a, X);
     else
-      k_overlap_radial<<<grid_cap_sm(((int64_t)total + 127) / 128, 16), 128, 0, stream>>>(
-          cls, stride, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, rot_block(db.rot_lmax), db.rotd, db.shell_nprim,
-          db.ppd, X);
+      k_overlap_radial<<<own + more, 128, 0, stream>>>(own, sites, cls, stride, db.pair_a, db.pair_b, db.pair_ppoff,
+                                                       db.pair_site, rot_block(db.rot_lmax), db.rotd, db.shell_nprim, db.ppd,
+                                                       X);
     k_twocentre_blocks<<<grid_cap_sm(((int64_t)total + kBlockWarps - 1) / kBlockWarps, 12), 32 * kBlockWarps,
                          sizeof(double) * kBlockWarps * (size_t)(ns + kLmax + 1), stream>>>(
         cls, lam_max, stride, !coulomb, q0, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, db.shell_nprim,
-        db.shell_foff, S, X, dt.c2_ptr, dt.c2_cbase, dt.c2_terms, mv, out);
+        db.shell_foff, S, X, dt.cx_rows, dt.cx_terms, mv, out);
   }
   e = cudaGetLastError();
   cudaFreeAsync(buf, stream);
