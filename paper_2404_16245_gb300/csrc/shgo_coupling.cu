@@ -52,25 +52,51 @@ __device__ double2 g_boys_top[(kLamDer + 1) * kBoysTopRows * kBoysTopStride / 2]
 // the tables large (the warps of a block share them).
 __host__ __device__ constexpr int coupling_warps(int lam) { return lam <= 5 ? 1 : (lam <= 8 ? 2 : 4); }
 
+constexpr int kHalf = 16;         // columns of the harmonic table
+constexpr int kHS = kHalf + 1;   // its row stride: odd, so that 8-byte loads of different rows fall in different banks
+
 template <int LAM>
 struct Shape {
   static constexpr int nS = n_harm(LAM), nB = n_beta(LAM), nR = n_r(LAM), NW = coupling_warps(LAM);
-  static constexpr size_t smem = 8 * (size_t)((nS + nB + 3) * kCS + nR + nS + 4 * nB + (LAM + 1)) +
+  static constexpr size_t smem = 8 * (size_t)(nS * kHS + (nB + 3) * kCS + nR + nS + 4 * nB + (LAM + 1)) +
                                  4 * (size_t)(2 * nB + 2 * (LAM + 1) + 8);
 };
 
-// Column split over NW warps: warp w takes |m| in [column_bound(w), column_bound(w + 1)), the columns' steps evened out
-// (warp 0 starts its share when the radial rows are done, like the others).
+// Column split over NW warps: warp w takes |m| in [column_bound(w), column_bound(w + 1)), the columns' steps evened out.
 __host__ __device__ constexpr int column_bound(int lam, int nw, int w) {
   if (w <= 0) return 0;
   if (w >= nw) return lam + 1;
-  const int total = (lam + 1) * (lam + 1);
+  const int total = (lam + 1) * (lam + 2) / 2;
   int m = 0, acc = 0;
-  while (m <= lam && nw * (acc + (lam - m + 1) * (m ? 2 : 1) / 2) < w * total) {
-    acc += (lam - m + 1) * (m ? 2 : 1);
-    ++m;
-  }
+  while (m <= lam && nw * (acc + (lam - m + 1) / 2) < w * total) acc += lam - m++ + 1;
   return m;
+}
+
+// Columns m = am (neg: -am), am in [A0, A1), of V_lm into rows h of St at column c: the two signs on the two halves of a
+// warp, so that 16 nuclei fill it.
+template <int LAM>
+__device__ __forceinline__ void harmonic_half(int A0, int A1, int set, bool neg, fx x, fx y, fx z, int2* St, int c) {
+  fx dp = {1 << kFxLimb, 0}, dm = {0, 0};  // (x + iy)^am
+  const fx ny = fx_neg(y);
+#pragma unroll 1
+  for (int am = 0; am < A1; ++am) {
+    if (am >= A0) {
+      fx v0 = {0, 0}, v1 = neg ? dm : dp;
+      const int sm = neg ? -am : am;
+#pragma unroll 1
+      for (int l = am;; ++l) {
+        if (!neg || am) St[(l * l + l + sm) * kHS + c] = make_int2(v1.h, v1.l);
+        if (l == LAM) break;
+        const int4 s = k_step[set + l * (l + 1) / 2 + am];
+        const fx vn = fx_step(fx{z.h << s.z, z.l << s.z}, v1, s.x, s.y, v0);
+        v0 = v1;
+        v1 = vn;
+      }
+    }
+    const fx t = fx_step(x, dp, ny.h, ny.l, dm);
+    dm = fx_step(y, dp, x.h, x.l, dm);
+    dp = t;
+  }
 }
 
 template <int LAM>
@@ -78,12 +104,12 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
   using Sh = Shape<LAM>;
   constexpr int NW = Sh::NW, NT = 32 * NW, nS = Sh::nS, nB = Sh::nB, nR = Sh::nR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  int2* St = reinterpret_cast<int2*>(smem_raw);             // [nS] harmonic rows
-  int2* Bt = St + nS * kCS;                                  // [nB] radial rows (axis columns: doubles)
+  int2* St = reinterpret_cast<int2*>(smem_raw);             // [nS] harmonic rows of 16 columns
+  int2* Bt = St + nS * kHS;                                  // [nB] radial rows (doubles, then fixed point but on the axis)
   int2* Xt = Bt + nB * kCS;                                  // [3] x, y, z of the columns
-  double* racc = reinterpret_cast<double*>(Xt + 3 * kCS);    // [nR] sums of the chunks so far
-  double* fard = racc + nR;                                  // [nS] far sums of the chunk
-  double* axs = fard + nS;                                   // [nB] axis sums of the chunk
+  double* nacc = reinterpret_cast<double*>(Xt + 3 * kCS);    // [nR] near sums
+  double* fard = nacc + nR;                                  // [nS] far sums
+  double* axs = fard + nS;                                   // [nB] axis sums
   double* sb = axs + nB;                                     // [nB] 2 pi k! p^{-(k+1)-L/2}
   double* cfa = sb + nB;                                     // [nB] a_{L,k}
   double* cfk = cfa + nB;                                    // [nB] 2 pi k!
@@ -108,17 +134,25 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
       cfk[f + k] = g_kfact[k];
     }
   }
-  wq_for_each(A.q, A.npp, s_next, &s_t0, [&](long long w) {
+  // a block takes A.group consecutive primitive pairs at a time, which mostly share their shell pair: the nuclei's
+  // pair-frame coordinates (13 of some 80 FP64 instructions at small Lambda) are then formed once for the shell pair
+  WorkQueue groups = A.q;
+  groups.items = nullptr;
+  wq_for_each(groups, (A.npp + A.group - 1) / A.group, s_next, &s_t0, [&](long long g) {
+   double gx = 0.0, gy = 0.0, gz = 0.0, gq = 0.0;  // coordinates and charge of nucleus `lane` for shell pair gpr
+   int gpr = -1;
+   for (int64_t i = g * A.group; i < min(A.npp, (int64_t)(g + 1) * A.group); ++i) {
+    const int64_t w = A.q.items ? A.q.items[i] : i;
     const int64_t q = A.pp_base + w;
     const int pr = A.pp_pair[q];
     const PPData pd = A.ppd[q];
     // primitive pairs with a zero prefactor (K_AB of Eq. 5 underflowed, or the pair is below the per-basis bound) are
     // skipped by the pair kernel too, so their coupling block is not needed
-    if (pd.pref == 0.0) return;
+    if (pd.pref == 0.0) continue;
     const double ip = pd.sp * pd.rp;  // p^{-1/2}
     int64_t cbeg, ncen;
     mol_centers(A.mv, pr, cbeg, ncen);
-    double* out = A.rbuf + A.rbase + w * (int64_t)nR;
+    bool havenear = false, havefar = false;
     for (int64_t c0 = 0; c0 < ncen || c0 == 0; c0 += kNch) {
       __syncthreads();  // the tables of the previous chunk (or primitive pair) are consumed
       if (wid == NW - 1 && c0 == 0 && lane <= LAM) {  // p^{-1-j/2}, lane = j
@@ -132,14 +166,19 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
       }
       if (wid == 0) {
         const bool valid = c0 + lane < ncen;
-        double dx = 0.0, dy = 0.0, zp = 0.0, Z = 0.0;
-        if (valid) {
-          const int64_t c = mol_center_index(A.mv, cbeg + c0 + lane);
-          // C - P = (C - A) - (beta/p)(B - A), in the pair frame where B - A is along z
-          frame_coords(A.site_rot + 9 * (int64_t)A.pair_site[pr], A.shell_xyz + 3 * (int64_t)A.pair_a[pr],
-                       A.centers + 3 * c, dx, dy, zp);
-          Z = A.charges[c];
+        if (pr != gpr || ncen > kNch) {
+          gx = gy = gz = gq = 0.0;
+          if (valid) {
+            const int64_t c = mol_center_index(A.mv, cbeg + c0 + lane);
+            // C - P = (C - A) - (beta/p)(B - A), in the pair frame where B - A is along z
+            frame_coords(A.site_rot + 9 * (int64_t)A.pair_site[pr], A.shell_xyz + 3 * (int64_t)A.pair_a[pr],
+                         A.centers + 3 * c, gx, gy, gz);
+            gq = A.charges[c];
+          }
+          gpr = pr;
         }
+        const double dx = gx, dy = gy, zp = gz;
+        double Z = gq;
         const double dz = zp - pd.shift;
         const double rho2 = fma(dy, dy, dx * dx), s2 = fma(dz, dz, rho2), T = pd.p * s2;
         const int hs = __double2hiint(s2);
@@ -184,7 +223,6 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
         radial_factors<LAM>(near, T, pd.sp * (s2 * ri), ri * ip, Z,
                             g_boys_top + (size_t)LAM * kBoysTopRows * (kBoysTopStride / 2), G, tau);
         const bool anynear = (mn | an) != 0u;
-        const bool wr = near ? valid : false;
         const int sgn = uz < 0.0 ? (int)0x80000000 : 0;
         int bo = 0;
 #pragma unroll
@@ -196,36 +234,45 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
             if (k > 0) acc = fma(tau[k], G[L + k], acc);
             const unsigned ha = (unsigned)__double2hiint(acc) & 0x7fffffffu;
             const int En = (int)(__reduce_max_sync(~0u, near && off ? ha : 0u) >> 20);
-            int E = En;
             if (k == 0) {
               const int Ef = (int)(__reduce_max_sync(~0u, !near && off ? ha : 0u) >> 20);
-              if (!near) E = Ef;
               if (lane == 0) ef[L] = Ef;
             }
             if (lane == 0) en[bo + k] = En;
-            if (valid && (wr || k == 0)) {
-              int2 v;
-              if (axis) {  // U_L0(0, 0, +-1) N_L0 = (+-1)^L
-                v = make_int2(__double2loint(acc), __double2hiint(acc) ^ ((L & 1) ? sgn : 0));
-              } else {
-                const fx b = fx_of(acc, E + 2);  // below 2^57: the sums of 32 products stay inside 64 bits
-                v = make_int2(b.h, b.l);
-              }
-              Bt[(bo + k) * kCS + pos] = v;
-            }
+            // U_L0(0, 0, +-1) N_L0 = (+-1)^L on the axis
+            if (valid && (near || k == 0))
+              Bt[(bo + k) * kCS + pos] =
+                  make_int2(__double2loint(acc), __double2hiint(acc) ^ (axis && (L & 1) ? sgn : 0));
           }
           bo += (LAM - L) / 2 + 1;
         }
       }
       __syncthreads();
       const int n1 = cnt[0], n2 = cnt[1], n3 = cnt[2], n4 = cnt[3], er = cnt[4];
-      if (lane < n2) {
-        const int2 a = Xt[lane], b = Xt[kCS + lane], c = Xt[2 * kCS + lane];
-        harmonic_columns<LAM>(A0, A1, er < 0 ? kSteps : 0, fx{a.x, a.y}, fx{b.x, b.y}, fx{c.x, c.y}, St, lane);
+      const int set = er < 0 ? kSteps : 0, col = lane & (kHalf - 1);
+      const int* rowcode = g_row + (er < 0 ? kRows : 0);
+      auto columns = [&](int h0) {
+        const int c = h0 + col;
+        if (c < n2) {
+          const int2 a = Xt[c], b = Xt[kCS + c], z = Xt[2 * kCS + c];
+          harmonic_half<LAM>(A0, A1, set, lane >= kHalf, fx{a.x, a.y}, fx{b.x, b.y}, fx{z.x, z.y}, St, col);
+        }
+      };
+      // radial rows into fixed point, lane = column
+      for (int b = wid; b < nB; b += NW) {
+        const int L = blk[b] & 0xff;
+        const bool lead = b == b0[L];
+        if (lane < n1 || (lead && lane < n2)) {
+          int2* v = Bt + b * kCS + lane;
+          // below 2^57: the sums of 16 products stay inside 64 bits
+          const fx f = fx_of(__hiloint2double(v->y, v->x), (lane < n1 ? en[b] : ef[L]) + 2);
+          *v = make_int2(f.h, f.l);
+        }
       }
+      columns(0);
       // axis sums of the radial rows and the rows' scales
       for (int b = tid; b < nB; b += NT) {
-        double s = 0.0;
+        double s = c0 == 0 ? 0.0 : axs[b];
         for (int c = n2; c < n3; ++c) {
           const int2 v = Bt[b * kCS + c];
           s += __hiloint2double(v.y, v.x);
@@ -240,53 +287,65 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
         if (c0 == 0) sb[b] = cfk[b] * pw[blk[b] >> 8];
       }
       __syncthreads();
-      const int* rowcode = g_row + (er < 0 ? kRows : 0);
-      if (n1 < n2) {
-        for (int h = tid; h < nS; h += NT) {
-          const int code = __ldg(rowcode + h), L = code >> 16;
-          const int2 *s = St + h * kCS, *b = Bt + b0[L] * kCS;
-          long long hh = 0, mid = 0;
-#pragma unroll 4
-          for (int c = n1; c < n2; ++c) {
-            const int2 u = s[c], v = b[c];
-            hh = fx_mad(u.x, v.x, hh);
-            mid = fx_mad(u.x, v.y, mid);
-            mid = fx_mad(u.y, v.x, mid);
-          }
-          const int E = ef[L];
-          fard[h] = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                               : fx_double(fx_sum(hh, mid), E + 2 - 1023 - kFxBits + er * (code & 0xff) - ((code >> 8) & 0xff));
+      for (int h0 = 0; h0 < n2; h0 += kHalf) {
+        if (h0 > 0) {
+          __syncthreads();  // the first half's harmonics are consumed
+          columns(h0);
+          __syncthreads();
         }
-        __syncthreads();
-      }
-      const bool first = c0 == 0, last = c0 + kNch >= ncen;
-      for (int e = tid; e < nR; e += NT) {
-        const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
-        const int rc = __ldg(rowcode + h);
-        double v = 0.0;
-        if (n1 > 0) {
-          const int2 *s = St + h * kCS, *r = Bt + b * kCS;
-          long long hh = 0, mid = 0;
+        const int hn = min(n1, h0 + kHalf), hf = min(n2, h0 + kHalf), f0 = max(n1, h0);
+        if (f0 < hf) {
+          for (int h = tid; h < nS; h += NT) {
+            const int code = __ldg(rowcode + h), L = code >> 16;
+            const int2 *s = St + h * kHS - h0, *b = Bt + b0[L] * kCS;
+            long long hh = 0, mid = 0;
 #pragma unroll 4
-          for (int c = 0; c < n1; ++c) {
-            const int2 u = s[c], x = r[c];
-            hh = fx_mad(u.x, x.x, hh);
-            mid = fx_mad(u.x, x.y, mid);
-            mid = fx_mad(u.y, x.x, mid);
+            for (int c = f0; c < hf; ++c) {
+              const int2 u = s[c], v = b[c];
+              hh = fx_mad(u.x, v.x, hh);
+              mid = fx_mad(u.x, v.y, mid);
+              mid = fx_mad(u.y, v.x, mid);
+            }
+            const int E = ef[L];
+            const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                        : fx_double(fx_sum(hh, mid),
+                                                    E + 2 - 1023 - kFxBits + er * (code & 0xff) - ((code >> 8) & 0xff));
+            fard[h] = havefar ? fard[h] + v : v;
           }
-          const int E = en[b];
-          v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                         : fx_double(fx_sum(hh, mid), E + 2 - 1023 - kFxBits + er * (rc & 0xff) - ((rc >> 8) & 0xff));
+          havefar = true;
         }
-        if (n1 < n2) v = fma(fard[h], cfa[b], v);
-        v = fma(v, __ldg(A.rnorm + e), (rc & 0xff) == 0 ? axs[b] : 0.0);
-        if (!first) v += racc[e];
-        if (last)
-          out[e] = v * sb[b];
-        else
-          racc[e] = v;
+        if (h0 < hn) {
+          for (int e = tid; e < nR; e += NT) {
+            const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
+            const int rc = __ldg(rowcode + h);
+            const int2 *s = St + h * kHS - h0, *r = Bt + b * kCS;
+            long long hh = 0, mid = 0;
+#pragma unroll 4
+            for (int c = h0; c < hn; ++c) {
+              const int2 u = s[c], x = r[c];
+              hh = fx_mad(u.x, x.x, hh);
+              mid = fx_mad(u.x, x.y, mid);
+              mid = fx_mad(u.y, x.x, mid);
+            }
+            const int E = en[b];
+            const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                        : fx_double(fx_sum(hh, mid),
+                                                    E + 2 - 1023 - kFxBits + er * (rc & 0xff) - ((rc >> 8) & 0xff));
+            nacc[e] = havenear ? nacc[e] + v : v;
+          }
+          havenear = true;
+        }
       }
     }
+    __syncthreads();
+    double* out = A.rbuf + A.rbase + w * (int64_t)nR;
+    for (int e = tid; e < nR; e += NT) {
+      const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
+      double v = havenear ? nacc[e] : 0.0;
+      if (havefar) v = fma(fard[h], cfa[b], v);
+      out[e] = fma(v, __ldg(A.rnorm + e), (__ldg(g_row + h) & 0xff) == 0 ? axs[b] : 0.0) * sb[b];
+    }
+   }
   });
 }
 
@@ -326,9 +385,14 @@ cudaError_t boys_top_table(int lam, const double2** out) {
   return e;
 }
 
-cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, int grid, cudaStream_t stream) {
+cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, cudaStream_t stream) {
   if (lam < 0 || lam > kLamDer) return cudaErrorInvalidValue;
-  kernel_at(lam, Lams{})<<<grid, 32 * coupling_warps(lam), smem_at(lam, Lams{}), stream>>>(args);
+  // up to 32 one-warp blocks per SM (the block limit), half of it where a block has two or four warps; primitive pairs
+  // are taken four at a time once that leaves every SM eight rounds or more (no result depends on it)
+  const int nw = coupling_warps(lam), per_sm = nw == 1 ? 32 : 16;
+  CouplingArgs a = args;
+  a.group = args.npp >= (int64_t)152 * per_sm * 8 ? 4 : 1;
+  kernel_at(lam, Lams{})<<<grid_cap_sm((args.npp + a.group - 1) / a.group, per_sm), 32 * nw, smem_at(lam, Lams{}), stream>>>(a);
   return cudaGetLastError();
 }
 

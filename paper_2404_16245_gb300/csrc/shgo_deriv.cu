@@ -674,7 +674,7 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
       ca.pair_site = db.pair_site;
       ca.ppd = db.ppd;
       ca.rbuf = r1buf;
-      e = launch_coupling_fp64(lam1, ca, grid_cap_sm(w.npp, 16), s);
+      e = launch_coupling_fp64(lam1, ca, s);
       if (e != cudaSuccess) break;
     }
     DerivArgs& d = P.d;

@@ -556,6 +556,7 @@ struct CouplingArgs {
   const float2* exp_ff = nullptr;
   const int* items = nullptr;         // work items of this Lambda (coupling_f32_items)
   const float2* rnorm_ff = nullptr;   // rnorm of this Lambda as (hi, lo) pairs
+  int group = 1;                      // FP64 kernel: consecutive primitive pairs a block takes at a time
   int small_blocks_ok = 0;            // small Lambda may run blocks of two warps (DeviceBasis::f32_small_blocks)
 };
 // Arguments of the pair kernel for one class (shgo_pair.cu).
@@ -584,8 +585,8 @@ struct PairArgs {
 cudaError_t launch_pair_block(const PairArgs& args, int grid, cudaStream_t stream);
 cudaError_t pair_block_setup();
 
-// Launches the Lambda = lam instantiation on `grid` blocks.
-cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, int grid, cudaStream_t stream);
+// Launches the Lambda = lam instantiation.
+cudaError_t launch_coupling_fp64(int lam, const CouplingArgs& args, cudaStream_t stream);
 // Constants and launch attributes of the FP64 coupling kernels on the current device, and of the potential's.
 cudaError_t coupling_fp64_setup();
 cudaError_t esp_fp64_setup();

@@ -446,7 +446,7 @@ struct Launcher {
       launch_coupling_f32(lam, db.precision == SHGO_PREC_FP32_BULK, a, grid_cap(w.npp, 8), s);
       return;
     }
-    launch_coupling_fp64(lam, a, grid_cap(w.npp, 16), s);
+    launch_coupling_fp64(lam, a, s);
   }
   void pair(const ClassWork& w, size_t c, int64_t rbase, cudaStream_t s) const {
     if (w.npairs == 0) return;
