@@ -42,10 +42,12 @@ FP64_DFMA_PER_CLK = 304
 # DRAM traffic of the coupling phase of one V of this workload (dram__bytes_read.sum +
 # dram__bytes_write.sum over the 28 coupling launches of one call, from an ncu capture of the current
 # kernel), or None while no capture of the current kernel exists.
-COUPLING_DRAM_BYTES_PER_V = 8.25e6
-COUPLING_DRAM_NOTE = ("dram__bytes_read.sum + dram__bytes_write.sum summed over the 28 k_coupling_fp64 launches of "
-                      "one V (8.25 MB read, 0 B written: the coupling blocks stay in L2), "
-                      "profiles/k_coupling_fp64_traffic_highl_fp64.md")
+COUPLING_DRAM_BYTES_PER_V = None
+COUPLING_DRAM_NOTE = "no capture of the current coupling kernel"
+# The model counts the method's operations as FP64 ones; most of them run as 58-bit fixed point on the integer pipe.
+FIXED_POINT_NOTE = ("algorithmic operations over the FP64 pipe's rate: the harmonics, nucleus sums and Clebsch-Gordan sums "
+                    "run as 58-bit fixed point on the integer pipe and far nuclei skip the Boys values, so the fraction "
+                    "may exceed 1; every operation of the model is done or shown not to be needed to 2^-56")
 
 
 def fp64_peak_tflops(sm_mhz: float) -> float:
@@ -384,7 +386,7 @@ def run_shgo(args, ws, rank, local):
         roofline = {"bound": "alu", "kernel": names[dom], "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak,
                     "traffic": COUPLING_DRAM_BYTES_PER_V if dom == 0 else None,
-                    "traffic_note": COUPLING_DRAM_NOTE,
+                    "traffic_note": COUPLING_DRAM_NOTE, "model_note": FIXED_POINT_NOTE,
                     "peak_source": "measured in this run: shgo_measure_fma_rate FP64 (DFMA, 2048 threads per SM x "
                                    "8 independent chains, CUDA events), best of 3",
                     "peak_derived_nominal": fp64_peak_tflops(clk), "peak_measurements": pk64}
@@ -636,7 +638,7 @@ def run_esp(args) -> int:
             "config": {"workload": f"potential of a density of the 32-atom l <= 6 basis at {args.points} points",
                        "shell_pairs": npairs, "shell_pair_points_per_s": npairs * args.points / (ms / 1e3),
                        "l2": "flushed between steps (256 MiB write, outside step events)"},
-            "roofline": {"bound": "alu", "kernel": "whole potential call (k_esp_fp64 per class after k_esp_adjoint)",
+            "roofline": {"bound": "alu", "kernel": "whole potential call (k_esp per class after k_esp_adjoint)",
                          "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
                          "model_tflop": [float(fp[0]) / 1e12, float(fp[1]) / 1e12],
                          "peak_source": "shgo_measure_fma_rate in this run (of measured)"},
@@ -687,7 +689,7 @@ def run_overlap(args) -> int:
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": f"overlap of the high-l benchmark basis: {len(b['l'])} shells, {B.nbf} functions",
                        "shell_pairs": B.npairs, "l2": "flushed between steps (256 MiB write, outside step events)"},
-            "roofline": {"bound": "hbm", "kernel": "k_overlap", "achieved": achieved, "peak": hbm,
+            "roofline": {"bound": "hbm", "kernel": "k_twocentre_blocks", "achieved": achieved, "peak": hbm,
                          "unit": "GB/s", "frac": achieved / hbm, "traffic": None,
                          "note": "bytes of the matrix written (both triangles) per step; the inputs are a few KB",
                          "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback 6.8 TB/s"}}
@@ -1144,7 +1146,7 @@ def run_coulomb2c(args) -> int:
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": f"(a|b) of the high-l benchmark basis: {len(b['l'])} shells, {B.nbf} functions",
                        "shell_pairs": npairs, "l2": "flushed between steps (256 MiB write, outside step events)"},
-            "roofline": {"bound": "hbm", "kernel": "k_coulomb2c", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+            "roofline": {"bound": "hbm", "kernel": "k_twocentre_blocks", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": None,
                          "note": "bytes of the matrix written (both triangles) per step; the inputs are a few KB",
                          "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback 6.8 TB/s"}}

@@ -26,12 +26,16 @@
 // 32 x 2^-59 or so of the largest product in it, where an FP64 sum rounds at 2^-53 of its partial sums.
 //
 // Phases of a block (NW warps, one primitive pair at a time): warp 0, lane = nucleus: geometry, kinds, radial rows;
-// all warps, lane = column: harmonic columns m, split by cost; thread = (L, M): sums over the far columns, then
-// thread = R' entry: sums over the near columns, far part, axis part and scales.
+// all warps: the radial rows into fixed point, then for 16 columns at a time (a smaller table, so more blocks on an SM) the
+// harmonics, |m| split over the warps by cost and the two signs of m on the halves of a warp; thread = (L, M): sums over
+// the far columns; thread = R' entry: sums over the near columns, far part, axis part and scales.
 //
 // Measured (GB300, whole calls, against the same kernel with every step in FP64): V of 32 atoms with l <= 6 501 -> 404 us,
 // of a contracted 29-atom molecule 7.00 -> 4.40 ms, of six such molecules in a batch 53.1 -> 29.8 ms; dV/dA of the
-// 32 atoms 1.63 -> 1.50 ms.  Errors against 64-bit quadrature are the same to two digits.
+// 32 atoms 1.63 -> 1.50 ms.  Tables of 32 columns to 16, rows converted by all warps, coordinates kept over a shell pair's
+// primitive pairs (after the pair kernel's contraction): 3.79 -> 3.69 ms, batch 27.6 -> 25.2 ms.  Errors against 64-bit
+// quadrature are the same to two digits.  At Lambda <= 2 the FP64 pipe is 76 % busy (84 % is what plain DFMAs reach), from
+// Lambda 4 on a primitive pair's dependent chains bound it (15 to 20 warps on an SM, FP64 pipe 45 to 55 % busy).
 #include <cuda_runtime.h>
 
 #include <utility>
@@ -139,213 +143,213 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
   WorkQueue groups = A.q;
   groups.items = nullptr;
   wq_for_each(groups, (A.npp + A.group - 1) / A.group, s_next, &s_t0, [&](long long g) {
-   double gx = 0.0, gy = 0.0, gz = 0.0, gq = 0.0;  // coordinates and charge of nucleus `lane` for shell pair gpr
-   int gpr = -1;
-   for (int64_t i = g * A.group; i < min(A.npp, (int64_t)(g + 1) * A.group); ++i) {
-    const int64_t w = A.q.items ? A.q.items[i] : i;
-    const int64_t q = A.pp_base + w;
-    const int pr = A.pp_pair[q];
-    const PPData pd = A.ppd[q];
-    // primitive pairs with a zero prefactor (K_AB of Eq. 5 underflowed, or the pair is below the per-basis bound) are
-    // skipped by the pair kernel too, so their coupling block is not needed
-    if (pd.pref == 0.0) continue;
-    const double ip = pd.sp * pd.rp;  // p^{-1/2}
-    int64_t cbeg, ncen;
-    mol_centers(A.mv, pr, cbeg, ncen);
-    bool havenear = false, havefar = false;
-    for (int64_t c0 = 0; c0 < ncen || c0 == 0; c0 += kNch) {
-      __syncthreads();  // the tables of the previous chunk (or primitive pair) are consumed
-      if (wid == NW - 1 && c0 == 0 && lane <= LAM) {  // p^{-1-j/2}, lane = j
-        double v = pd.rp, b = ip;
+    double gx = 0.0, gy = 0.0, gz = 0.0, gq = 0.0;  // coordinates and charge of nucleus `lane` for shell pair gpr
+    int gpr = -1;
+    for (int64_t i = g * A.group; i < min(A.npp, (int64_t)(g + 1) * A.group); ++i) {
+      const int64_t w = A.q.items ? A.q.items[i] : i;
+      const int64_t q = A.pp_base + w;
+      const int pr = A.pp_pair[q];
+      const PPData pd = A.ppd[q];
+      // primitive pairs with a zero prefactor (K_AB of Eq. 5 underflowed, or the pair is below the per-basis bound) are
+      // skipped by the pair kernel too, so their coupling block is not needed
+      if (pd.pref == 0.0) continue;
+      const double ip = pd.sp * pd.rp;  // p^{-1/2}
+      int64_t cbeg, ncen;
+      mol_centers(A.mv, pr, cbeg, ncen);
+      bool havenear = false, havefar = false;
+      for (int64_t c0 = 0; c0 < ncen || c0 == 0; c0 += kNch) {
+        __syncthreads();  // the tables of the previous chunk (or primitive pair) are consumed
+        if (wid == NW - 1 && c0 == 0 && lane <= LAM) {  // p^{-1-j/2}, lane = j
+          double v = pd.rp, b = ip;
 #pragma unroll
-        for (int bit = 0; (1 << bit) <= LAM; ++bit) {
-          if ((lane >> bit) & 1) v *= b;
-          b *= b;
-        }
-        pw[lane] = v;
-      }
-      if (wid == 0) {
-        const bool valid = c0 + lane < ncen;
-        if (pr != gpr || ncen > kNch) {
-          gx = gy = gz = gq = 0.0;
-          if (valid) {
-            const int64_t c = mol_center_index(A.mv, cbeg + c0 + lane);
-            // C - P = (C - A) - (beta/p)(B - A), in the pair frame where B - A is along z
-            frame_coords(A.site_rot + 9 * (int64_t)A.pair_site[pr], A.shell_xyz + 3 * (int64_t)A.pair_a[pr],
-                         A.centers + 3 * c, gx, gy, gz);
-            gq = A.charges[c];
+          for (int bit = 0; (1 << bit) <= LAM; ++bit) {
+            if ((lane >> bit) & 1) v *= b;
+            b *= b;
           }
-          gpr = pr;
+          pw[lane] = v;
         }
-        const double dx = gx, dy = gy, zp = gz;
-        double Z = gq;
-        const double dz = zp - pd.shift;
-        const double rho2 = fma(dy, dy, dx * dx), s2 = fma(dz, dz, rho2), T = pd.p * s2;
-        const int hs = __double2hiint(s2);
-        if ((hs & 0x7ff00000) == 0x7ff00000) Z = __longlong_as_double(0x7ff8000000000000ll);  // no finite distance
-        double ri = 0.0, ux = 0.0, uy = 0.0, uz = 1.0;
-        if (hs >= kTinyHi) {
-          ri = inverse_distance(s2);
-          ux = dx * ri;
-          uy = dy * ri;
-          uz = dz * ri;
-        }
-        // on the A-B line to within rounding of the rotation: rho below 2^-48 of |z_C - z_A|
-        const int erho = (__double2hiint(rho2) >> 20) & 0x7ff, ezp = (__double2hiint(zp) >> 20) & 0x7ff;
-        const bool axis = hs < 0x7ff00000 && (ri == 0.0 || erho == 0 || erho + 96 + 1023 < 2 * ezp);
-        constexpr double kFar = far_t(LAM);
-        const bool near = __double2hiint(T) < __double2hiint(kFar);
-        const unsigned mn = __ballot_sync(~0u, valid && near && !axis), mf = __ballot_sync(~0u, valid && !near && !axis);
-        const unsigned an = __ballot_sync(~0u, valid && near && axis), af = __ballot_sync(~0u, valid && !near && axis);
-        const int n1 = __popc(mn), n2 = n1 + __popc(mf), n3 = n2 + __popc(an), n4 = n3 + __popc(af);
-        const unsigned below = (1u << lane) - 1u;
-        const int pos = axis ? (near ? n2 + __popc(an & below) : n3 + __popc(af & below))
-                             : (near ? __popc(mn & below) : n1 + __popc(mf & below));
-        // scale of x and y: the power of two of the largest in the chunk
-        const bool off = valid && !axis;
-        const unsigned hxy = max(__double2hiint(ux) & 0x7fffffff, __double2hiint(uy) & 0x7fffffff);
-        const int exy = (int)(__reduce_max_sync(~0u, off ? hxy : 0u) >> 20) - 1023;
-        const int er = exy >= -1 ? 0 : exy + 2;
-        if (off) {
-          const fx fxx = fx_of(ux, 1023 + er), fxy = fx_of(uy, 1023 + er), fxz = fx_of(uz, 1023);
-          Xt[pos] = make_int2(fxx.h, fxx.l);
-          Xt[kCS + pos] = make_int2(fxy.h, fxy.l);
-          Xt[2 * kCS + pos] = make_int2(fxz.h, fxz.l);
-        }
-        if (lane == 0) {
-          cnt[0] = n1;
-          cnt[1] = n2;
-          cnt[2] = n3;
-          cnt[3] = n4;
-          cnt[4] = er;
-        }
-        double G[LAM + 1], tau[LAM / 2 + 1];
-        radial_factors<LAM>(near, T, pd.sp * (s2 * ri), ri * ip, Z,
-                            g_boys_top + (size_t)LAM * kBoysTopRows * (kBoysTopStride / 2), G, tau);
-        const bool anynear = (mn | an) != 0u;
-        const int sgn = uz < 0.0 ? (int)0x80000000 : 0;
-        int bo = 0;
-#pragma unroll
-        for (int L = 0; L <= LAM; ++L) {
-          double acc = G[L];
-#pragma unroll
-          for (int k = 0; k <= (LAM - L) / 2; ++k) {
-            if (k > 0 && !anynear) break;
-            if (k > 0) acc = fma(tau[k], G[L + k], acc);
-            const unsigned ha = (unsigned)__double2hiint(acc) & 0x7fffffffu;
-            const int En = (int)(__reduce_max_sync(~0u, near && off ? ha : 0u) >> 20);
-            if (k == 0) {
-              const int Ef = (int)(__reduce_max_sync(~0u, !near && off ? ha : 0u) >> 20);
-              if (lane == 0) ef[L] = Ef;
+        if (wid == 0) {
+          const bool valid = c0 + lane < ncen;
+          if (pr != gpr || ncen > kNch) {
+            gx = gy = gz = gq = 0.0;
+            if (valid) {
+              const int64_t c = mol_center_index(A.mv, cbeg + c0 + lane);
+              // C - P = (C - A) - (beta/p)(B - A), in the pair frame where B - A is along z
+              frame_coords(A.site_rot + 9 * (int64_t)A.pair_site[pr], A.shell_xyz + 3 * (int64_t)A.pair_a[pr],
+                           A.centers + 3 * c, gx, gy, gz);
+              gq = A.charges[c];
             }
-            if (lane == 0) en[bo + k] = En;
-            // U_L0(0, 0, +-1) N_L0 = (+-1)^L on the axis
-            if (valid && (near || k == 0))
-              Bt[(bo + k) * kCS + pos] =
-                  make_int2(__double2loint(acc), __double2hiint(acc) ^ (axis && (L & 1) ? sgn : 0));
+            gpr = pr;
           }
-          bo += (LAM - L) / 2 + 1;
+          const double dx = gx, dy = gy, zp = gz;
+          double Z = gq;
+          const double dz = zp - pd.shift;
+          const double rho2 = fma(dy, dy, dx * dx), s2 = fma(dz, dz, rho2), T = pd.p * s2;
+          const int hs = __double2hiint(s2);
+          if ((hs & 0x7ff00000) == 0x7ff00000) Z = __longlong_as_double(0x7ff8000000000000ll);  // no finite distance
+          double ri = 0.0, ux = 0.0, uy = 0.0, uz = 1.0;
+          if (hs >= kTinyHi) {
+            ri = inverse_distance(s2);
+            ux = dx * ri;
+            uy = dy * ri;
+            uz = dz * ri;
+          }
+          // on the A-B line to within rounding of the rotation: rho below 2^-48 of |z_C - z_A|
+          const int erho = (__double2hiint(rho2) >> 20) & 0x7ff, ezp = (__double2hiint(zp) >> 20) & 0x7ff;
+          const bool axis = hs < 0x7ff00000 && (ri == 0.0 || erho == 0 || erho + 96 + 1023 < 2 * ezp);
+          constexpr double kFar = far_t(LAM);
+          const bool near = __double2hiint(T) < __double2hiint(kFar);
+          const unsigned mn = __ballot_sync(~0u, valid && near && !axis), mf = __ballot_sync(~0u, valid && !near && !axis);
+          const unsigned an = __ballot_sync(~0u, valid && near && axis), af = __ballot_sync(~0u, valid && !near && axis);
+          const int n1 = __popc(mn), n2 = n1 + __popc(mf), n3 = n2 + __popc(an), n4 = n3 + __popc(af);
+          const unsigned below = (1u << lane) - 1u;
+          const int pos = axis ? (near ? n2 + __popc(an & below) : n3 + __popc(af & below))
+                               : (near ? __popc(mn & below) : n1 + __popc(mf & below));
+          // scale of x and y: the power of two of the largest in the chunk
+          const bool off = valid && !axis;
+          const unsigned hxy = max(__double2hiint(ux) & 0x7fffffff, __double2hiint(uy) & 0x7fffffff);
+          const int exy = (int)(__reduce_max_sync(~0u, off ? hxy : 0u) >> 20) - 1023;
+          const int er = exy >= -1 ? 0 : exy + 2;
+          if (off) {
+            const fx fxx = fx_of(ux, 1023 + er), fxy = fx_of(uy, 1023 + er), fxz = fx_of(uz, 1023);
+            Xt[pos] = make_int2(fxx.h, fxx.l);
+            Xt[kCS + pos] = make_int2(fxy.h, fxy.l);
+            Xt[2 * kCS + pos] = make_int2(fxz.h, fxz.l);
+          }
+          if (lane == 0) {
+            cnt[0] = n1;
+            cnt[1] = n2;
+            cnt[2] = n3;
+            cnt[3] = n4;
+            cnt[4] = er;
+          }
+          double G[LAM + 1], tau[LAM / 2 + 1];
+          radial_factors<LAM>(near, T, pd.sp * (s2 * ri), ri * ip, Z,
+                              g_boys_top + (size_t)LAM * kBoysTopRows * (kBoysTopStride / 2), G, tau);
+          const bool anynear = (mn | an) != 0u;
+          const int sgn = uz < 0.0 ? (int)0x80000000 : 0;
+          int bo = 0;
+#pragma unroll
+          for (int L = 0; L <= LAM; ++L) {
+            double acc = G[L];
+#pragma unroll
+            for (int k = 0; k <= (LAM - L) / 2; ++k) {
+              if (k > 0 && !anynear) break;
+              if (k > 0) acc = fma(tau[k], G[L + k], acc);
+              const unsigned ha = (unsigned)__double2hiint(acc) & 0x7fffffffu;
+              const int En = (int)(__reduce_max_sync(~0u, near && off ? ha : 0u) >> 20);
+              if (k == 0) {
+                const int Ef = (int)(__reduce_max_sync(~0u, !near && off ? ha : 0u) >> 20);
+                if (lane == 0) ef[L] = Ef;
+              }
+              if (lane == 0) en[bo + k] = En;
+              // U_L0(0, 0, +-1) N_L0 = (+-1)^L on the axis
+              if (valid && (near || k == 0))
+                Bt[(bo + k) * kCS + pos] =
+                    make_int2(__double2loint(acc), __double2hiint(acc) ^ (axis && (L & 1) ? sgn : 0));
+            }
+            bo += (LAM - L) / 2 + 1;
+          }
+        }
+        __syncthreads();
+        const int n1 = cnt[0], n2 = cnt[1], n3 = cnt[2], n4 = cnt[3], er = cnt[4];
+        const int set = er < 0 ? kSteps : 0, col = lane & (kHalf - 1);
+        const int* rowcode = g_row + (er < 0 ? kRows : 0);
+        auto columns = [&](int h0) {
+          const int c = h0 + col;
+          if (c < n2) {
+            const int2 a = Xt[c], b = Xt[kCS + c], z = Xt[2 * kCS + c];
+            harmonic_half<LAM>(A0, A1, set, lane >= kHalf, fx{a.x, a.y}, fx{b.x, b.y}, fx{z.x, z.y}, St, col);
+          }
+        };
+        // radial rows into fixed point, lane = column
+        for (int b = wid; b < nB; b += NW) {
+          const int L = blk[b] & 0xff;
+          const bool lead = b == b0[L];
+          if (lane < n1 || (lead && lane < n2)) {
+            int2* v = Bt + b * kCS + lane;
+            // below 2^57: the sums of 16 products stay inside 64 bits
+            const fx f = fx_of(__hiloint2double(v->y, v->x), (lane < n1 ? en[b] : ef[L]) + 2);
+            *v = make_int2(f.h, f.l);
+          }
+        }
+        columns(0);
+        // axis sums of the radial rows and the rows' scales
+        for (int b = tid; b < nB; b += NT) {
+          double s = c0 == 0 ? 0.0 : axs[b];
+          for (int c = n2; c < n3; ++c) {
+            const int2 v = Bt[b * kCS + c];
+            s += __hiloint2double(v.y, v.x);
+          }
+          if (n3 < n4) {
+            const int2* row = Bt + b0[blk[b] & 0xff] * kCS;
+            double f = 0.0;
+            for (int c = n3; c < n4; ++c) f += __hiloint2double(row[c].y, row[c].x);
+            s = fma(f, cfa[b], s);
+          }
+          axs[b] = s;
+          if (c0 == 0) sb[b] = cfk[b] * pw[blk[b] >> 8];
+        }
+        __syncthreads();
+        for (int h0 = 0; h0 < n2; h0 += kHalf) {
+          if (h0 > 0) {
+            __syncthreads();  // the first half's harmonics are consumed
+            columns(h0);
+            __syncthreads();
+          }
+          const int hn = min(n1, h0 + kHalf), hf = min(n2, h0 + kHalf), f0 = max(n1, h0);
+          if (f0 < hf) {
+            for (int h = tid; h < nS; h += NT) {
+              const int code = __ldg(rowcode + h), L = code >> 16;
+              const int2 *s = St + h * kHS - h0, *b = Bt + b0[L] * kCS;
+              long long hh = 0, mid = 0;
+#pragma unroll 4
+              for (int c = f0; c < hf; ++c) {
+                const int2 u = s[c], v = b[c];
+                hh = fx_mad(u.x, v.x, hh);
+                mid = fx_mad(u.x, v.y, mid);
+                mid = fx_mad(u.y, v.x, mid);
+              }
+              const int E = ef[L];
+              const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                          : fx_double(fx_sum(hh, mid),
+                                                      E + 2 - 1023 - kFxBits + er * (code & 0xff) - ((code >> 8) & 0xff));
+              fard[h] = havefar ? fard[h] + v : v;
+            }
+            havefar = true;
+          }
+          if (h0 < hn) {
+            for (int e = tid; e < nR; e += NT) {
+              const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
+              const int rc = __ldg(rowcode + h);
+              const int2 *s = St + h * kHS - h0, *r = Bt + b * kCS;
+              long long hh = 0, mid = 0;
+#pragma unroll 4
+              for (int c = h0; c < hn; ++c) {
+                const int2 u = s[c], x = r[c];
+                hh = fx_mad(u.x, x.x, hh);
+                mid = fx_mad(u.x, x.y, mid);
+                mid = fx_mad(u.y, x.x, mid);
+              }
+              const int E = en[b];
+              const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                          : fx_double(fx_sum(hh, mid),
+                                                      E + 2 - 1023 - kFxBits + er * (rc & 0xff) - ((rc >> 8) & 0xff));
+              nacc[e] = havenear ? nacc[e] + v : v;
+            }
+            havenear = true;
+          }
         }
       }
       __syncthreads();
-      const int n1 = cnt[0], n2 = cnt[1], n3 = cnt[2], n4 = cnt[3], er = cnt[4];
-      const int set = er < 0 ? kSteps : 0, col = lane & (kHalf - 1);
-      const int* rowcode = g_row + (er < 0 ? kRows : 0);
-      auto columns = [&](int h0) {
-        const int c = h0 + col;
-        if (c < n2) {
-          const int2 a = Xt[c], b = Xt[kCS + c], z = Xt[2 * kCS + c];
-          harmonic_half<LAM>(A0, A1, set, lane >= kHalf, fx{a.x, a.y}, fx{b.x, b.y}, fx{z.x, z.y}, St, col);
-        }
-      };
-      // radial rows into fixed point, lane = column
-      for (int b = wid; b < nB; b += NW) {
-        const int L = blk[b] & 0xff;
-        const bool lead = b == b0[L];
-        if (lane < n1 || (lead && lane < n2)) {
-          int2* v = Bt + b * kCS + lane;
-          // below 2^57: the sums of 16 products stay inside 64 bits
-          const fx f = fx_of(__hiloint2double(v->y, v->x), (lane < n1 ? en[b] : ef[L]) + 2);
-          *v = make_int2(f.h, f.l);
-        }
-      }
-      columns(0);
-      // axis sums of the radial rows and the rows' scales
-      for (int b = tid; b < nB; b += NT) {
-        double s = c0 == 0 ? 0.0 : axs[b];
-        for (int c = n2; c < n3; ++c) {
-          const int2 v = Bt[b * kCS + c];
-          s += __hiloint2double(v.y, v.x);
-        }
-        if (n3 < n4) {
-          const int2* row = Bt + b0[blk[b] & 0xff] * kCS;
-          double f = 0.0;
-          for (int c = n3; c < n4; ++c) f += __hiloint2double(row[c].y, row[c].x);
-          s = fma(f, cfa[b], s);
-        }
-        axs[b] = s;
-        if (c0 == 0) sb[b] = cfk[b] * pw[blk[b] >> 8];
-      }
-      __syncthreads();
-      for (int h0 = 0; h0 < n2; h0 += kHalf) {
-        if (h0 > 0) {
-          __syncthreads();  // the first half's harmonics are consumed
-          columns(h0);
-          __syncthreads();
-        }
-        const int hn = min(n1, h0 + kHalf), hf = min(n2, h0 + kHalf), f0 = max(n1, h0);
-        if (f0 < hf) {
-          for (int h = tid; h < nS; h += NT) {
-            const int code = __ldg(rowcode + h), L = code >> 16;
-            const int2 *s = St + h * kHS - h0, *b = Bt + b0[L] * kCS;
-            long long hh = 0, mid = 0;
-#pragma unroll 4
-            for (int c = f0; c < hf; ++c) {
-              const int2 u = s[c], v = b[c];
-              hh = fx_mad(u.x, v.x, hh);
-              mid = fx_mad(u.x, v.y, mid);
-              mid = fx_mad(u.y, v.x, mid);
-            }
-            const int E = ef[L];
-            const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                        : fx_double(fx_sum(hh, mid),
-                                                    E + 2 - 1023 - kFxBits + er * (code & 0xff) - ((code >> 8) & 0xff));
-            fard[h] = havefar ? fard[h] + v : v;
-          }
-          havefar = true;
-        }
-        if (h0 < hn) {
-          for (int e = tid; e < nR; e += NT) {
-            const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
-            const int rc = __ldg(rowcode + h);
-            const int2 *s = St + h * kHS - h0, *r = Bt + b * kCS;
-            long long hh = 0, mid = 0;
-#pragma unroll 4
-            for (int c = h0; c < hn; ++c) {
-              const int2 u = s[c], x = r[c];
-              hh = fx_mad(u.x, x.x, hh);
-              mid = fx_mad(u.x, x.y, mid);
-              mid = fx_mad(u.y, x.x, mid);
-            }
-            const int E = en[b];
-            const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                        : fx_double(fx_sum(hh, mid),
-                                                    E + 2 - 1023 - kFxBits + er * (rc & 0xff) - ((rc >> 8) & 0xff));
-            nacc[e] = havenear ? nacc[e] + v : v;
-          }
-          havenear = true;
-        }
+      double* out = A.rbuf + A.rbase + w * (int64_t)nR;
+      for (int e = tid; e < nR; e += NT) {
+        const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
+        double v = havenear ? nacc[e] : 0.0;
+        if (havefar) v = fma(fard[h], cfa[b], v);
+        out[e] = fma(v, __ldg(A.rnorm + e), (__ldg(g_row + h) & 0xff) == 0 ? axs[b] : 0.0) * sb[b];
       }
     }
-    __syncthreads();
-    double* out = A.rbuf + A.rbase + w * (int64_t)nR;
-    for (int e = tid; e < nR; e += NT) {
-      const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
-      double v = havenear ? nacc[e] : 0.0;
-      if (havefar) v = fma(fard[h], cfa[b], v);
-      out[e] = fma(v, __ldg(A.rnorm + e), (__ldg(g_row + h) & 0xff) == 0 ? axs[b] : 0.0) * sb[b];
-    }
-   }
   });
 }
 

@@ -3,9 +3,9 @@
 // GB300 issues 64 integer multiply-adds (32 x 32 + 64 bits) per clock and SM and 1.7 FP64 ones (measured;
 // shgo_measure_fma_rate for the latter), so a product of two 58-bit numbers formed from three such multiply-adds
 // costs a twelfth of an FP64 one and carries five bits more than its mantissa.  Values are scaled by a power of two
-// to |v| <= 1 and held as q = round(v 2^58) = h 2^29 + l with l in [-2^28, 2^28).  A sum of at most 32 products
-// keeps the partial sums of h h and of h l + l h in one 64-bit accumulator each; the products l l (at most 2^-60 of
-// a full-scale product) are left out.
+// to |v| <= 1 and held as q = round(v 2^58) = h 2^29 + l with l in [-2^28, 2^28).  A sum of at most 35
+// products keeps the partial sums of h h and of h l + l h in one 64-bit accumulator each (32 nuclei, or the 2 Lambda + 1
+// terms of a degree, 35 at Lambda = 17); the products l l (at most 2^-60 of a full-scale one) are left out.
 #pragma once
 
 #include <cuda_runtime.h>

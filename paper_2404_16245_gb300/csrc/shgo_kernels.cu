@@ -1,20 +1,7 @@
-// CUDA kernels (sm_103a, FP64) of the SHGO nuclear-attraction path.
-//
-//  k_coupling_block  (S1 + S2): one warp per primitive pair (alpha_i on a, beta_j on b).
-//      Gaussian product (Eq. 5): p, P.  Then, for every nucleus C (one lane per nucleus,
-//      chunks of 32 or 16): d = C - P, T = p |d|^2, Boys F_0..F_Lambda(T), the radial factors
-//      beta_{L,k}(T) = sum_j k!/j! T^j F_{L+j}(T) scaled by Z_C, and the real solid harmonics
-//      S_LM(d); the lanes stage them in shared memory and then contract over the nuclei of the
-//      chunk, each lane owning entries of
-//          R[L,M,k] = sum_C Z_C S_LM(C - P) beta_{L,k}(T_C),
-//      which is stored as R' = 2 pi p^{-(k+1)} R (the one-centre integral of Eq. 12 in coupled
-//      form, before the Gaunt coupling).
-//  k_pair_block      (S3 + S4 + S5): one warp per shell pair.  Couples R' of each primitive
-//      pair with the real Gaunt coefficients into W[l1 m1][l2 m2], scales by c_i c_j K_AB
-//      (beta/p)^{la-l1} (alpha/p)^{lb-l2} and sums over primitive pairs (Eq. 11); then the
-//      translation ("vector uncoupling", Eq. 7) V = T_A W T_B^T with
-//      T_A[ma][l1 m1] = sum_nu E^{la}(ma; l1 m1; nu) S_{la-l1,nu}(b - a) and T_B likewise with
-//      a - b; writes the block and its transpose into V.
+// Once-per-basis kernels of the SHGO path (S1: Gaussian products, rotations of the pair frames), the launches of V and the
+// four-centre electron-repulsion integrals (sm_103a, FP64).  The nucleus loop (S2) is in shgo_coupling.cu and
+// shgo_coupling_f32.cu, the coupling, translation and write (S3 to S5) in shgo_pair.cu, the potential in shgo_esp.cu, the
+// derivatives in shgo_deriv.cu, overlap and two-centre Coulomb integrals in shgo_twocentre.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>
