@@ -129,14 +129,18 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
   constexpr int cb1 = column_bound(LAM, NW, 1), cb2 = column_bound(LAM, NW, 2), cb3 = column_bound(LAM, NW, 3);
   const int A0 = wid == 0 ? 0 : (wid == 1 ? cb1 : (wid == 2 ? cb2 : cb3));
   const int A1 = wid == NW - 1 ? LAM + 1 : (wid == 0 ? cb1 : (wid == 1 ? cb2 : cb3));
-  for (int L = tid; L <= LAM; L += NT) {
-    const int f = beta_first(LAM, L);
-    b0[L] = f;
-    for (int k = 0; k <= (LAM - L) / 2; ++k) {
-      blk[f + k] = L | (L + 2 * k) << 8;
-      cfa[f + k] = g_far[L * (kLamDer / 2 + 1) + k];
-      cfk[f + k] = g_kfact[k];
+  // one radial row per thread, so that the loads of all rows are in flight together instead of one after another per L
+  // (V of 32 atoms with l <= 6 378 -> 372 us, of 5 such atoms 100 -> 95 us, 9 atoms with l <= 3 46.5 -> 45.4 us)
+  for (int b = tid; b < nB; b += NT) {
+    int L = 0, k = b;
+    for (int n = LAM / 2 + 1; k >= n; n = (LAM - L) / 2 + 1) {
+      k -= n;
+      ++L;
     }
+    if (k == 0) b0[L] = b;
+    blk[b] = L | (L + 2 * k) << 8;
+    cfa[b] = g_far[L * (kLamDer / 2 + 1) + k];
+    cfk[b] = g_kfact[k];
   }
   // a block takes A.group consecutive primitive pairs at a time, which mostly share their shell pair: the nuclei's
   // pair-frame coordinates (13 of some 80 FP64 instructions at small Lambda) are then formed once for the shell pair
