@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
           if ((hs & 0x7ff00000) == 0x7ff00000) Z = __longlong_as_double(0x7ff8000000000000ll);  // no finite distance
           double ri = 0.0, ux = 0.0, uy = 0.0, uz = 1.0;
           if (hs >= kTinyHi) {
-            ri = inverse_distance(s2);
+            ri = rsqrt(s2);
             ux = dx * ri;
             uy = dy * ri;
             uz = dz * ri;

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(32 * kEspWarps) k_esp(EspArgs A) {
     const double s2 = fma(z, z, fma(y, y, x * x)), T = pd.p * s2;
     double ri = 0.0, ux = 0.0, uy = 0.0, uz = 1.0;
     if (__double2hiint(s2) >= kTinyHi) {
-      ri = inverse_distance(s2);
+      ri = rsqrt(s2);
       ux = x * ri;
       uy = y * ri;
       uz = z * ri;

@@ -48,8 +48,7 @@ __host__ __device__ constexpr int beta_first(int lam, int L) {  // first radial 
   return n;
 }
 
-// C - A of a nucleus (or point) at c in the pair frame Q, and 1/|d| by the hardware estimate and one third-order step;
-// |d| below 2^-500 counts as 0 (ri = 0): only L = 0 survives there.
+// C - A of a nucleus (or point) at c in the pair frame Q.
 __device__ __forceinline__ void frame_coords(const double* Q, const double* xa, const double* c, double& x, double& y,
                                              double& z) {
   const double vx = c[0] - xa[0], vy = c[1] - xa[1], vz = c[2] - xa[2];
@@ -57,13 +56,8 @@ __device__ __forceinline__ void frame_coords(const double* Q, const double* xa, 
   y = Q[3] * vx + Q[4] * vy + Q[5] * vz;
   z = Q[6] * vx + Q[7] * vy + Q[8] * vz;
 }
-__device__ __forceinline__ double inverse_distance(double s2) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s2));
-  const double e = fma(-(s2 * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-constexpr int kTinyHi = 0x01700000;  // high word of the least |d|^2 that counts as nonzero
+// High word of the least |d|^2 that counts as nonzero: |d| below 2^-500 counts as 0, only L = 0 survives there.
+constexpr int kTinyHi = 0x01700000;
 
 // 2^a z v + n w (fixed point; the caller passes z's limbs already shifted by a).
 __device__ __forceinline__ fx fx_step(fx z, fx v, int nh, int nl, fx w) {
