@@ -92,9 +92,12 @@ struct Tables {
   // The pair kernel's form of the same programs (shgo_pair.cu).  Contracted entries of a class, (l1, l2) by (l1, l2)
   // (index l1 (lb + 1) + l2), then L = |l1 - l2|, .., l1 + l2 in steps of 2, then M: rt_src[rt_base[c] + e] = R' index
   // (L, M, (l1 + l2 - L)/2) | (l1 (lb + 1) + l2) << 16.  Rows of the class (aligned with g_rowinfo): px_rows = (W index, or
-  // 0xffff for padding, | term count << 16, first term); terms (fixed-point limbs of the coefficient, contracted entry, R' index),
+  // 0xffff for padding, | term count << 16, first term); terms (fixed-point limbs of the coefficient, contracted entry, entry of rs_src),
   // interleaved as g_terms.  axial[(l (kLmax + 1) + ..)]: E^l(m; l1 m; 0) at l (kLmax + 1)^2 + l1 (l + 1) + m, 0 for m > l1.
+  // rs_src is the same list without the blocks l1 < l2, whose entries are those of (l2, l1): it serves a single primitive
+  // pair, which needs no factors of its own.
   std::vector<int> rt_src, rt_base;  // [n classes + 1]
+  std::vector<int> rs_src, rs_base;  // [n classes + 1]
   std::vector<int2> px_rows;
   std::vector<int4> px_terms;
   std::vector<double> axial;
@@ -108,7 +111,6 @@ struct Tables {
   // R layout per Lambda: packed (harm index | beta index << 12 | k << 24) for entry e.
   std::vector<int> rmap;
   std::vector<int> rmap_off;  // [kLamDer + 2]
-  std::vector<int> rdeg;      // L + 2k of entry e, aligned with rmap
   std::vector<double> rnorm;  // N_LM of entry e (HarmCoef::n), aligned with rmap
   // Real rotation matrices D^{l+1} from D^l (S_lm(R y) = sum_m' D^l[m][m'] S_lm'(y)): the
   // harmonic part of u_c S_{l,m'}(u) for a Cartesian component c is sum_M G(1 m(c), l m'; l+1 M)
@@ -222,10 +224,10 @@ struct DeviceTables {
   double* d_low = nullptr;
   int* dt_ptr = nullptr;
   GTerm* dt_terms = nullptr;
-  int* rdeg = nullptr;        // Tables::rdeg
   // pair kernel (Tables::axial, rt_src, px_*)
   double* axial = nullptr;
   int* rt_src = nullptr;
+  int* rs_src = nullptr;
   int2* px_rows = nullptr;
   int4* px_terms = nullptr;
 };
@@ -573,7 +575,8 @@ struct PairArgs {
   const double* axial = nullptr;   // Tables::axial
   int nrt = 0;                     // contracted entries of the class
   const int* rt_src = nullptr;     // Tables::rt_src of the class
-  const int* rdeg = nullptr;       // Tables::rdeg of la + lb
+  int nrs = 0;                     // the same for one primitive pair
+  const int* rs_src = nullptr;     // Tables::rs_src of the class
   const int2* rows = nullptr;      // Tables::px_rows of the class
   const int4* terms = nullptr;     // Tables::px_terms
   const PPData* ppd = nullptr;

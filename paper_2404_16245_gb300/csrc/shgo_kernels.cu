@@ -267,9 +267,9 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = upload(&d.d_raise, t.d_raise);
   if (e == cudaSuccess) e = upload(&d.d_field, t.d_field);
   if (e == cudaSuccess) e = upload(&d.d_low, t.d_low);
-  if (e == cudaSuccess) e = upload(&d.rdeg, t.rdeg);
   if (e == cudaSuccess) e = upload(&d.axial, t.axial);
   if (e == cudaSuccess) e = upload(&d.rt_src, t.rt_src);
+  if (e == cudaSuccess) e = upload(&d.rs_src, t.rs_src);
   if (e == cudaSuccess) e = upload(&d.px_rows, t.px_rows);
   if (e == cudaSuccess) e = upload(&d.px_terms, t.px_terms);
   if (e == cudaSuccess) e = upload(&d.dt_ptr, t.dt_ptr);
@@ -456,7 +456,8 @@ struct Launcher {
     p.axial = dt.axial;
     p.nrt = th.rt_base[cid + 1] - th.rt_base[cid];
     p.rt_src = dt.rt_src + th.rt_base[cid];
-    p.rdeg = dt.rdeg + th.rmap_off[w.la + w.lb];
+    p.nrs = th.rs_base[cid + 1] - th.rs_base[cid];
+    p.rs_src = dt.rs_src + th.rs_base[cid];
     p.rows = dt.px_rows + th.g_rowbase[cid];
     p.terms = dt.px_terms + th.g_termbase[cid];
     p.ppd = db.ppd;

@@ -105,8 +105,8 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   Packer pk2;
   const size_t o_axial = pk2.add(t.axial.size() * sizeof(double));
   const size_t o_rtsrc = pk2.add(t.rt_src.size() * sizeof(int));
+  const size_t o_rssrc = pk2.add(t.rs_src.size() * sizeof(int));
   const size_t o_rows = pk2.add(t.px_rows.size() * sizeof(int2));
-  const size_t o_rdeg = pk2.add(t.rdeg.size() * sizeof(int));
   if (pk2.used > kNoallocTableBytes) {
     *err = "constant tables do not fit their static array";
     return SHGO_ERR_OOM;
@@ -118,8 +118,8 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   } pieces[] = {{d.base + o_boys, t.boys.data(), t.boys.size() * sizeof(double)},
                 {base2 + o_axial, t.axial.data(), t.axial.size() * sizeof(double)},
                 {base2 + o_rtsrc, t.rt_src.data(), t.rt_src.size() * sizeof(int)},
+                {base2 + o_rssrc, t.rs_src.data(), t.rs_src.size() * sizeof(int)},
                 {base2 + o_rows, t.px_rows.data(), t.px_rows.size() * sizeof(int2)},
-                {base2 + o_rdeg, t.rdeg.data(), t.rdeg.size() * sizeof(int)},
                 {d.base + o_terms, t.px_terms.data(), t.px_terms.size() * sizeof(int4)},
                 {d.base + o_rmap, t.rmap.data(), t.rmap.size() * sizeof(int)},
                 {d.base + o_rnorm, t.rnorm.data(), t.rnorm.size() * sizeof(double)},
@@ -137,10 +137,10 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   d.tabs.boys = reinterpret_cast<double*>(d.base + o_boys);
   d.tabs.axial = reinterpret_cast<double*>(base2 + o_axial);
   d.tabs.rt_src = reinterpret_cast<int*>(base2 + o_rtsrc);
+  d.tabs.rs_src = reinterpret_cast<int*>(base2 + o_rssrc);
   d.tabs.px_rows = reinterpret_cast<int2*>(base2 + o_rows);
   d.tabs.px_terms = reinterpret_cast<int4*>(d.base + o_terms);
   d.tabs.rmap = reinterpret_cast<int*>(d.base + o_rmap);
-  d.tabs.rdeg = reinterpret_cast<int*>(base2 + o_rdeg);
   d.tabs.rnorm = reinterpret_cast<double*>(d.base + o_rnorm);
   d.tabs.rot_ptr = reinterpret_cast<int*>(d.base + o_rotptr);
   d.tabs.rot_terms = reinterpret_cast<GTerm*>(d.base + o_rotterms);

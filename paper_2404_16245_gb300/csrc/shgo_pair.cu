@@ -11,13 +11,16 @@
 // What bounds it: in FP64 (1.7 lanes per clock and SM) the coupling is nearly half of the operations; integer
 // multiply-adds issue at 62.  Rt is therefore held as 58-bit fixed point with one exponent per (l1, l2); the coupling
 // coefficients are at most 1 and a row's absolute sum at most 1.33, so W stays in fixed point without a test, and the
-// factors of Z are scaled per (l1, |mb|).  Each sum is then within 2^-57 or so of its largest product.  Rt, Z, V' and the
-// rotation stay FP64.  The rest is latency: the threads take every entry of a chunk of eight primitive pairs without a
+// factors of Z are scaled per (l1, |mb|).  W is then within 2^-57 or so of the largest entry of its (l1, l2), Z of its
+// largest product.  Rt, Z, V' and the rotation stay FP64.  The rest is latency: the threads take every entry of a chunk of eight primitive pairs without a
 // barrier, and a row of the coupling program is one header and K coalesced 16-byte terms.
 //
 // Measured (GB300, pair phase of one V, against FP64 throughout with the coupling once per primitive pair): contracted
 // 29-atom molecule 1.14 -> 0.37 ms (V 4.40 -> 3.79 ms, six such molecules 29.8 -> 27.6 ms); 32 atoms with l <= 6,
-// uncontracted, 0.184 -> 0.160 ms (V 404 -> 392 us).
+// uncontracted, 0.184 -> 0.160 ms (V 404 -> 392 us).  One scale per (l1, l2) for single primitive pairs too, instead of
+// one per degree l1 + l2 over entries that (l1, l2) does not read: the same time (V of the 32 atoms 373 and 375 us), and
+// blocks of high degrees alone, as on one centre with la - lb >= 2, keep their digits ((6, 2), p = 100, a nucleus 20 bohr off:
+// 5.7e-8 of the largest element before).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -118,9 +121,13 @@ __global__ void __launch_bounds__(128) k_pair_block(PairArgs A) {
     const int npp = A.shell_nprim[a] * A.shell_nprim[b];
     const int64_t q0 = A.pair_ppoff[pr];
     const double dist = rd[0];
-    // one primitive pair: the coupling reads R' itself, scaled per degree L + 2k = l1 + l2 (an entry has one degree but
-    // serves several (l1, l2)), and f joins the factors of Z
-    const bool single = npp == 1 && nR < nrt;
+    // one primitive pair: the entries are R' itself, blocks (l1, l2) and (l2, l1) share them, and f joins the factors of Z.
+    // A block's scale comes from the degrees L it reads alone: for far nuclei R' falls as t^{-(L+1)}, and a pair on one
+    // centre has nothing but (la, lb), with L >= la - lb
+    const bool single = npp == 1 && A.nrs < nrt;
+    const auto scale_of = [&](int l1, int l2) {
+      return single && l1 < l2 ? l2 * (lb + 1) + l1 : l1 * (lb + 1) + l2;
+    };
     __syncthreads();  // the previous pair is done with the tables
     // translation along z (Eq. 7 with Eq. 8 coefficients, real basis): only nu = 0 survives,
     // t_A(l1, ma) = E^{la}(ma; l1 ma; 0) |b-a|^{la-l1}, t_B(l2, mb) = E^{lb}(mb; l2 mb; 0) (-|b-a|)^{lb-l2}; both depend on
@@ -163,10 +170,11 @@ __global__ void __launch_bounds__(128) k_pair_block(PairArgs A) {
       const bool first = !live;
       live = true;
       if (single) {
-        for (int e = tid; e < nR; e += nth) {
-          const double v = R[e];
+        for (int e = tid; e < A.nrs; e += nth) {
+          const int src = __ldg(A.rs_src + e);
+          const double v = R[src & 0xffff];
           Rt[e] = v;
-          atomicMax(En + __ldg(A.rdeg + e), (__double2hiint(v) >> 20) & 0x7ff);
+          atomicMax(En + (src >> 16), (__double2hiint(v) >> 20) & 0x7ff);
         }
       } else if (G == 1) {
         for (int e = tid; e < nrt; e += nth) {
@@ -207,8 +215,10 @@ __global__ void __launch_bounds__(128) k_pair_block(PairArgs A) {
         atomicMax(En + blk, (__double2hiint(s) >> 20) & 0x7ff);
       }
       __syncthreads();
-      for (int e = tid; e < (single ? nR : nrt); e += nth) {
-        const fx f = fx_of(Rt[e], En[single ? __ldg(A.rdeg + e) : __ldg(A.rt_src + e) >> 16] + 2);
+      const int* srcs = single ? A.rs_src : A.rt_src;
+      for (int e = tid; e < (single ? A.nrs : nrt); e += nth) {
+        const int src = __ldg(srcs + e);
+        const fx f = fx_of(Rt[e], En[src >> 16] + 2);
         Rx[e] = make_int2(f.h, f.l);
       }
       for (int e = tid; e < nbk; e += nth) {
@@ -216,7 +226,7 @@ __global__ void __launch_bounds__(128) k_pair_block(PairArgs A) {
         int E = kNoScale;
         for (int l2 = mb; l2 <= lb; ++l2) {
           const double c = single ? tB[l2 * (lb + 1) + mb] * fab[l1 * (lb + 1) + l2] : tB[l2 * (lb + 1) + mb];
-          const int ec = (__double2hiint(c) >> 20) & 0x7ff, n = En[single ? l1 + l2 : l1 * (lb + 1) + l2];
+          const int ec = (__double2hiint(c) >> 20) & 0x7ff, n = En[scale_of(l1, l2)];
           if (ec == 0x7ff || n == 0x7ff)
             E = kNotFinite;
           else if (ec > 0 && n > 0)
@@ -231,7 +241,7 @@ __global__ void __launch_bounds__(128) k_pair_block(PairArgs A) {
         while ((l2 + 1) * (l2 + 2) / 2 <= r) ++l2;
         const int mb = r - l2 * (l2 + 1) / 2;
         const double c = single ? tB[l2 * (lb + 1) + mb] * fab[l1 * (lb + 1) + l2] : tB[l2 * (lb + 1) + mb];
-        const fx f = fx_of(c, 1023 + Ec[l1 * (lb + 1) + mb] - En[single ? l1 + l2 : l1 * (lb + 1) + l2]);
+        const fx f = fx_of(c, 1023 + Ec[l1 * (lb + 1) + mb] - En[scale_of(l1, l2)]);
         cx[e] = make_int2(f.h, f.l);
       }
       // coupling: rows r of one warp form one group: equal trip counts, one coalesced load per term

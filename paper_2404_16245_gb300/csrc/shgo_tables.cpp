@@ -338,12 +338,6 @@ void build_tables(Tables& t) {
       boff += km + 1;
     }
   }
-  t.rdeg.resize(t.rmap.size());
-  for (size_t e = 0; e < t.rmap.size(); ++e) {
-    int L = 0;
-    while ((L + 1) * (L + 1) <= (t.rmap[e] & 0xfff)) ++L;
-    t.rdeg[e] = L + 2 * (t.rmap[e] >> 24);
-  }
   t.rnorm.resize(t.rmap.size());
   for (size_t e = 0; e < t.rmap.size(); ++e) t.rnorm[e] = harm_coef_host().n[t.rmap[e] & 0xfff];
   build_deriv_tables(t);
@@ -469,6 +463,8 @@ void build_tables(Tables& t) {
   t.g_terms.clear();
   t.rt_base.assign(kNumClasses + 1, 0);
   t.rt_src.clear();
+  t.rs_base.assign(kNumClasses + 1, 0);
+  t.rs_src.clear();
   t.px_rows.clear();
   t.px_terms.clear();
   t.axial.assign((size_t)(kLmax + 1) * (kLmax + 1) * (kLmax + 1), 0.0);
@@ -549,6 +545,21 @@ void build_tables(Tables& t) {
               }
           }
         t.rt_base[cid + 1] = (int)t.rt_src.size();
+        t.rs_base[cid] = (int)t.rs_src.size();
+        std::vector<int> one(t.rt_src.size() - t.rt_base[cid]), order;  // rs_src entry of a contracted entry
+        for (size_t e = 0; e < one.size(); ++e) {
+          const int blk = t.rt_src[t.rt_base[cid] + e] >> 16;
+          if (blk / (lb + 1) >= blk % (lb + 1)) order.push_back((int)e);
+        }
+        auto ri = [&](int e) { return t.rt_src[t.rt_base[cid] + e] & 0xffff; };
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return ri(x) < ri(y); });
+        for (int e : order) {
+          const int src = t.rt_src[t.rt_base[cid] + e], blk = src >> 16, l1 = blk / (lb + 1), l2 = blk % (lb + 1);
+          one[e] = (int)t.rs_src.size() - t.rs_base[cid];
+          if (l1 <= lb) one[at[l2 * (lb + 1) + l1][src & 0xffff]] = one[e];
+          t.rs_src.push_back(src);
+        }
+        t.rs_base[cid + 1] = (int)t.rs_src.size();
         for (int r = 0; r < nrp; ++r) {
           const int info = t.g_rowinfo[t.g_rowbase[cid] + r], g = t.g_grpbase[cid] + r / 32, K = t.g_grp[2 * g + 1];
           const int first = t.g_grp[2 * g] + r % 32, l1 = (info >> 16) & 15, l2 = (info >> 20) & 15;
@@ -558,7 +569,8 @@ void build_tables(Tables& t) {
             const long long q = std::llrint(std::ldexp(gt.coef, 58));  // limbs as in shgo_fixed.cuh
             const long long lo = (long long)((unsigned long long)q << 35) >> 35;
             int4& x = t.px_terms[t.g_termbase[cid] + first + 32 * j];
-            x = make_int4((int)((q - lo) >> 29), (int)lo, gt.coef != 0.0 ? at[l1 * (lb + 1) + l2][gt.ridx] : 0, gt.ridx);
+            const int src = gt.coef != 0.0 ? at[l1 * (lb + 1) + l2][gt.ridx] : 0;
+            x = make_int4((int)((q - lo) >> 29), (int)lo, src, one[src]);
           }
         }
       }
