@@ -7,6 +7,9 @@
 // The gradient is the same form: d/dx of the integral of f(r - P)/|r - x| is that of the gradient of f, whose
 // one-centre parts are fixed combinations of order Lambda + 1 (Tables::d_field, d_raise), so the adjoint of that step and
 // the rotation to the molecular frame give three sets of weights of order Lambda + 1, summed against one set of tables.
+// Far away that sum over the rows of a degree cancels down to the degrees L + 1 (t^2 in accuracy: 5e-12 of a p-s pair's
+// gradient at p = 100, 20 bohr off), so the far weights of the gradient come from those of the potential instead, by the
+// derivative of S_LM(d) / |d|^{2L+1} (Tables::fr_terms; 3e-16 there, 1 % of the call of 251 points).
 //
 // What bounds it: as in the coupling kernel FP64 (1.7 lanes per clock and SM) is kept for the geometry, the radial
 // values and one multiply-add per radial row; the harmonics and the sums over M run in 58-bit fixed point on the integer
@@ -262,7 +265,7 @@ __host__ __device__ inline size_t adjoint_smem(int la, int lb) {
   const int nWa = (la + 1) * (la + 1), na = 2 * la + 1, nb = 2 * lb + 1, lm = la > lb ? la : lb;
   const int lam1 = la + lb + (NC == 3 ? 1 : 0);
   return sizeof(double) * ((size_t)nWa * w_stride(lb) + na * na + nb * nb + (la + 1) * na + (lb + 1) * nb +
-                           3 * na * nb + (la + 1) * (lb + 1) + lam1 + 1 + lm + 1 + 8 + n_r(la + lb) +
+                           3 * na * nb + (la + 1) * (lb + 1) + lam1 + 1 + lm + 1 + 8 + n_r(la + lb) + (NC == 3 ? n_harm(la + lb) : 0) +
                            NC * (n_r(lam1) + n_harm(lam1))) +
          sizeof(int) * (size_t)(NC * (n_beta(lam1) + lam1 + 1) + 3 * (lam1 + 2) + 8);
 }
@@ -283,6 +286,7 @@ struct AdjointArgs {
   const GTerm* gt_terms;
   const int* dt_ptr;       // transposed field step of la + lb (gradient)
   const GTerm* dt_terms;
+  const GTerm* fr_terms;   // derivative of the far field (gradient)
   const int* rmap;         // layout of the weights' order
   const double* rnorm;
   const PPData* ppd;
@@ -313,7 +317,8 @@ __global__ void __launch_bounds__(128) k_esp_adjoint(AdjointArgs A) {
   double* dpow = pw + lam1 + 1;
   double* scal = dpow + lm + 1;
   double* g0 = scal + 8;                   // [nR0] weights of the unscaled coupling block
-  double* fin = g0 + nR0;                  // [NC][nR] weights
+  double* qf = g0 + nR0;                   // [n_harm(lam)] far field of the coupling block (gradient)
+  double* fin = qf + (NC == 3 ? n_harm(lam) : 0);  // [NC][nR] weights
   double* far = fin + NC * nR;             // [NC][nS] weights of the far points
   int* ex = reinterpret_cast<int*>(far + NC * nS);  // [NC][nB], [NC][lam1 + 1] biased exponents
   int* b0 = ex + NC * (nB + lam1 + 1);     // first radial row of L
@@ -443,13 +448,41 @@ __global__ void __launch_bounds__(128) k_esp_adjoint(AdjointArgs A) {
           for (int x = 0; x < 3; ++x) fin[x * nR + e] = Q[x] * h[0] + Q[3 + x] * h[1] + Q[6 + x] * h[2];
         }
       }
+      if constexpr (NC == 3) {
+        int r = 0, L = 0;  // first entry of degree L in g0
+        for (int h = tid; h < n_harm(lam); h += nth) {
+          for (; (L + 1) * (L + 1) <= h; ++L) r += (2 * L + 1) * ((lam - L) / 2 + 1);
+          const int nk = (lam - L) / 2 + 1;
+          const double* v = g0 + r + (h - L * L) * nk;
+          double s = 0.0;
+          for (int k = 0; k < nk; ++k) s = fma(g_far[L * (kLamDer / 2 + 1) + k] * (g_kfact[k] * pw[L + 2 * k]), v[k], s);
+          qf[h] = s;
+        }
+      }
       __syncthreads();
-      for (int x = tid; x < NC * nS; x += nth) {
-        const int c = x / nS, h = x - c * nS, L = __ldg(rowcode + h) >> 16, nk = (lam1 - L) / 2 + 1;
-        const double* v = fin + c * nR + rb[L] + (h - L * L) * nk;
-        double s = 0.0;
-        for (int k = 0; k < nk; ++k) s = fma(g_far[L * (kLamDer / 2 + 1) + k], v[k], s);
-        far[x] = s;
+      if constexpr (NC == 1) {
+        for (int h = tid; h < nS; h += nth) {
+          const int L = __ldg(rowcode + h) >> 16, nk = (lam1 - L) / 2 + 1;
+          const double* v = fin + rb[L] + (h - L * L) * nk;
+          double s = 0.0;
+          for (int k = 0; k < nk; ++k) s = fma(g_far[L * (kLamDer / 2 + 1) + k], v[k], s);
+          far[h] = s;
+        }
+      } else {
+        // gradient of the far field sum q_LM S_LM(u) t^{-(L+1)}, which has degrees L + 1 alone (the sums over k of the
+        // weights above hold degrees L - 1 as well, that cancel in exact arithmetic only: t^2 in accuracy)
+        for (int h = tid; h < nS; h += nth) {
+          const int L = __ldg(rowcode + h) >> 16;
+          const double s = pd.sp * __ldg(A.rnorm + rb[L] + (h - L * L) * ((lam1 - L) / 2 + 1));
+          double f[kFarSlots];
+#pragma unroll
+          for (int j = 0; j < kFarSlots; ++j) {
+            const GTerm t = A.fr_terms[kFarSlots * h + j];
+            f[j] = t.coef * qf[t.ridx];
+          }
+          const double gx = (f[0] + f[1]) * s, gy = (f[2] + f[3]) * s, gz = f[4] * s;
+          for (int x = 0; x < 3; ++x) far[x * nS + h] = Q[x] * gx + Q[3 + x] * gy + Q[6 + x] * gz;
+        }
       }
       __syncthreads();
       // exponent of each row: the largest of |W_M| 2^-e(L,M)
@@ -592,6 +625,7 @@ cudaError_t launch_pieces(const DeviceBasis& db, const DeviceTables& dt, const s
       a.gt_terms = dt.gt_terms + th.gt_termbase[cid];
       a.dt_ptr = dt.dt_ptr + th.dt_base[lam];
       a.dt_terms = dt.dt_terms;
+      a.fr_terms = dt.fr_terms;
       a.rmap = dt.rmap + th.rmap_off[lam1];
       a.rnorm = dt.rnorm + th.rmap_off[lam1];
       a.ppd = db.ppd;

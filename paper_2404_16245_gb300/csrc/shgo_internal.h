@@ -68,6 +68,8 @@ struct __align__(16) GTerm {
 };
 
 // Host tables, built once per process (long double arithmetic, stored as double).
+constexpr int kFarSlots = 5;  // Tables::fr_terms
+
 struct Tables {
   std::vector<double> boys;  // [kBoysNg][kBoysStride]
   std::vector<double> boys_top;  // [kLamDer + 1][kBoysTopRows][kBoysTopStride]
@@ -154,6 +156,9 @@ struct Tables {
   // dt_terms[dt_ptr[dt_base[Lambda] + 3 e' + c] .. + 1] = (coefficient, e, 1 for a d_raise term).
   std::vector<int> dt_ptr, dt_base;
   std::vector<GTerm> dt_terms;
+  // d/dr_c S_LM(r) / |r|^{2L+1} is a sum over (L + 1, M'): for h = harmonic index of (L + 1, M'), (coefficient, harmonic index
+  // of (L, M)) at fr_terms[kFarSlots h + s], s = 0, 1 for c = x, 2, 3 for y, 4 for z (unused ones with coefficient 0).
+  std::vector<GTerm> fr_terms;
   // Four-centre electron repulsion: r^{2k} S_LM(r) e^{-p r^2} = sum_{n<=k} eps_{k,n}(L) p^{-(k+n)}
   // Laplacian^n [S_LM(r) e^{-p r^2}], with eps_{k,n}(L) at eri_eps[(L (kC2K + 1) + k)(kC2K + 1) + n].
   std::vector<double> eri_eps;
@@ -224,6 +229,7 @@ struct DeviceTables {
   double* d_low = nullptr;
   int* dt_ptr = nullptr;
   GTerm* dt_terms = nullptr;
+  GTerm* fr_terms = nullptr;
   // pair kernel (Tables::axial, rt_src, px_*)
   double* axial = nullptr;
   int* rt_src = nullptr;

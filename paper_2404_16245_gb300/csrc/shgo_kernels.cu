@@ -274,6 +274,7 @@ shgo_status device_tables(int device, const DeviceTables** out, std::string* err
   if (e == cudaSuccess) e = upload(&d.px_terms, t.px_terms);
   if (e == cudaSuccess) e = upload(&d.dt_ptr, t.dt_ptr);
   if (e == cudaSuccess) e = upload(&d.dt_terms, t.dt_terms);
+  if (e == cudaSuccess) e = upload(&d.fr_terms, t.fr_terms);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_harm, &harm_coef_host(), sizeof(HarmCoef));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_boys, &boys_const_host(), sizeof(BoysConst));
   if (e == cudaSuccess) e = coupling_fp64_setup();

@@ -272,6 +272,21 @@ void build_deriv_tables(Tables& t) {
     t.dt_ptr.push_back((int)t.dt_terms.size());
   }
   t.dt_base[kLamMax + 1] = (int)t.dt_ptr.size();
+  // S_LM(r) / |r|^{2L+1} = (-1)^L / (2L - 1)!! S_LM(grad) 1/|r| (Hobson), r_c S_LM = sum G S_{L+1,M'} + |r|^2 (..) by the
+  // product rule, and the Laplacian of 1/|r| is zero: the derivative is -(2L + 1) sum G(1 c, L M; L+1 M') S_{L+1,M'} / |r|^{2L+3}
+  t.fr_terms.assign((size_t)kFarSlots * n_harm(kLamMax + 1), GTerm{0.0, 0, 0});
+  for (int L = 0; L <= kLamMax; ++L)
+    for (int Mp = -(L + 1); Mp <= L + 1; ++Mp)
+      for (int c = 0; c < 3; ++c) {
+        GTerm* slots = &t.fr_terms[(size_t)kFarSlots * harm_index(L + 1, Mp) + 2 * c];
+        int n = 0;
+        for (int M = -L; M <= L; ++M) {
+          const double g = gaunt_real(1, mc[c], L, M, L + 1, Mp);
+          if (std::fabs(g) <= 1e-15) continue;
+          if (n == (c == 2 ? 1 : 2)) throw std::logic_error("far field derivative: more terms than slots");
+          slots[n++] = GTerm{-(2 * L + 1) * g, harm_index(L, M), 0};
+        }
+      }
   t.d_low_off.assign(kLmax + 2, 0);
   t.d_low.clear();
   for (int l = 0; l <= kLmax; ++l) {
