@@ -25,7 +25,8 @@
 //
 // Measured (GB300, 32 atoms with l <= 6, 25,200 shell pairs): (a|b) 421 -> 63 us against one block per shell pair for all
 // steps, overlap 95 -> 55 us against a warp per pair with D^la diag(d) (D^lb)^T.  Of that, rows of terms read coalesced
-// instead of one list per lane and the harmonics in the radial launch instead of their own: 86 -> 63, 78 -> 55 us.
+// instead of one list per lane and the harmonics in the radial launch instead of their own: 86 -> 63, 78 -> 55 us.  The overlap of small bases keeps
+// the warp-per-pair form in one launch (overlap_in_one_launch).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -272,6 +273,174 @@ __global__ void __launch_bounds__(32 * kBlockWarps) k_twocentre_blocks(
   }
 }
 
+// Overlap of small bases, all steps of a shell pair in one warp and one launch: S' = diag(d) of the pair frame rotated
+// back, S = D^{la} diag(d) (D^{lb})^T.  More FP64 operations than the X_L form but no second launch, no tables and no
+// work array in between (rule and figures at overlap_in_one_launch).
+//
+// Shared doubles of one warp for angular momenta up to lm: D^{la} and D^{lb}, t_A and t_B, w(l1), |b - a|^k,
+// d(m) and X = D^{la} diag(d).
+__host__ __device__ inline int overlap_warp_doubles(int lm) {
+  const int n = 2 * lm + 1;
+  return 3 * n * n + 2 * (lm + 1) * n + 2 * (lm + 1) + n + 1;
+}
+
+__global__ void __launch_bounds__(32 * kBlockWarps) k_overlap(PairClasses cls, int lm_max,
+                                                                const int* __restrict__ pair_a,
+                                                                const int* __restrict__ pair_b,
+                                                                const int64_t* __restrict__ pair_ppoff,
+                                                                const int* __restrict__ pair_site, int64_t rot_per,
+                                                                const double* __restrict__ rotd,
+                                                                const int* __restrict__ shell_nprim,
+                                                                const int64_t* __restrict__ shell_foff,
+                                                                const double* __restrict__ etab,
+                                                                const int* __restrict__ eoff,
+                                                                const PPData* __restrict__ ppd, MolView mv,
+                                                                double* __restrict__ out) {
+  extern __shared__ double smem[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  double* wsm = smem + wib * overlap_warp_doubles(lm_max);
+  const int total = cls.first[cls.n];
+  for (int item = blockIdx.x * kBlockWarps + wib; item < total; item += gridDim.x * kBlockWarps) {
+    const int c = class_of_item(cls, item);
+    const int la = cls.la[c], lb = cls.lb[c];
+    const int pr = cls.pair_base[c] + (item - cls.first[c]);
+    const int na = 2 * la + 1, nb = 2 * lb + 1;
+    const int lm = la > lb ? la : lb, ln = la < lb ? la : lb;
+    const int nDb = la != lb ? nb * nb : 0;
+    double* Dm = wsm;  // D^{la}(Q^T), then D^{lb}(Q^T) when lb != la
+    double* tA = Dm + na * na + nb * nb;
+    double* tB = tA + (la + 1) * na;
+    double* wl = tB + (lb + 1) * nb;  // w(l1)
+    double* dpow = wl + lm + 1;       // |b - a|^k
+    double* dm = dpow + lm + 1;       // d(m), m = -ln..ln
+    double* X = dm + 2 * lm + 1;      // [ma][m] = D^{la}[ma][m] d(m)
+    const int nm = 2 * ln + 1;
+    const int a = pair_a[pr], b = pair_b[pr];
+    const double* rd = rotd + (int64_t)pair_site[pr] * rot_per;
+    __syncwarp();  // the warp's previous pair is done with its tables
+    if (lane == 0) {
+      const double dist = rd[0];
+      double v = 1.0;
+      for (int k = 0; k <= lm; ++k) {
+        dpow[k] = v;
+        v *= dist;
+      }
+    }
+    for (int e = lane; e < na * na; e += 32) Dm[e] = rd[1 + rot_doff(la) + e];
+    for (int e = lane; e < nDb; e += 32) Dm[na * na + e] = rd[1 + rot_doff(lb) + e];
+    // radial sums over primitive pairs, one l1 per lane
+    if (lane <= ln) {
+      const int l1 = lane;
+      double dfact = 1.0;
+      for (int k = 2 * l1 - 1; k > 1; k -= 2) dfact *= k;
+      // 4 pi (pi/2)^{1/2} / 2^{l1 + 3/2} (2 l1 - 1)!!
+      double cf = 4.0 * 3.14159265358979323846 * 1.2533141373155002512 * dfact * 0.35355339059327376220;
+      for (int k = 0; k < l1; ++k) cf *= 0.5;
+      const int64_t q0 = pair_ppoff[pr];
+      const int npp = shell_nprim[a] * shell_nprim[b];
+      double acc = 0.0;
+      for (int ij = 0; ij < npp; ++ij) {
+        const PPData pd = ppd[q0 + ij];
+        if (pd.pref == 0.0) continue;
+        double v = pd.pref * pd.rp * (pd.sp * pd.rp);  // p^{-3/2}
+        for (int k = 0; k < l1; ++k) v *= pd.rp;
+        for (int k = 0; k < la - l1; ++k) v *= pd.ra;
+        for (int k = 0; k < lb - l1; ++k) v *= pd.rb;
+        acc += v;
+      }
+      wl[l1] = cf * acc;
+    }
+    __syncwarp();
+    for (int e = lane; e < (la + 1) * na; e += 32) {
+      const int l1 = e / na, ma = e % na - la, lr = la - l1;
+      tA[e] = l1 >= (ma < 0 ? -ma : ma) ? etab[eoff[la] + translation_offset_dev(la, ma, l1, ma) + lr] * dpow[lr] : 0.0;
+    }
+    for (int e = lane; e < (lb + 1) * nb; e += 32) {
+      const int l2 = e / nb, mb = e % nb - lb, lr = lb - l2;
+      tB[e] = l2 >= (mb < 0 ? -mb : mb)
+                  ? etab[eoff[lb] + translation_offset_dev(lb, mb, l2, mb) + lr] * ((lr & 1) ? -dpow[lr] : dpow[lr])
+                  : 0.0;
+    }
+    __syncwarp();
+    // S' = diag(d), d(m) = sum_{l1 >= |m|} t_A(l1, m) t_B(l1, m) w(l1) for |m| <= min(la, lb), once per pair
+    if (lane < nm) {
+      const int m = lane - ln, am = m < 0 ? -m : m;
+      double d = 0.0;
+      for (int l1 = am; l1 <= ln; ++l1) d = fma(tA[l1 * na + m + la] * tB[l1 * nb + m + lb], wl[l1], d);
+      dm[lane] = d;
+    }
+    __syncwarp();
+    const double* Da = Dm;
+    const double* Db = la != lb ? Dm + na * na : Dm;
+    for (int e = lane; e < na * nm; e += 32) {
+      const int r = e / nm, j = e - r * nm;
+      X[e] = Da[r * na + j - ln + la] * dm[j];
+    }
+    __syncwarp();
+    // S = X (D^{lb})^T; a diagonal block (a == b) takes the entry below its diagonal from the products of the
+    // entry above it, so it is exactly symmetric
+    const int64_t fa0 = shell_foff[a], fb0 = shell_foff[b];
+    int64_t obase, ld;
+    mol_output(mv, pr, obase, ld);
+    double* o = out + obase;
+    for (int e = lane; e < na * nb; e += 32) {
+      const int ma = e / nb, mb = e % nb;
+      const bool lower = a == b && ma > mb;
+      const int r = lower ? mb : ma, q = lower ? ma : mb;
+      double s = 0.0;
+      for (int j = 0; j < nm; ++j) s = fma(X[r * nm + j], Db[q * nb + j - ln + lb], s);
+      o[(fa0 + ma) * ld + fb0 + mb] = s;
+      if (a != b) o[(fb0 + mb) * ld + fa0 + ma] = s;
+    }
+  }
+}
+
+// FP64 warp instructions of k_overlap for the shell pairs of `work`, about: per primitive pair the power products, per shell
+// pair the translation factors and the rotation.  Up to kOneLaunch of them per SM (FP64 takes 19 clocks each) the one
+// launch is over before the two launches of the X_L form, whose chains take 20 to 90 us whatever the size.  Measured (GB300,
+// one launch and two, with the count per SM): 2 atoms with l <= 8 (100) 23 and 47 us, 10 with l <= 3 contracted (1000) 17 and
+// 32, 3 contracted atoms up to g shells (1400) 59 and 92, 40 with l <= 2 (2200) 17 and 26, 14 with l <= 6 (2300) 25 and 32,
+// 16 with l <= 6 (3000) 34 and 31, 20 with l <= 6 (4600) 41 and 36.
+constexpr int64_t kOneLaunch = 2600;
+bool overlap_in_one_launch(const std::vector<ClassWork>& work) {
+  int64_t w = 0;
+  for (const ClassWork& c : work) {
+    const int na = 2 * c.la + 1, nb = 2 * c.lb + 1;
+    const auto rows = [](int n) { return (n + 31) / 32; };
+    w += c.npp * (14 + c.la + c.lb) + c.npairs * (int64_t)(20 + c.la + 3 * c.lb + rows(na * nb) * (nb + 2) +
+                                                          rows((c.la + 1) * na) + rows((c.lb + 1) * nb));
+  }
+  return w <= kOneLaunch * grid_cap_sm(INT64_MAX, 1);
+}
+
+shgo_status launch_overlap_small(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
+                                 const MolView& mv, double* out, cudaStream_t stream, std::string* err) {
+  PairClasses cls{};
+  int total = 0, lm = 0;
+  for (const ClassWork& w : work) {
+    if (w.npairs == 0) continue;
+    cls.first[cls.n] = total;
+    cls.pair_base[cls.n] = w.pair_base;
+    cls.la[cls.n] = (unsigned char)w.la;
+    cls.lb[cls.n] = (unsigned char)w.lb;
+    ++cls.n;
+    total += w.npairs;
+    lm = std::max(lm, w.la);
+  }
+  cls.first[cls.n] = total;
+  if (total == 0) return SHGO_OK;
+  k_overlap<<<grid_cap_sm(((int64_t)total + kBlockWarps - 1) / kBlockWarps, 12), 32 * kBlockWarps,
+              sizeof(double) * kBlockWarps * (size_t)overlap_warp_doubles(lm), stream>>>(
+      cls, lm, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, rot_block(db.rot_lmax), db.rotd, db.shell_nprim,
+      db.shell_foff, dt.etab, dt.eoff, db.ppd, mv, out);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    *err = std::string("overlap launch: ") + cudaGetErrorString(e);
+    return SHGO_ERR_CUDA;
+  }
+  return SHGO_OK;
+}
+
 // Doubles of X formed at a time (128 MiB); larger bases run in pieces of whole shell pairs.
 constexpr int64_t kXDoubles = (int64_t)1 << 24;
 
@@ -367,6 +536,7 @@ shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTa
 
 shgo_status launch_overlap(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work,
                            const MolView& mv, double* out, cudaStream_t stream, std::string* err) {
+  if (overlap_in_one_launch(work)) return launch_overlap_small(db, dt, work, mv, out, stream, err);
   return launch_twocentre(false, db, dt, work, mv, out, stream, err);
 }
 
