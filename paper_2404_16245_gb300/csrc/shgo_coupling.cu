@@ -36,6 +36,9 @@
 // primitive pairs (after the pair kernel's contraction): 3.79 -> 3.69 ms, batch 27.6 -> 25.2 ms.  Errors against 64-bit
 // quadrature are the same to two digits.  At Lambda <= 2 the FP64 pipe is 76 % busy (84 % is what plain DFMAs reach), from
 // Lambda 4 on a primitive pair's dependent chains bound it (15 to 20 warps on an SM, FP64 pipe 45 to 55 % busy).
+// Small calls, where a launch is one chain (7 to 9 us at Lambda <= 4): block tables by asynchronous copies, harmonic steps and row
+// codes in shared memory, shorter sums and one split of shared memory for all kernels of a call: V of 20 atoms with l <= 2
+// 50 -> 42 us, of 4 contracted atoms 46 -> 40, of 3 atoms with l <= 2 34 -> 33 (all in FP64: 52, 57, 32).
 #include <cuda_runtime.h>
 
 #include <utility>
@@ -57,12 +60,21 @@ __device__ double2 g_boys_top[(kLamDer + 1) * kBoysTopRows * kBoysTopStride / 2]
 __host__ __device__ constexpr int coupling_warps(int lam) { return lam <= 5 ? 1 : (lam <= 8 ? 2 : 4); }
 
 constexpr int kHalf = 16;         // columns of the harmonic table
-constexpr int kHS = kHalf + 1;   // its row stride: odd, so that 8-byte loads of different rows fall in different banks
+constexpr int kHS = kHalf + 1;   // its row stride: odd, so that 8-byte loads of different rows fall in different banks; the
+                                 // last word holds the row's codes (g_row) of the two sets of scales
+
+// Global to shared memory without a register: the tables of a block arrive behind the first nuclei's loads.
+template <int N>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"(N));
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int LAM>
 struct Shape {
   static constexpr int nS = n_harm(LAM), nB = n_beta(LAM), nR = n_r(LAM), NW = coupling_warps(LAM);
-  static constexpr size_t smem = 8 * (size_t)(nS * kHS + (nB + 3) * kCS + nR + nS + 4 * nB + (LAM + 1)) +
+  static constexpr int nK = NW == 1 ? (LAM + 1) * (LAM + 2) / 2 : 0;  // steps kept in shared memory, per set
+  static constexpr size_t smem = 32 * (size_t)nK + 8 * (size_t)(nS * kHS + (nB + 3) * kCS + nR + nS + 4 * nB + (LAM + 1)) +
                                  4 * (size_t)(2 * nB + 2 * (LAM + 1) + 8);
 };
 
@@ -79,7 +91,7 @@ __host__ __device__ constexpr int column_bound(int lam, int nw, int w) {
 // Columns m = am (neg: -am), am in [A0, A1), of V_lm into rows h of St at column c: the two signs on the two halves of a
 // warp, so that 16 nuclei fill it.
 template <int LAM>
-__device__ __forceinline__ void harmonic_half(int A0, int A1, int set, bool neg, fx x, fx y, fx z, int2* St, int c) {
+__device__ __forceinline__ void harmonic_half(int A0, int A1, const int4* steps, bool neg, fx x, fx y, fx z, int2* St, int c) {
   fx dp = {1 << kFxLimb, 0}, dm = {0, 0};  // (x + iy)^am
   const fx ny = fx_neg(y);
 #pragma unroll 1
@@ -91,7 +103,7 @@ __device__ __forceinline__ void harmonic_half(int A0, int A1, int set, bool neg,
       for (int l = am;; ++l) {
         if (!neg || am) St[(l * l + l + sm) * kHS + c] = make_int2(v1.h, v1.l);
         if (l == LAM) break;
-        const int4 s = k_step[set + l * (l + 1) / 2 + am];
+        const int4 s = steps[l * (l + 1) / 2 + am];
         const fx vn = fx_step(fx{z.h << s.z, z.l << s.z}, v1, s.x, s.y, v0);
         v0 = v1;
         v1 = vn;
@@ -108,7 +120,8 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
   using Sh = Shape<LAM>;
   constexpr int NW = Sh::NW, NT = 32 * NW, nS = Sh::nS, nB = Sh::nB, nR = Sh::nR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  int2* St = reinterpret_cast<int2*>(smem_raw);             // [nS] harmonic rows of 16 columns
+  int4* Ks = reinterpret_cast<int4*>(smem_raw);             // [2][nK] steps of the harmonics
+  int2* St = reinterpret_cast<int2*>(Ks + 2 * Sh::nK);             // [nS] harmonic rows of 16 columns
   int2* Bt = St + nS * kHS;                                  // [nB] radial rows (doubles, then fixed point but on the axis)
   int2* Xt = Bt + nB * kCS;                                  // [3] x, y, z of the columns
   double* nacc = reinterpret_cast<double*>(Xt + 3 * kCS);    // [nR] near sums
@@ -139,8 +152,16 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
     }
     if (k == 0) b0[L] = b;
     blk[b] = L | (L + 2 * k) << 8;
-    cfa[b] = g_far[L * (kLamDer / 2 + 1) + k];
-    cfk[b] = g_kfact[k];
+    copy_async<8>(cfa + b, g_far + L * (kLamDer / 2 + 1) + k);
+    copy_async<8>(cfk + b, g_kfact + k);
+  }
+  // the tables of a block: a small call is one block's chain of dependent instructions and cold loads per launch, so none of
+  // these loads is waited for before the first nuclei's own
+  for (int k = tid; k < 2 * Sh::nK; k += NT) copy_async<16>(Ks + k, g_step + (k < Sh::nK ? k : kSteps + k - Sh::nK));
+  for (int h = tid; h < nS; h += NT) {
+    int2* code = St + h * kHS + kHalf;
+    copy_async<4>(&code->x, g_row + h);
+    copy_async<4>(&code->y, g_row + kRows + h);
   }
   // a block takes A.group consecutive primitive pairs at a time, which mostly share their shell pair: the nuclei's
   // pair-frame coordinates (13 of some 80 FP64 instructions at small Lambda) are then formed once for the shell pair
@@ -255,15 +276,17 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
             bo += (LAM - L) / 2 + 1;
           }
         }
+        copy_wait();  // the block's tables, on its first primitive pair
         __syncthreads();
         const int n1 = cnt[0], n2 = cnt[1], n3 = cnt[2], n4 = cnt[3], er = cnt[4];
-        const int set = er < 0 ? kSteps : 0, col = lane & (kHalf - 1);
-        const int* rowcode = g_row + (er < 0 ? kRows : 0);
+        const int4* steps = NW == 1 ? Ks + (er < 0 ? Sh::nK : 0) : k_step + (er < 0 ? kSteps : 0);
+        const int col = lane & (kHalf - 1);
+        const int* rowcode = reinterpret_cast<const int*>(St + kHalf) + (er < 0 ? 1 : 0);  // row h at 2 h kHS
         auto columns = [&](int h0) {
           const int c = h0 + col;
           if (c < n2) {
             const int2 a = Xt[c], b = Xt[kCS + c], z = Xt[2 * kCS + c];
-            harmonic_half<LAM>(A0, A1, set, lane >= kHalf, fx{a.x, a.y}, fx{b.x, b.y}, fx{z.x, z.y}, St, col);
+            harmonic_half<LAM>(A0, A1, steps, lane >= kHalf, fx{a.x, a.y}, fx{b.x, b.y}, fx{z.x, z.y}, St, col);
           }
         };
         // radial rows into fixed point, lane = column
@@ -304,10 +327,10 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
           const int hn = min(n1, h0 + kHalf), hf = min(n2, h0 + kHalf), f0 = max(n1, h0);
           if (f0 < hf) {
             for (int h = tid; h < nS; h += NT) {
-              const int code = __ldg(rowcode + h), L = code >> 16;
+              const int code = rowcode[2 * h * kHS], L = code >> 16;
               const int2 *s = St + h * kHS - h0, *b = Bt + b0[L] * kCS;
               long long hh = 0, mid = 0;
-#pragma unroll 4
+#pragma unroll (NW == 1 ? 1 : 4)  // short code where a warp is alone: each launch fetches it anew
               for (int c = f0; c < hf; ++c) {
                 const int2 u = s[c], v = b[c];
                 hh = fx_mad(u.x, v.x, hh);
@@ -325,10 +348,10 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
           if (h0 < hn) {
             for (int e = tid; e < nR; e += NT) {
               const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
-              const int rc = __ldg(rowcode + h);
+              const int rc = rowcode[2 * h * kHS];
               const int2 *s = St + h * kHS - h0, *r = Bt + b * kCS;
               long long hh = 0, mid = 0;
-#pragma unroll 4
+#pragma unroll (NW == 1 ? 1 : 4)  // short code where a warp is alone: each launch fetches it anew
               for (int c = h0; c < hn; ++c) {
                 const int2 u = s[c], x = r[c];
                 hh = fx_mad(u.x, x.x, hh);
@@ -351,10 +374,11 @@ __global__ void __launch_bounds__(32 * coupling_warps(LAM)) k_coupling_fp64(Coup
         const int code = __ldg(A.rmap + e), h = code & 0xfff, b = (code >> 12) & 0xfff;
         double v = havenear ? nacc[e] : 0.0;
         if (havefar) v = fma(fard[h], cfa[b], v);
-        out[e] = fma(v, __ldg(A.rnorm + e), (__ldg(g_row + h) & 0xff) == 0 ? axs[b] : 0.0) * sb[b];
+        out[e] = fma(v, __ldg(A.rnorm + e), (St[h * kHS + kHalf].x & 0xff) == 0 ? axs[b] : 0.0) * sb[b];
       }
     }
   });
+  copy_wait();
 }
 
 using CouplingKernel = void (*)(CouplingArgs);
@@ -381,8 +405,10 @@ cudaError_t coupling_fp64_setup() {
   cudaError_t e = upload_nucleus_constants();
   const std::vector<double>& bt = tables_host().boys_top;
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_boys_top, bt.data(), sizeof(double) * bt.size());
-  for (int lam = 0; lam <= kLamDer && e == cudaSuccess; ++lam)
+  for (int lam = 0; lam <= kLamDer && e == cudaSuccess; ++lam) {
     e = set_max_dynamic_smem((const void*)kernel_at(lam, Lams{}));
+    if (e == cudaSuccess) e = set_max_carveout((const void*)kernel_at(lam, Lams{}));
+  }
   return e;
 }
 

@@ -27,6 +27,7 @@ __constant__ BoysConst k_boys;
 // (2^e_1 <= 1 / max |V / (x + iy)^m|, reached at z = 1).
 constexpr int kSteps = (kLamDer + 1) * (kLamDer + 2) / 2;
 __constant__ int4 k_step[2 * kSteps];
+__device__ int4 g_step[2 * kSteps];  // the same, for copies to shared memory
 // Per set and harmonic row h = (L, M): |M| | e(L, M) << 8 | L << 16.
 constexpr int kRows = (kLamDer + 1) * (kLamDer + 1);
 __device__ int g_row[2 * kRows];
@@ -213,6 +214,7 @@ inline cudaError_t upload_nucleus_constants() {
   for (int k = 1; k <= kLamDer / 2; ++k) kf[k] = kf[k - 1] * k;
   cudaError_t e = cudaMemcpyToSymbol(k_boys, &boys_const_host(), sizeof(BoysConst));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(k_step, step.data(), sizeof(int4) * step.size());
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_step, step.data(), sizeof(int4) * step.size());
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_row, row.data(), sizeof(int) * row.size());
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_far, far, sizeof(far));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_kfact, kf, sizeof(kf));
