@@ -269,8 +269,11 @@ shgo_status shgo_nuclear_attraction_batched(shgo_basis* batch, const double* cen
  * point then needs only the Boys values and solid harmonics of x_k - P per primitive pair (Eq. 11).
  * density: device, nbf x nbf row-major, symmetric (D_ab and D_ba both enter).  points: device
  * [n][3] (bohr).  phi: device [n], overwritten.  Single bases only (a batch, or a basis whose
- * coupling buffer is split into regions, gives SHGO_ERR_INVALID_ARG); uses the basis's coupling
- * buffer, so calls on one basis must be ordered with its other calls.  Asynchronous on `stream`. */
+ * coupling buffer is split into regions, gives SHGO_ERR_INVALID_ARG).  The weights of the primitive pairs
+ * (about n_r(la + lb) doubles each) are a work array of the call, taken stream-ordered in pieces of up to
+ * 64 MiB on each of 16 internal streams (SHGO_ESP_SCRATCH_DOUBLES sets another size), in smaller pieces
+ * where the device has no room for these; SHGO_ERR_OOM if one shell pair per stream does not fit.
+ * Asynchronous on `stream`. */
 shgo_status shgo_esp(const shgo_basis* basis, const double* density, const shgo_centers* points, double* phi,
                      void* stream);
 

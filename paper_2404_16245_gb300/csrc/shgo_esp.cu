@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdlib>
 #include <string>
 #include <utility>
 #include <vector>
@@ -557,7 +558,11 @@ std::vector<ClassWork> pieces(const ClassWork& w, const int64_t* ppoff, int64_t 
   return out;
 }
 
-constexpr int64_t kPieceWords = (int64_t)1 << 24;  // weights of one piece: 128 MiB (one region per pool stream)
+// Weights of one piece, in 8-byte words, one region per pool stream: 64 MiB, so that the regions of all 16 streams stay
+// within what the workspace pool keeps between calls (600 points of 150 atoms with l <= 6 take 27.6 ms, gradient 55.6 ms,
+// with 32, 64 and 128 MiB alike).
+// SHGO_ESP_SCRATCH_DOUBLES sets another size.
+constexpr int64_t kPieceWords = (int64_t)1 << 23;
 
 template <int NC>
 cudaError_t launch_pieces(const DeviceBasis& db, const DeviceTables& dt, const std::vector<ClassWork>& work, int64_t nbf,
@@ -580,22 +585,33 @@ cudaError_t launch_pieces(const DeviceBasis& db, const DeviceTables& dt, const s
   });
   const int ns = (int)std::min<size_t>(order.size(), (size_t)std::max(npool, 1));
   if (ns == 0) return cudaSuccess;
+  int64_t words = kPieceWords;
+  if (const char* env = std::getenv("SHGO_ESP_SCRATCH_DOUBLES")) words = std::max<int64_t>(1, std::atoll(env));
   std::vector<std::vector<ClassWork>> cut(order.size());
-  std::vector<int64_t> region(ns, 0), at(ns, 0);
-  for (size_t k = 0; k < order.size(); ++k) {
-    const ClassWork& w = work[order[k]];
-    const int64_t per = weight_words(w.la + w.lb + (NC == 3), NC);
-    cut[k] = pieces(w, db.h_ppoff, per, kPieceWords);
-    for (const ClassWork& c : cut[k]) region[k % ns] = std::max(region[k % ns], c.npp * per);
-  }
-  int64_t total = 0;
-  for (int i = 0; i < ns; ++i) {
-    at[i] = total;
-    total += region[i];
-  }
+  std::vector<int64_t> at(ns, 0);
   int2* buf = nullptr;
-  e = workspace_alloc((void**)&buf, sizeof(int2) * (size_t)std::max<int64_t>(total, 1), stream);
-  if (e != cudaSuccess) return e;
+  for (;; words /= 2) {  // smaller pieces where the device has no room for these, down to a shell pair at a time
+    std::vector<int64_t> region(ns, 0);
+    bool more = false;  // some piece has several shell pairs
+    for (size_t k = 0; k < order.size(); ++k) {
+      const ClassWork& w = work[order[k]];
+      const int64_t per = weight_words(w.la + w.lb + (NC == 3), NC);
+      cut[k] = pieces(w, db.h_ppoff, per, words);
+      for (const ClassWork& c : cut[k]) {
+        region[k % ns] = std::max(region[k % ns], c.npp * per);
+        more |= c.npairs > 1;
+      }
+    }
+    int64_t total = 0;
+    for (int i = 0; i < ns; ++i) {
+      at[i] = total;
+      total += region[i];
+    }
+    e = workspace_alloc((void**)&buf, sizeof(int2) * (size_t)std::max<int64_t>(total, 1), stream);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || !more) return e;
+  }
   cudaEvent_t fork = nullptr;
   e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventRecord(fork, stream);
@@ -659,14 +675,24 @@ cudaError_t launch_pieces(const DeviceBasis& db, const DeviceTables& dt, const s
       if (e != cudaSuccess) break;
     }
   }
-  for (int i = 0; i < ns && fork; ++i) {
+  bool joined = true;
+  for (int i = 0; i < ns && fork && joined; ++i) {
     cudaEvent_t join;
-    if (cudaEventCreateWithFlags(&join, cudaEventDisableTiming) != cudaSuccess) break;
+    if (cudaEventCreateWithFlags(&join, cudaEventDisableTiming) != cudaSuccess) {
+      joined = false;
+      break;
+    }
     cudaEventRecord(join, pool[i]);
     cudaStreamWaitEvent(stream, join, 0);
     cudaEventDestroy(join);
   }
   if (fork) cudaEventDestroy(fork);
+  if (!joined) {
+    // `stream` does not wait for every pool stream: finish their work before the weights are returned
+    for (int i = 0; i < ns; ++i) cudaStreamSynchronize(pool[i]);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaErrorUnknown;
+  }
   cudaFreeAsync(buf, stream);
   return e;
 }
