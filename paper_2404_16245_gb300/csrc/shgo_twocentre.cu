@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdlib>
 #include <string>
 #include <vector>
 
@@ -68,8 +69,36 @@ __device__ __forceinline__ int class_of_item(const PairClasses& cls, int item) {
   return c;
 }
 
-// S_LM(n), L <= lam, of the unit vector n = (B - A)/|B - A| (z for A = B) of every ordered pair of centres, one thread per
-// column M: the share of block `block` of `blocks`.  The radial launches carry these blocks after their own.
+// Column M of S_LM(n), L = |M| .. lam, of the unit vector n = (B - A)/|B - A| (z for A = B): put(L, S_LM).
+template <typename Put>
+__device__ __forceinline__ void site_column(const double* __restrict__ n, int lam, int m, Put&& put) {
+  const int am = m < 0 ? -m : m;
+  const double x = n[0], y = n[1], z = n[2];
+  double sp = 1.0, sm = 0.0;  // S_{l,l}, S_{l,-l}
+  if (am >= 1) {
+    sp = x;
+    sm = y;
+    for (int l = 1; l < am; ++l) {
+      const double c = k_harm.c[l];
+      const double np = c * (x * sp - y * sm), nm = c * (y * sp + x * sm);
+      sp = np;
+      sm = nm;
+    }
+  }
+  double prv = 0.0, cur = m < 0 ? sm : sp;
+  put(am, cur);
+  for (int l = am; l < lam; ++l) {
+    const int k = l * l + l + m;
+    double v = k_harm.a[k] * (z * cur);
+    if (m > -l && m < l) v -= k_harm.b[k] * prv;
+    put(l + 1, v);
+    prv = cur;
+    cur = v;
+  }
+}
+
+// The columns of every ordered pair of centres, one thread per column: the share of block `block` of `blocks`.  The radial
+// launches carry these blocks after their own.
 struct SiteArgs {
   int n_sites, lam;
   const double* site_rot;
@@ -80,30 +109,9 @@ __device__ __forceinline__ void site_harmonics(const SiteArgs& A, int block, int
   for (int64_t t = block * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)A.n_sites * ncol;
        t += (int64_t)blocks * blockDim.x) {
     const int64_t site = t / ncol;
-    const int m = (int)(t - site * ncol) - lam, am = m < 0 ? -m : m;
-    const double x = A.site_rot[9 * site + 6], y = A.site_rot[9 * site + 7], z = A.site_rot[9 * site + 8];
+    const int m = (int)(t - site * ncol) - lam;
     double* o = A.S + site * ns;
-    double sp = 1.0, sm = 0.0;  // S_{l,l}, S_{l,-l}
-    if (am >= 1) {
-      sp = x;
-      sm = y;
-      for (int l = 1; l < am; ++l) {
-        const double c = k_harm.c[l];
-        const double np = c * (x * sp - y * sm), nm = c * (y * sp + x * sm);
-        sp = np;
-        sm = nm;
-      }
-    }
-    double prv = 0.0, cur = m < 0 ? sm : sp;
-    o[am * am + am + m] = cur;
-    for (int l = am; l < lam; ++l) {
-      const int k = l * l + l + m;
-      double v = k_harm.a[k] * (z * cur);
-      if (m > -l && m < l) v -= k_harm.b[k] * prv;
-      o[(l + 1) * (l + 1) + l + 1 + m] = v;
-      prv = cur;
-      cur = v;
-    }
+    site_column(A.site_rot + 9 * site + 6, lam, m, [&](int l, double v) { o[l * l + l + m] = v; });
   }
 }
 
@@ -213,13 +221,14 @@ __global__ void __launch_bounds__(128) k_overlap_radial(int own, SiteArgs sites,
 }
 
 // Blocks from the X_L: a warp per shell pair, four per block.  nx[] = rows of X per pair: its primitive pairs from
-// pair_ppoff - q0 on (Coulomb), or the item itself (per_pair).
+// pair_ppoff - q0 on (Coulomb), or the item itself (per_pair).  S: the harmonics of every pair of centres, or NULL, and the
+// warp forms those of its pair.
 constexpr int kBlockWarps = 4;
 __global__ void __launch_bounds__(32 * kBlockWarps) k_twocentre_blocks(
     PairClasses cls, int lam_max, int stride, bool per_pair, int64_t q0, const int* __restrict__ pair_a,
     const int* __restrict__ pair_b, const int64_t* __restrict__ pair_ppoff, const int* __restrict__ pair_site,
-    const int* __restrict__ shell_nprim, const int64_t* __restrict__ shell_foff, const double* __restrict__ S,
-    const double* __restrict__ X, const int2* __restrict__ cx_rows, const GTerm* __restrict__ cx_terms, MolView mv,
+    const double* __restrict__ site_rot, const int* __restrict__ shell_nprim, const int64_t* __restrict__ shell_foff,
+    const double* __restrict__ S, const double* __restrict__ X, const int2* __restrict__ cx_rows, const GTerm* __restrict__ cx_terms, MolView mv,
     double* __restrict__ out) {
   extern __shared__ double smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, ns = (lam_max + 1) * (lam_max + 1);
@@ -239,11 +248,18 @@ __global__ void __launch_bounds__(32 * kBlockWarps) k_twocentre_blocks(
       xs[lane] = s;
     }
     __syncwarp();
-    const double* Sp = S + (int64_t)pair_site[pr] * ns;
-    for (int k = 0; k <= lb; ++k) {
-      const int L = lam - 2 * k;
-      const double x = xs[k];
-      for (int m = lane; m <= 2 * L; m += 32) SX[L * L + m] = Sp[L * L + m] * x;
+    if (S) {
+      const double* Sp = S + (int64_t)pair_site[pr] * ns;
+      for (int k = 0; k <= lb; ++k) {
+        const int L = lam - 2 * k;
+        const double x = xs[k];
+        for (int m = lane; m <= 2 * L; m += 32) SX[L * L + m] = Sp[L * L + m] * x;
+      }
+    } else {
+      for (int m = lane - lam; m <= lam; m += 32)
+        site_column(site_rot + 9 * (int64_t)pair_site[pr] + 6, lam, m, [&](int l, double v) {
+          if (l >= la - lb && ((lam - l) & 1) == 0) SX[l * l + l + m] = v * xs[(lam - l) >> 1];
+        });
     }
     __syncwarp();
     const int2* rows = cx_rows + cls.rows[c];
@@ -441,7 +457,10 @@ shgo_status launch_overlap_small(const DeviceBasis& db, const DeviceTables& dt, 
   return SHGO_OK;
 }
 
-// Doubles of X formed at a time (128 MiB); larger bases run in pieces of whole shell pairs.
+// Doubles of X formed at a time (128 MiB); larger bases run in pieces of whole shell pairs.  S is formed whole: it takes
+// (2 lmax + 1)^2 doubles per pair of centres, no more than the matrix where centres carry shells of the basis's lmax.  Where
+// the device has no room for it each warp forms the harmonics of its pair (300 atoms with l <= 3: overlap 0.60 -> 1.76 ms,
+// (a|b) 0.80 -> 1.97 ms).  SHGO_TWOCENTRE_SCRATCH_DOUBLES sets another size of X, and a limit for S.
 constexpr int64_t kXDoubles = (int64_t)1 << 24;
 
 shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTables& dt,
@@ -454,40 +473,51 @@ shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTa
     npp += w.npp;
   }
   if (npairs == 0) return SHGO_OK;
-  // pieces: consecutive (class, pairs) runs whose rows of X fit
-  std::vector<std::vector<ClassWork>> pieces(1);
-  int64_t rows = 0, most = 0;
-  for (const ClassWork& w : work) {
-    for (int q = w.pair_base; q < w.pair_base + w.npairs;) {
-      ClassWork c{w.la, w.lb, 0, q, 0, db.h_ppoff[q]};
-      int64_t r = 0;
-      while (q < w.pair_base + w.npairs) {
-        const int64_t add = coulomb ? db.h_ppoff[q + 1] - db.h_ppoff[q] : 1;
-        if (rows + r + add > std::max<int64_t>(kXDoubles / stride, 1) && rows + r > 0) break;
-        r += add;
-        ++c.npairs;
-        ++q;
-      }
-      c.npp = db.h_ppoff[q] - c.pp_base;
-      if (c.npairs) pieces.back().push_back(c);
-      rows += r;
-      most = std::max(most, rows);
-      if (q < w.pair_base + w.npairs) {
-        pieces.emplace_back();
-        rows = 0;
+  int64_t xcap = kXDoubles, scap = INT64_MAX;
+  if (const char* env = std::getenv("SHGO_TWOCENTRE_SCRATCH_DOUBLES")) xcap = scap = std::max<int64_t>(1, std::atoll(env));
+  int64_t slen = (int64_t)db.n_sites * ns <= scap ? (int64_t)db.n_sites * ns : 0;
+  std::vector<std::vector<ClassWork>> pieces;
+  double* buf = nullptr;  // S of every pair of centres, then X
+  for (;;) {  // less at a time where the device has no room: no S, then smaller pieces, down to a shell pair
+    // pieces: consecutive (class, pairs) runs whose rows of X fit
+    pieces.assign(1, {});
+    int64_t rows = 0, most = 0;
+    for (const ClassWork& w : work) {
+      for (int q = w.pair_base; q < w.pair_base + w.npairs;) {
+        ClassWork c{w.la, w.lb, 0, q, 0, db.h_ppoff[q]};
+        int64_t r = 0;
+        while (q < w.pair_base + w.npairs) {
+          const int64_t add = coulomb ? db.h_ppoff[q + 1] - db.h_ppoff[q] : 1;
+          if (rows + r + add > std::max<int64_t>(xcap / stride, 1) && rows + r > 0) break;
+          r += add;
+          ++c.npairs;
+          ++q;
+        }
+        c.npp = db.h_ppoff[q] - c.pp_base;
+        if (c.npairs) pieces.back().push_back(c);
+        rows += r;
+        most = std::max(most, rows);
+        if (q < w.pair_base + w.npairs) {
+          pieces.emplace_back();
+          rows = 0;
+        }
       }
     }
-  }
-  double* buf = nullptr;  // S of every pair of centres, then X
-  cudaError_t e = workspace_alloc((void**)&buf, sizeof(double) * ((size_t)db.n_sites * ns + (size_t)most * stride), stream);
-  if (e != cudaSuccess) {
+    const cudaError_t e = workspace_alloc((void**)&buf, sizeof(double) * (size_t)(slen + most * stride), stream);
+    if (e == cudaSuccess) break;
     cudaGetLastError();
-    *err = std::string("two-centre buffers: ") + cudaGetErrorString(e);
-    return SHGO_ERR_OOM;
+    if (e != cudaErrorMemoryAllocation || (slen == 0 && xcap <= stride)) {
+      *err = std::string("two-centre buffers: ") + cudaGetErrorString(e);
+      return SHGO_ERR_OOM;
+    }
+    if (slen > 0)
+      slen = 0;
+    else
+      xcap = std::min(xcap, most * stride) / 2;
   }
-  double *S = buf, *X = buf + (size_t)db.n_sites * ns;
+  double *S = slen > 0 ? buf : nullptr, *X = buf + slen;
   const Tables& th = tables_host();
-  const int site_blocks = grid_cap_sm(((int64_t)db.n_sites * (2 * lam_max + 1) + 127) / 128, 16);
+  const int site_blocks = S ? grid_cap_sm(((int64_t)db.n_sites * (2 * lam_max + 1) + 127) / 128, 16) : 0;
   const SiteArgs sites{db.n_sites, lam_max, db.site_rot, S};
   bool first = true;
   for (const std::vector<ClassWork>& piece : pieces) {
@@ -520,10 +550,10 @@ shgo_status launch_twocentre(bool coulomb, const DeviceBasis& db, const DeviceTa
                                                        X);
     k_twocentre_blocks<<<grid_cap_sm(((int64_t)total + kBlockWarps - 1) / kBlockWarps, 12), 32 * kBlockWarps,
                          sizeof(double) * kBlockWarps * (size_t)(ns + kLmax + 1), stream>>>(
-        cls, lam_max, stride, !coulomb, q0, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, db.shell_nprim,
-        db.shell_foff, S, X, dt.cx_rows, dt.cx_terms, mv, out);
+        cls, lam_max, stride, !coulomb, q0, db.pair_a, db.pair_b, db.pair_ppoff, db.pair_site, db.site_rot,
+        db.shell_nprim, db.shell_foff, S, X, dt.cx_rows, dt.cx_terms, mv, out);
   }
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   cudaFreeAsync(buf, stream);
   if (e != cudaSuccess) {
     *err = std::string(coulomb ? "two-centre launch: " : "overlap launch: ") + cudaGetErrorString(e);
