@@ -493,6 +493,18 @@ shgo_status build_basis(int32_t n_shells, const int32_t* l, const int32_t* n_pri
   for (const auto& w : b->work) rlen += w.npp * n_r(w.la + w.lb);
   b->h_ppoff.assign(ppoff.begin(), ppoff.end());
   b->h_ppoff.push_back(ppcount);
+  std::vector<int> pair_order;
+  if (!batch) {
+    pair_order.resize(pa.size());
+    for (auto& w : b->work) {
+      int at = w.pair_base;
+      for (int con = 0; con < 2; ++con) {
+        if (con) w.ncon = w.pair_base + w.npairs - at;
+        for (int q = w.pair_base; q < w.pair_base + w.npairs; ++q)
+          if ((b->h_ppoff[q + 1] - b->h_ppoff[q] >= deriv_con_prims(w.la, w.lb)) == (con != 0)) pair_order[at++] = q - w.pair_base;
+      }
+    }
+  }
   for (const auto& w : b->work)
     for (int q = w.pair_base; q < w.pair_base + w.npairs; ++q)
       max_pair_r = std::max(max_pair_r, (b->h_ppoff[q + 1] - b->h_ppoff[q]) * (int64_t)n_r(w.la + w.lb));
@@ -552,6 +564,7 @@ shgo_status build_basis(int32_t n_shells, const int32_t* l, const int32_t* n_pri
   const size_t o_ppoff = im.put(ppoff);
   const size_t o_srot = im.put(site_rot);
   const size_t o_psite = im.put(pair_site);
+  const size_t o_order = batch ? 0 : im.put(pair_order);
   const size_t o_srep = im.put(site_rep);
   const size_t o_pppair = im.put(pp_pair);
   const size_t o_ppij = im.put(pp_ij);
@@ -598,6 +611,7 @@ shgo_status build_basis(int32_t n_shells, const int32_t* l, const int32_t* n_pri
     b->d.pair_ppoff = reinterpret_cast<int64_t*>(base + o_ppoff);
     b->d.site_rot = reinterpret_cast<double*>(base + o_srot);
     b->d.pair_site = reinterpret_cast<int*>(base + o_psite);
+    if (!batch) b->d.pair_order = reinterpret_cast<const int*>(base + o_order);
     b->d.site_rep = reinterpret_cast<int*>(base + o_srep);
     b->d.pp_pair = reinterpret_cast<int*>(base + o_pppair);
     b->d.pp_ij = reinterpret_cast<int*>(base + o_ppij);

@@ -86,7 +86,8 @@ __host__ __device__ inline size_t deriv_contract_doubles(int la, int lb, int kin
 }
 
 struct DerivArgs {
-  int la = 0, lb = 0, npairs = 0, pair_base = 0;
+  int la = 0, lb = 0, npairs = 0, pair_base = 0;  // npairs: of the launch
+  const int* order = nullptr;      // their indices within the class (NULL: all of it)
   int64_t pp_base = 0, rbase = 0;  // the class's first primitive pair; its coupling blocks at r1buf + rbase
   int nkind = 0;
   int kinds[8] = {};
@@ -108,6 +109,7 @@ struct DerivArgs {
   const int* rowinfo[3] = {};  // Gaunt programs: the class, the class lowered on a, lowered on b
   const int* grp[3] = {};
   const GTerm* gterms[3] = {};
+  int con_prims = 0;               // primitive pairs from which the contracting launch contracts
   int nrt[3] = {};                 // the pair kernel's form of the programs (Tables::rt_src, px_rows, px_terms)
   const int* rt_src[3] = {};
   const int2* rows[3] = {};
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(128, CON ? 6 : 8) k_deriv_block(DerivArgs A) {
   double* Rt = fc + 2 * kDerivChunk * nfab;  // [nacc][nrt] contracted entries
   int* En = reinterpret_cast<int*>(Rt + nacc * nrt);  // [nacc][nfab]
   for (int w = blockIdx.x; w < A.npairs; w += gridDim.x) {
-    const int pr = A.pair_base + w;
+    const int pr = A.pair_base + (A.order ? A.order[w] : w);
     const int a = A.pair_a[pr], b = A.pair_b[pr];
     const double* rd = A.rotd + (int64_t)A.pair_site[pr] * A.rot_per;
     __syncthreads();
@@ -286,7 +288,7 @@ __global__ void __launch_bounds__(128, CON ? 6 : 8) k_deriv_block(DerivArgs A) {
     const int64_t q0 = A.pair_ppoff[pr];
     bool live = false;  // uniform over the block
     const int npp = npa * npb;
-    const bool con = CON && npp > 1;
+    const bool con = CON && npp >= A.con_prims;
     if (con) {
       for (int e = tid; e < nacc * nrt; e += nth) Rt[e] = 0.0;
       for (int e = tid; e < nacc * nfab; e += nth) En[e] = 0;
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(128, CON ? 6 : 8) k_deriv_block(DerivArgs A) {
     }
     for (int t = 0; t < nacc; ++t) {
       __syncthreads();
-      double* o = A.scratch + (int64_t)w * A.per_pair + A.soff[t == 0 ? slot0 : kSlotB + comp];
+      double* o = A.scratch + (int64_t)(A.order ? A.order[w] : w) * A.per_pair + A.soff[t == 0 ? slot0 : kSlotB + comp];
       if (!live) {
         for (int e = tid; e < (lowered ? 3 * NA * NB : na * nb); e += nth) o[e] = 0.0;
         continue;
@@ -687,9 +689,9 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
   struct Plan {
     DerivArgs d;
     CombineArgs c;
-    size_t smem = 0;
+    size_t smem = 0, smem_con = 0;
     int threads = 32;
-    bool con = false;  // the class has shell pairs of several primitive pairs
+    int ncon = 0;  // shell pairs that contract their primitive pairs first
     int64_t r1 = 0, scr = 0;  // doubles
   };
   std::vector<Plan> plan(work.size());
@@ -733,9 +735,11 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
       const int g = kinds[k] == kKindLowA ? 1 : (kinds[k] == kKindLowB ? 2 : 0);
       more = std::max(more, sizeof(double) * (base + deriv_contract_doubles(w.la, w.lb, kinds[k], d.nrt[g])));
     }
-    // contracted where the shared memory of a block allows it (a rule on the class, which every class to (8, 8) meets)
-    P.con = w.npp > w.npairs && more <= kConMaxBytes;
-    if (P.con) P.smem = more;
+    // contracted where the shared memory of a block allows it (every class to (8, 8) does)
+    P.ncon = more <= kConMaxBytes ? w.ncon : 0;
+    d.con_prims = deriv_con_prims(w.la, w.lb);
+    if (P.ncon > 0 && w.la + w.lb < 9) P.ncon = w.npairs;  // the contracting launch takes the others too, uncontracted
+    P.smem_con = more;
     // scratch blocks of a shell pair
     const int64_t nab = (int64_t)(2 * w.la + 1) * (2 * w.lb + 1);
     int64_t off = 0;
@@ -859,12 +863,21 @@ shgo_status launch_nuclear_deriv(const DeviceBasis& db, const DeviceTables& dt, 
     d.low_b = w.lb > 0 ? dt.d_low + th.d_low_off[w.lb] : nullptr;
     d.ppd = db.ppd;
     d.r1buf = r1buf;
-    const dim3 grid((unsigned)grid_cap_sm(w.npairs, 16), (unsigned)d.nkind);
-    if (P.con)
-      k_deriv_block<true><<<grid, P.threads, P.smem, s>>>(d);
-    else
-      k_deriv_block<false><<<grid, P.threads, P.smem, s>>>(d);
-    e = cudaGetLastError();
+    // From la + lb = 9 on a launch for each kind of pair, so that a few contracted pairs do not put the contracting variant's
+    // shared memory on all of a class; below, where that costs little, one launch.  dV/dA of 32 atoms with l <= 6, one
+    // shell per l of two primitives: one launch 2.23 ms, this 1.73 (no contracted shell: 1.50); of 16 atoms with l <= 8 3.95
+    // and 2.49.  Two launches for every class: forces of a contracted 17-atom molecule 2.27 -> 2.32 ms.
+    for (int con = 0; con < 2 && e == cudaSuccess; ++con) {
+      d.npairs = con ? P.ncon : w.npairs - P.ncon;
+      if (d.npairs == 0) continue;
+      d.order = P.ncon == 0 || P.ncon == w.npairs ? nullptr : db.pair_order + w.pair_base + (con ? w.npairs - P.ncon : 0);
+      const dim3 grid((unsigned)grid_cap_sm(d.npairs, 16), (unsigned)d.nkind);
+      if (con)
+        k_deriv_block<true><<<grid, P.threads, P.smem_con, s>>>(d);
+      else
+        k_deriv_block<false><<<grid, P.threads, P.smem, s>>>(d);
+      e = cudaGetLastError();
+    }
     if (e != cudaSuccess) break;
     if (contract) {
       ContractArgs g;

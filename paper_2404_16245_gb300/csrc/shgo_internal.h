@@ -374,6 +374,7 @@ struct ClassWork {
   int pair_base;   // first pair of the class in the pair arrays
   int64_t npp;     // primitive pairs of the class
   int64_t pp_base; // first primitive pair of the class in the primitive-pair arrays
+  int ncon = 0;    // shell pairs of deriv_con_prims or more primitive pairs (a basis's own classes; DeviceBasis::pair_order)
 };
 
 // Rotations of the pair frames, from the basis alone, built once per basis by k_pair_rotations for
@@ -395,6 +396,12 @@ void build_site_pairs(const double* shell_xyz, const std::vector<int>& pa, const
 struct PPData {
   double p, rp, sp, kab, pref, ra, rb, shift;
 };
+
+// Shell pairs of this many primitive pairs have them contracted before the coupling in the derivative integrals.  The
+// contracting variant takes about twice the shared memory, which from la + lb = 9 on leaves one or two blocks on an SM.
+// Measured (GB300, dV/dA of 32 atoms, contracted and not): shells up to l = 3 of two primitives (4 primitive pairs) 373 and
+// 458 us, up to l = 6 4.74 and 4.21 ms, with this line 4.11.
+constexpr int deriv_con_prims(int la, int lb) { return la + lb >= 9 ? 5 : 3; }
 
 struct DeviceBasis {
   // shells
@@ -429,6 +436,9 @@ struct DeviceBasis {
   // stream and each class runs in chunks of whole shell pairs that fit its stream's region;
   // h_ppoff (host, npairs + 1) gives the primitive-pair offsets used to cut the chunks.
   int64_t region = 0;
+  // Single bases: shell pairs of a class (index within it) by the derivative kernel's variant, those below
+  // deriv_con_prims primitive pairs first; the class's entries start at its pair_base.
+  const int* pair_order = nullptr;
   const int64_t* h_ppoff = nullptr;
   // work queues (nullptr ctrl: strided blocks, no time limit): control block, items per class in
   // decreasing cost (local indices at the class's primitive-pair / pair offset; nullptr = index order),
