@@ -207,9 +207,9 @@ shgo_status shgo_basis_sync(const shgo_basis* basis);
  * Same result as shgo_basis_create + shgo_nuclear_attraction + shgo_free, from the same host
  * basis arrays, device nuclei/charges and device output, on the current device.  It never calls
  * cudaMalloc, cudaFree or any allocating CUDA routine: the constant tables, this call's shells and
- * pair lists and its coupling buffer all live in one static device array of
- * SHGO_NOALLOC_SCRATCH_BYTES that the library holds on every GPU where it has been called, until the
- * process exits.  The CUDA driver loads the library's device code lazily (the default since CUDA
+ * pair lists and its coupling buffer all live in a static device array of
+ * SHGO_NOALLOC_SCRATCH_BYTES (and another of 128 KiB) that the library holds on every GPU where it has been
+ * called, until the process exits.  The CUDA driver loads the library's device code lazily (the default since CUDA
  * 12.2), so the array's memory is committed on a device when the first call runs there: make that
  * first call before an external pool manager takes the device's free memory.  If the device has no
  * room for the array at that point the call returns SHGO_ERR_OOM.  A problem whose shells, pairs and coupling buffer do not fit the part of that array left

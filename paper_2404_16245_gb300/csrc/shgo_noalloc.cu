@@ -4,10 +4,11 @@
 // pool manager that forbids foreign allocations, or code that must not enter the CUDA allocator
 // while it runs.  shgo_basis_create allocates (shell arrays, pair lists, the per-primitive-pair
 // coupling buffer, and on first use the constant tables), so such callers get this one entry
-// point instead.  Everything it needs on the device lives in one file-scope static array of
+// point instead.  Everything it needs on the device lives in a file-scope static array of
 // kNoallocScratchBytes (SHGO_NOALLOC_SCRATCH_BYTES), which every GPU that loads the library keeps
 // until the process exits:
 //   [ constant tables, copied in once per device ][ this call's shells, pair lists and coupling buffer ]
+// and in one of 128 KiB for the tables that have no room there.
 // The kernels are the ones shgo_nuclear_attraction launches; only their buffers differ.
 #include <cuda_runtime.h>
 
@@ -34,10 +35,10 @@ constexpr size_t kNoallocScratchBytes = (size_t)SHGO_NOALLOC_SCRATCH_BYTES;
 // The scratch.  In host code this name is only a stand-in for the device array: its device address
 // comes from cudaGetSymbolAddress at set-up and is what the kernels receive.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
-// The pair kernel's row headers, entry lists and axial factors have an array of their own; the scratch keeps the room of
-// the smaller tables they replaced (kNoallocReserved), so that it accepts the same problems.
-constexpr size_t kNoallocTableBytes = (size_t)1 << 20;
-constexpr size_t kNoallocReserved = 363008;
+// The room of the tables at the front of the scratch is fixed, so that the accepted problems do not depend on them; what
+// does not fit beside the pair kernel's row headers has an array of its own.
+constexpr size_t kNoallocFront = 496384;
+constexpr size_t kNoallocTableBytes = (size_t)1 << 17;
 static __device__ __align__(256) unsigned char g_noalloc_tables[kNoallocTableBytes];
 
 struct NoallocDevice {
@@ -84,8 +85,13 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   d.base = static_cast<unsigned char*>(ptr);
   const Tables& t = tables_host();
   Packer pk;
-  const size_t o_boys = pk.add(t.boys.size() * sizeof(double));
-  pk.add(kNoallocReserved);
+  const size_t o_rows = pk.add(t.px_rows.size() * sizeof(int2));
+  const size_t o_rssrc = pk.add(t.rs_src.size() * sizeof(int));
+  if (pk.used > kNoallocFront) {
+    *err = "constant tables do not fit the front of the static scratch";
+    return SHGO_ERR_OOM;
+  }
+  pk.used = kNoallocFront;
   const size_t o_terms = pk.add(t.px_terms.size() * sizeof(int4));
   const size_t o_rmap = pk.add(t.rmap.size() * sizeof(int));
   const size_t o_rnorm = pk.add(t.rnorm.size() * sizeof(double));
@@ -105,8 +111,6 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   Packer pk2;
   const size_t o_axial = pk2.add(t.axial.size() * sizeof(double));
   const size_t o_rtsrc = pk2.add(t.rt_src.size() * sizeof(int));
-  const size_t o_rssrc = pk2.add(t.rs_src.size() * sizeof(int));
-  const size_t o_rows = pk2.add(t.px_rows.size() * sizeof(int2));
   if (pk2.used > kNoallocTableBytes) {
     *err = "constant tables do not fit their static array";
     return SHGO_ERR_OOM;
@@ -115,11 +119,10 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
     unsigned char* dst;
     const void* src;
     size_t bytes;
-  } pieces[] = {{d.base + o_boys, t.boys.data(), t.boys.size() * sizeof(double)},
-                {base2 + o_axial, t.axial.data(), t.axial.size() * sizeof(double)},
+  } pieces[] = {{base2 + o_axial, t.axial.data(), t.axial.size() * sizeof(double)},
                 {base2 + o_rtsrc, t.rt_src.data(), t.rt_src.size() * sizeof(int)},
-                {base2 + o_rssrc, t.rs_src.data(), t.rs_src.size() * sizeof(int)},
-                {base2 + o_rows, t.px_rows.data(), t.px_rows.size() * sizeof(int2)},
+                {d.base + o_rssrc, t.rs_src.data(), t.rs_src.size() * sizeof(int)},
+                {d.base + o_rows, t.px_rows.data(), t.px_rows.size() * sizeof(int2)},
                 {d.base + o_terms, t.px_terms.data(), t.px_terms.size() * sizeof(int4)},
                 {d.base + o_rmap, t.rmap.data(), t.rmap.size() * sizeof(int)},
                 {d.base + o_rnorm, t.rnorm.data(), t.rnorm.size() * sizeof(double)},
@@ -134,11 +137,10 @@ shgo_status noalloc_setup(int device, NoallocDevice** out, std::string* err) {
   }
   shgo_status st = upload_constants(err);
   if (st != SHGO_OK) return st;
-  d.tabs.boys = reinterpret_cast<double*>(d.base + o_boys);
   d.tabs.axial = reinterpret_cast<double*>(base2 + o_axial);
   d.tabs.rt_src = reinterpret_cast<int*>(base2 + o_rtsrc);
-  d.tabs.rs_src = reinterpret_cast<int*>(base2 + o_rssrc);
-  d.tabs.px_rows = reinterpret_cast<int2*>(base2 + o_rows);
+  d.tabs.rs_src = reinterpret_cast<int*>(d.base + o_rssrc);
+  d.tabs.px_rows = reinterpret_cast<int2*>(d.base + o_rows);
   d.tabs.px_terms = reinterpret_cast<int4*>(d.base + o_terms);
   d.tabs.rmap = reinterpret_cast<int*>(d.base + o_rmap);
   d.tabs.rnorm = reinterpret_cast<double*>(d.base + o_rnorm);
