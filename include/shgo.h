@@ -18,6 +18,13 @@
  *    a stream are asynchronous and stream-ordered (stream = a cudaStream_t, NULL = the legacy
  *    default stream).  Errors found before any launch are returned synchronously and the
  *    outputs are left untouched; a CUDA error is returned as SHGO_ERR_CUDA.
+ *  - Accuracy (FP64): a few times 1e-15 of the largest element of a shell pair's block (of the largest
+ *    gradient, for the potential's gradient).  The sums run in 58-bit fixed point with a common scale for the
+ *    entries of a row, so an element that is smaller than its block by a factor f, as for a nearly planar or
+ *    nearly linear arrangement with the pair on a coordinate axis, keeps that absolute accuracy and has f times
+ *    the relative error.  Elements that vanish by symmetry are zero to that accuracy.
+ *  - Work arrays of the calls come stream-ordered from a pool of the library's own, of which up to 1 GiB per device
+ *    stays with the library between calls, until the last basis on the device is freed.
  *  - Failing calls leave a message for shgo_last_error() (thread-local).
  */
 #ifndef SHGO_H
@@ -158,6 +165,8 @@ shgo_status shgo_nuclear_attraction_timed(const shgo_basis* basis, const shgo_ce
  *             radial factors, S_LM(C - P) by recursion, and 2 per entry of R[L,M,k];
  *   flops[1]  per primitive pair: 2 per Gaunt term + 4 per W entry; per shell pair: building
  *             T_A, T_B and the two dense products T_A W T_B^T.
+ *             The pair kernel contracts the primitive pairs of a shell pair before the coupling, so on contracted
+ *             bases it does less than this count.
  * triples[0] receives the shell-triples (unique shell pairs x nuclei), triples[1] the primitive
  * triples (primitive pairs x nuclei). */
 shgo_status shgo_basis_flops(const shgo_basis* basis, int64_t n_centers, double* flops, double* triples);
@@ -250,9 +259,8 @@ int64_t shgo_batch_out_size(const shgo_basis* batch);
 /* V_m for every molecule (Eq. 11 per molecule with its own nuclei).  centers [sum n_c][3] and
  * charges [sum n_c] are device arrays in molecule order; out is a device array of
  * shgo_batch_out_size doubles, fully overwritten.
- * The first call on a batch tunes, per (la, lb) class, the nucleus-chunk size of the coupling
- * kernel and the threads per block of the pair kernel by timing them on this work (it
- * synchronises `stream`; its output is exact).  The next call captures the whole launch sequence
+ * The first call on a batch launches its kernels directly (with a time limit set it waits for `stream`).
+ * The next call captures the whole launch sequence
  * into a CUDA graph on an internal stream; later calls with the same centers/charges/out pointers and
  * time limit replay it with one cudaGraphLaunch on `stream` (new pointers or a new limit re-capture).
  * Calls on one batch must be ordered, and batched calls on one device should come from one host thread
@@ -280,10 +288,11 @@ shgo_status shgo_esp(const shgo_basis* basis, const double* density, const shgo_
 /* Gradient of that potential with respect to each point, grad[k][c] = d phi_k / d x_{k,c}
  *   = sum_{a,b} D_ab d/dx_{k,c} < phi_a | 1/|r - x_k| | phi_b >
  * (for a point charge q_k the force from the density's part of the energy sum_k q_k phi_k is -q_k grad[k];
- * for a nucleus, its Hellmann-Feynman term).  Same pipeline as shgo_esp with derivative tables per
- * point: gradients of the solid-harmonic polynomials (degree L -> L - 1, the raising/lowering of Eq. 3)
- * and dB_{L,k}/dT = -T^k/k! F_{L+k+1} (one more Boys order).  grad: device [n][3], overwritten.  Same
- * arguments, restrictions and errors as shgo_esp. */
+ * for a nucleus, its Hellmann-Feynman term).  Same pipeline as shgo_esp: the gradient of a one-centre integral is
+ * a combination of those of order la + lb + 1 (the raising and lowering of Eq. 3), so each primitive pair has three
+ * sets of weights of that order, which serve every point; far from the pair they follow from the far potential's, by
+ * the derivative of S_LM(d) / |d|^{2L+1}.  grad: device [n][3], overwritten.  Same
+ * arguments, restrictions and errors as shgo_esp; the weights take three times the work array. */
 shgo_status shgo_esp_gradient(const shgo_basis* basis, const double* density, const shgo_centers* points,
                               double* grad, void* stream);
 
@@ -361,8 +370,8 @@ shgo_status shgo_coulomb_2c(const shgo_basis* basis, double* out, void* stream);
  * unique quartet once, written to its eight permutations).  A per-call device buffer of
  * sum over primitive pairs of (2la+1)(2lb+1) C(la+lb+3, 3) doubles, plus a scratch region of partial
  * blocks per pool stream (at most 8M doubles each, or the count in the environment variable
- * SHGO_ERI_SCRATCH_DOUBLES; larger work is cut into pieces that fit), is taken from the device's default
- * stream-ordered pool and returned on `stream`.  Asynchronous on `stream`.  Errors: SHGO_ERR_INVALID_ARG
+ * SHGO_ERI_SCRATCH_DOUBLES; larger work is cut into pieces that fit), is taken from the library's
+ * pool and returned on `stream`.  Asynchronous on `stream`.  Errors: SHGO_ERR_INVALID_ARG
  * (NULL basis or out, a batch, nbf > 40000), SHGO_ERR_UNSUPPORTED_L (a shell with l > 4), SHGO_ERR_OOM,
  * SHGO_ERR_CUDA. */
 shgo_status shgo_eri(const shgo_basis* basis, double* out, void* stream);

@@ -9,7 +9,7 @@
 //
 // What bounds it: FP64 issues 1.7 lanes per clock and SM on GB300, integer multiply-adds 62 (measured).  So FP64 is kept for
 // what needs its range (geometry, Boys values, radial sums), once per nucleus, and the rest, the harmonics and the
-// sums over nuclei, runs in 58-bit fixed point (shgo_fixed.cuh), which has more bits than an FP64 mantissa.
+// sums over nuclei, runs in 58-bit fixed point (shgo_fixed.cuh), which has more bits than an FP64 mantissa at full scale.
 //
 // The nuclei of a chunk of 32 fall in three kinds, and take columns of the shared tables in this order:
 //  - near: T below kFarT[Lambda].  Boys values by Taylor expansion from a grid that reaches that T (one branch, no
@@ -23,7 +23,9 @@
 //    added in FP64 to the M = 0 entries alone.
 // Radial rows are scaled by the largest exponent among the row's columns, near and far separately; harmonic rows by a
 // power of two per (l, |m|), and x, y of a chunk close to the axis by that of the chunk's largest.  A sum is therefore within
-// 32 x 2^-59 or so of the largest product in it, where an FP64 sum rounds at 2^-53 of its partial sums.
+// 32 x 2^-59 or so of its scale, the row's largest radial value times the harmonics' bound, where an FP64 sum rounds at
+// 2^-53 of its partial sums: entries (L, M) much smaller than their row (x or y of every nucleus far below that of one that
+// sets the scale) have fewer digits of their own than in FP64, the block's larger elements have more.
 //
 // Phases of a block (NW warps, one primitive pair at a time): warp 0, lane = nucleus: geometry, kinds, radial rows;
 // all warps: the radial rows into fixed point, then for 16 columns at a time (a smaller table, so more blocks on an SM) the

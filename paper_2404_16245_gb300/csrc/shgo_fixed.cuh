@@ -2,8 +2,9 @@
 //
 // GB300 issues 64 integer multiply-adds (32 x 32 + 64 bits) per clock and SM and 1.7 FP64 ones (measured;
 // shgo_measure_fma_rate for the latter), so a product of two 58-bit numbers formed from three such multiply-adds
-// costs a twelfth of an FP64 one and carries five bits more than its mantissa.  Values are scaled by a power of two
-// to |v| <= 1 and held as q = round(v 2^58) = h 2^29 + l with l in [-2^28, 2^28).  A sum of at most 35
+// costs a twelfth of an FP64 one.  Values are scaled by a power of two, common to the entries that are summed together,
+// to |v| <= 1, so the largest carry five bits more than an FP64 mantissa and one smaller by 2^-k carries 58 - k bits: sums
+// are accurate relative to their scale, not relative to each entry.  A value is held as q = round(v 2^58) = h 2^29 + l with l in [-2^28, 2^28).  A sum of at most 35
 // products keeps the partial sums of h h and of h l + l h in one 64-bit accumulator each (32 nuclei, or the 2 Lambda + 1
 // terms of a degree, 35 at Lambda = 17); the products l l (at most 2^-60 of a full-scale one) are left out.
 #pragma once
