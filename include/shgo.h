@@ -346,7 +346,10 @@ shgo_status shgo_nuclear_field(const shgo_basis* basis, const shgo_centers* cent
  * diagonal in (l, m) by the orthogonality of Eq. 10, then rotated from the pair frame back to the
  * molecular frame.  out: device array, row-major nbf x nbf for a basis (symmetric, fully
  * overwritten), the batched layout of shgo_batch_layout for a batch.  Asynchronous on `stream`;
- * no nuclei are involved.  Errors: SHGO_ERR_INVALID_ARG (NULL basis or out), SHGO_ERR_CUDA. */
+ * no nuclei are involved.  Larger bases take a stream-ordered work array: up to 128 MiB of radial values and
+ * (2 lmax + 1)^2 doubles per pair of centres, less where the device has no room (down to a shell pair;
+ * SHGO_TWOCENTRE_SCRATCH_DOUBLES sets another size for both).  Errors: SHGO_ERR_INVALID_ARG (NULL basis or out),
+ * SHGO_ERR_OOM, SHGO_ERR_CUDA. */
 shgo_status shgo_overlap(const shgo_basis* basis, double* out, void* stream);
 
 /* Two-centre Coulomb integrals (a|b) = int int phi_a(r1) phi_b(r2) / |r1 - r2| (the two-centre case of the
@@ -355,8 +358,8 @@ shgo_status shgo_overlap(const shgo_basis* basis, double* out, void* stream);
  * respect to its centre, so (a|b) is S_la(grad_R) S_lb(grad_R) applied to the s-s integral, a function of
  * |A - B|^2 through F_0; the product rule of solid harmonics (the Gaunt coupling) and Hobson's theorem
  * turn it into sum_{L,M} G 2^L S_LM(A - B) times Boys values F_{L+k+j}.  Computed in FP64 whatever the
- * basis's precision option.  out: as for shgo_overlap (symmetric, fully overwritten).  Asynchronous on
- * `stream`.  Errors: SHGO_ERR_INVALID_ARG (NULL basis or out), SHGO_ERR_CUDA. */
+ * basis's precision option.  out: as for shgo_overlap (symmetric, fully overwritten), with the
+ * same work arrays.  Asynchronous on `stream`.  Errors: SHGO_ERR_INVALID_ARG (NULL basis or out), SHGO_ERR_OOM, SHGO_ERR_CUDA. */
 shgo_status shgo_coulomb_2c(const shgo_basis* basis, double* out, void* stream);
 
 /* Four-centre electron-repulsion integrals (ab|cd) = int int phi_a(r1) phi_b(r1) phi_c(r2) phi_d(r2) /
