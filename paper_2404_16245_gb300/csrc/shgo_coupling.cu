@@ -39,8 +39,10 @@
 // quadrature are the same to two digits.  At Lambda <= 2 the FP64 pipe is 76 % busy (84 % is what plain DFMAs reach), from
 // Lambda 4 on a primitive pair's dependent chains bound it (15 to 20 warps on an SM, FP64 pipe 45 to 55 % busy).
 // Small calls, where a launch is one chain (7 to 9 us at Lambda <= 4): block tables by asynchronous copies, harmonic steps and row
-// codes in shared memory, shorter sums and one split of shared memory for all kernels of a call: V of 20 atoms with l <= 2
-// 50 -> 42 us, of 4 contracted atoms 46 -> 40, of 3 atoms with l <= 2 34 -> 33 (all in FP64: 52, 57, 32).
+// codes in shared memory, shorter sums: V of 14 atoms with l <= 2 43 -> 42 us, of 4 contracted atoms 46 -> 45, of 3 atoms
+// with l <= 2 33.3 -> 33.0 (all in FP64: 45, 57, 31.5); large calls 1 to 2 % (29-atom molecule 3.64 -> 3.57 ms).  One preferred
+// split of shared memory for all kernels of a call saves 3 to 7 us of device time there, but setting it costs a quarter of a
+// microsecond of host time per launch, and calls on changing buffers are bound by the host: 57 -> 60 us.
 #include <cuda_runtime.h>
 
 #include <utility>
@@ -407,10 +409,8 @@ cudaError_t coupling_fp64_setup() {
   cudaError_t e = upload_nucleus_constants();
   const std::vector<double>& bt = tables_host().boys_top;
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_boys_top, bt.data(), sizeof(double) * bt.size());
-  for (int lam = 0; lam <= kLamDer && e == cudaSuccess; ++lam) {
+  for (int lam = 0; lam <= kLamDer && e == cudaSuccess; ++lam)
     e = set_max_dynamic_smem((const void*)kernel_at(lam, Lams{}));
-    if (e == cudaSuccess) e = set_max_carveout((const void*)kernel_at(lam, Lams{}));
-  }
   return e;
 }
 

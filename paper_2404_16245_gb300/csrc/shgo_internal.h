@@ -492,12 +492,6 @@ inline cudaError_t set_max_dynamic_smem(const void* func) {
   return e;
 }
 
-// The largest split of an SM's memory for shared memory: the classes of a call run side by side, and an SM changes its
-// split, which by default follows the kernel, only when it is empty (V of 20 atoms with l <= 2 50 -> 43 us).
-inline cudaError_t set_max_carveout(const void* func) {
-  return cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-}
-
 // Raises `func`'s dynamic shared-memory limit to `bytes` (0: the most a block may take) on the current
 // device, once per (kernel, device) and under a lock: the attribute belongs to one device, so a process
 // on several devices sets it on each.

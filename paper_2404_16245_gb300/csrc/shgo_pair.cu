@@ -362,9 +362,6 @@ cudaError_t launch_pair_block(const PairArgs& args, int grid, cudaStream_t strea
   return cudaGetLastError();
 }
 
-cudaError_t pair_block_setup() {
-  const cudaError_t e = set_max_dynamic_smem((const void*)k_pair_block);
-  return e == cudaSuccess ? set_max_carveout((const void*)k_pair_block) : e;
-}
+cudaError_t pair_block_setup() { return set_max_dynamic_smem((const void*)k_pair_block); }
 
 }  // namespace shgo
